@@ -1,35 +1,29 @@
 // sort.cu -- Alg. 1 CreateTiles, DuplicateWithKeys, SortByKeys and
 // IdentifyTileRanges.
 //
-// The instance key is (global tile index, camera depth) and the sort is a
-// stable LSD radix sort of it.  Every instance of one projected row carries
-// the same depth, so the depth digits (the least significant ones) are sorted
-// once per row, before duplication: rows are radix-sorted by the IEEE bits
-// of their depth (positive floats order like their bit patterns), the
-// instances are emitted in that row order, and the tile digits are then
-// radix-sorted stably.  The result is the order of a stable sort of the full
-// key in emission order.
+// The instance key is (global tile index, camera depth), the lists ordered as
+// by a stable sort of the full key in emission order.  Every instance of one
+// projected row carries the same depth, so neither path sorts instances by it.
 //
-// Radix passes are single-pass "onesweep"-style: one 8-bit digit per pass,
-// partitions of 4096 keys taken in ticket order by persistent CTAs, local
-// ranking of the keys of a warp (digit-bit ballots or a match instruction)
-// with shared-memory counters, and a decoupled look-back across partitions
-// whose waits are bounded (SPLAT_ERR_TIMEOUT on expiry).  On the binned path
-// the depth passes sort each view's rows in place (partitions stay inside a
-// view, digit counts and look-back are per view), so four passes give the
-// (view, depth) order.
+// The binned path (the default up to 40960 tiles per view) lists every row in
+// the 8x8-tile super-tiles that its rectangle meets, sorts each super-tile's
+// list by (depth bits, row) on its own (k_cell_count, k_cell_scan,
+// k_cell_scatter, k_unit_sort), and filters it into its tiles' lists in order:
+// the first 512 entries by a saturation head (k_head_count, a CTA per tile
+// row), the rest in parallel segments (k_tile_filter), the counts turned into
+// ranges by one look-back pass (k_tile_ranges) and the lists written by one
+// pass.  With culling on, a list holds only the tiles the opacity footprint
+// reaches and ends where every pixel of the tile has certainly saturated (tile
+// saturation, below); neither changes a result.
 //
-// The binned path (the default up to 40960 tiles per view) orders by tile
-// without tile-digit passes: the depth-ordered rows are split stably by
-// 8x8-tile super-tile in one onesweep-style pass over equal runs of list
-// slots (k_super_split), then each super-tile's list is filtered into its
-// tiles' lists in order: the first 512 entries by a saturation head
-// (k_head_count, a CTA per tile row), the rest in parallel segments
-// (k_tile_filter), the counts turned into ranges by one look-back pass
-// (k_tile_ranges) and the lists written by one pass.  With culling on, a list
-// holds only the tiles the opacity footprint reaches and ends where every
-// pixel of the tile has certainly saturated (tile saturation, below); neither
-// changes a result.  12 launches for any number of views.
+// The radix path sorts the rows by the IEEE bits of their depth (positive
+// floats order like their bit patterns), emits the instances in that row order
+// and radix-sorts the tile digits stably.  Its passes are single-pass
+// "onesweep"-style: one 8-bit digit per pass, partitions of 4096 keys taken in
+// ticket order by persistent CTAs, local ranking of the keys of a warp
+// (digit-bit ballots or a match instruction) with shared-memory counters, and a
+// decoupled look-back across partitions whose waits are bounded
+// (SPLAT_ERR_TIMEOUT on expiry).
 #include <algorithm>
 
 #include "splat_internal.cuh"
@@ -76,7 +70,9 @@ __device__ __forceinline__ unsigned long long block_excl_scan256_u64(unsigned lo
     return wsum + x - v;
 }
 
-__device__ __forceinline__ uint32_t block_excl_scan256(uint32_t v, uint32_t* s_tmp, uint32_t* total)
+// WARPS warps
+template <int WARPS>
+__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* s_tmp, uint32_t* total)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t x = v;
@@ -89,7 +85,7 @@ __device__ __forceinline__ uint32_t block_excl_scan256(uint32_t v, uint32_t* s_t
     __syncthreads();
     uint32_t wsum = 0, all = 0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) {
+    for (int w = 0; w < WARPS; ++w) {
         const uint32_t t = s_tmp[w];
         if (w < warp) wsum += t;
         all += t;
@@ -99,94 +95,48 @@ __device__ __forceinline__ uint32_t block_excl_scan256(uint32_t v, uint32_t* s_t
     return wsum + x - v;
 }
 
+__device__ __forceinline__ uint32_t block_excl_scan256(uint32_t v, uint32_t* s_tmp, uint32_t* total)
+{
+    return block_excl_scan<8>(v, s_tmp, total);
+}
+
 // ---------------------------------------------------------------------------
 // Depth keys of the projected rows + histograms of their 4 digits
 // ---------------------------------------------------------------------------
 
 struct DepthArgs {
     splat_proj proj;
-    int V, blocks_per_view;
+    int64_t n_rows;
     uint32_t* keys;
     uint32_t* vals;
-    uint32_t* dhist;        // [4][V][256] digit counts per view
-    uint32_t* super_total;  // [total_super] entries of each super-tile list (binned path), or null
-    int super_base[SPLAT_MAX_VIEWS];
-    int STX[SPLAT_MAX_VIEWS], STY[SPLAT_MAX_VIEWS];
+    uint32_t* dhist;        // [4][256] digit counts (zeroed)
     uint32_t* zero_a;
     int64_t n_zero_a;
     unsigned long long* zero_b;
     int64_t n_zero_b;
-    unsigned long long* zero_c;
-    int64_t n_zero_c;
 };
 
-// Block b serves view b / blocks_per_view.  The super-tile list sizes (binned
-// path) are counted through a 2D difference array of the view's super-tile
-// grid in dynamic shared memory ((STX + 1) x (STY + 1) words): a row adds its
-// super-rectangle with four corner updates, and the block's prefix sums over
-// x then y give its counts per super-tile.
 __global__ void __launch_bounds__(256) k_depth_keys(DepthArgs a)
 {
-    extern __shared__ uint32_t s_diff[];
     __shared__ uint32_t s_hist[4][kRadix];
-    const int v = (int)(blockIdx.x / a.blocks_per_view), bi = (int)(blockIdx.x - v * a.blocks_per_view);
-    const int SX = a.super_total ? a.STX[v] + 1 : 0, SY = a.super_total ? a.STY[v] + 1 : 0;
     for (int i = threadIdx.x; i < 4 * kRadix; i += blockDim.x) (&s_hist[0][0])[i] = 0;
-    for (int i = threadIdx.x; i < SX * SY; i += blockDim.x) s_diff[i] = 0;
     __syncthreads();
-    const int64_t n = a.proj.n, r_base = (int64_t)v * n;
-    for (int64_t i = bi * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)a.blocks_per_view * blockDim.x) {
-        const int64_t r = r_base + i;
-        const uint32_t nt = a.proj.n_tiles[r];
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t gt = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (int64_t r = gt; r < a.n_rows; r += stride) {
         const float depth = ((const float4*)a.proj.rgb_depth)[r].w;
-        const uint32_t k = nt > 0 ? __float_as_uint(depth) : 0xffffffffu;
+        const uint32_t k = a.proj.n_tiles[r] > 0 ? __float_as_uint(depth) : 0xffffffffu;
         a.keys[r] = k;
         a.vals[r] = (uint32_t)r;
 #pragma unroll
         for (int p = 0; p < 4; ++p) atomicAdd(&s_hist[p][(k >> (8 * p)) & 0xff], 1u);
-        if (nt > 0 && SX) {  // the super-rectangle [sx0, sx1) x [sy0, sy1) of the row's tile rectangle
-            const int4 rc = ((const int4*)a.proj.rect)[r];
-            const int sx0 = rc.x >> 3, sy0 = rc.y >> 3, sx1 = (rc.z + 7) >> 3, sy1 = (rc.w + 7) >> 3;
-            atomicAdd(&s_diff[sy0 * SX + sx0], 1u);
-            atomicAdd(&s_diff[sy0 * SX + sx1], 0xffffffffu);
-            atomicAdd(&s_diff[sy1 * SX + sx0], 0xffffffffu);
-            atomicAdd(&s_diff[sy1 * SX + sx1], 1u);
-        }
     }
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t gt = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     for (int64_t i = gt; i < a.n_zero_a; i += stride) a.zero_a[i] = 0;
     for (int64_t i = gt; i < a.n_zero_b; i += stride) a.zero_b[i] = 0;
-    for (int64_t i = gt; i < a.n_zero_c; i += stride) a.zero_c[i] = 0;
     __syncthreads();
     for (int i = threadIdx.x; i < 4 * kRadix; i += blockDim.x) {
         const uint32_t c = (&s_hist[0][0])[i];
-        const int p = i / kRadix, d = i - p * kRadix;
-        if (c) atomicAdd(&a.dhist[((size_t)p * a.V + v) * kRadix + d], c);
-    }
-    if (SX) {
-        for (int y = threadIdx.x; y < SY; y += blockDim.x) {  // prefix along x
-            uint32_t run = 0;
-            for (int x = 0; x < SX; ++x) {
-                run += s_diff[y * SX + x];
-                s_diff[y * SX + x] = run;
-            }
-        }
-        __syncthreads();
-        for (int x = threadIdx.x; x < SX; x += blockDim.x) {  // then along y
-            uint32_t run = 0;
-            for (int y = 0; y < SY; ++y) {
-                run += s_diff[y * SX + x];
-                s_diff[y * SX + x] = run;
-            }
-        }
-        __syncthreads();
-        const int STX = SX - 1, nsup = STX * (SY - 1);
-        for (int i = threadIdx.x; i < nsup; i += blockDim.x) {
-            const int y = i / STX, x = i - y * STX;
-            const uint32_t c = s_diff[y * SX + x];
-            if (c) atomicAdd(&a.super_total[a.super_base[v] + i], c);
-        }
+        if (c) atomicAdd(&a.dhist[i], c);
     }
 }
 
@@ -202,7 +152,7 @@ struct PassArgs {
     const int64_t* n_dev;  // element count on the device (null: n_host)
     int64_t n_host;
     int64_t cap;
-    const uint32_t* hist;  // [segments][256] digit counts of this pass
+    const uint32_t* hist;  // [256] digit counts of this pass
     uint32_t* lb;          // [parts][256] look-back words of this pass (zeroed)
     uint32_t* lb_next;     // [parts][256] zeroed here for the next pass (may be null)
     uint32_t* ticket;
@@ -210,9 +160,6 @@ struct PassArgs {
     int stage;
     int shift;
     int64_t spin_limit;
-    int64_t seg_len;       // > 0: the keys form segments of seg_len keys (the views' rows), each sorted on
-                           // its own in place, with hist holding [segments][256] counts; 0: one segment
-    int hist_sum;          // one segment: the digit counts are the sum of hist_sum [256] arrays
     int ballot_rank;       // rank by digit-bit ballots (many distinct digits per warp) instead of match
 };
 
@@ -230,15 +177,10 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(PassArgs a)
     if (status_failed(a.status)) return;
     const int64_t n = a.n_dev ? min(*a.n_dev, a.cap) : a.n_host;
     if (n <= 0) return;
-    // segments of seg keys, pps partitions each; a partition never crosses a
-    // segment boundary, and its look-back stops at its segment's first one
-    const int64_t seg = a.seg_len > 0 ? a.seg_len : n;
-    const int64_t pps = (seg + kSortPart - 1) / kSortPart;
-    const int64_t parts = pps * ((n + seg - 1) / seg);
+    const int64_t parts = (n + kSortPart - 1) / kSortPart;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt = lanemask_lt();
-    int64_t cur_seg = -1;
-    uint32_t gofs = 0;  // first output position of digit tid in the current segment
+    const uint32_t gofs = block_excl_scan256(a.hist[tid], s_tmp, nullptr);  // first output position of digit tid
 
     for (;;) {
         if (tid == 0) s_ticket = atomicAdd(a.ticket, 1u);
@@ -247,22 +189,10 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(PassArgs a)
         __syncthreads();
         const int64_t ticket = s_ticket;
         if (ticket >= parts) break;
-        const int64_t sg = ticket / pps, lp = ticket - sg * pps, first = sg * pps;
-        if (sg != cur_seg) {  // block-uniform
-            cur_seg = sg;
-            uint32_t h = 0;
-            if (a.seg_len > 0) {
-                h = a.hist[sg * kRadix + tid];
-            } else {
-                for (int q = 0; q < a.hist_sum; ++q) h += a.hist[q * kRadix + tid];
-            }
-            gofs = (uint32_t)(sg * seg) + block_excl_scan256(h, s_tmp, nullptr);
-        }
-        const int64_t seg_end = min(n, (sg + 1) * seg);
-        const int64_t base = sg * seg + lp * kSortPart;
+        const int64_t base = ticket * kSortPart;
         const int64_t wbase = base + (int64_t)warp * 32 * kSortItems;
         // keys of this warp's share of the partition: its items j * 32 + lane < wrem
-        const int64_t wr = seg_end - wbase;
+        const int64_t wr = n - wbase;
         const int wrem = wr <= 0 ? 0 : (wr >= 32 * kSortItems ? 32 * kSortItems : (int)wr);
         const uint32_t* kin = a.keys_in + wbase;
         const uint32_t* vin = a.vals_in + wbase;
@@ -317,7 +247,7 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(PassArgs a)
             cnt += c;
         }
         uint32_t* my = a.lb + ticket * kRadix + d;
-        st_relaxed(my, (lp == 0 ? kFlagPrefix : kFlagAgg) | cnt);
+        st_relaxed(my, (ticket == 0 ? kFlagPrefix : kFlagAgg) | cnt);
         if (a.lb_next) a.lb_next[ticket * kRadix + d] = 0;
         s_dstart[d] = block_excl_scan256(cnt, s_tmp, nullptr);
         // decoupled look-back for digit d, kLookWindow predecessors per step
@@ -325,14 +255,14 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(PassArgs a)
         // so a walk of one predecessor per L2 round trip would make the last
         // partition wait for about half the partition count of round trips
         uint32_t excl = 0;
-        if (lp > 0) {
+        if (ticket > 0) {
             int64_t j = ticket - 1;  // nearest predecessor not yet added
             int64_t spins = 0;
             for (;;) {
                 uint32_t w[kLookWindow];
 #pragma unroll
                 for (int q = 0; q < kLookWindow; ++q)
-                    w[q] = j - q >= first ? ld_relaxed(a.lb + (j - q) * kRadix + d) : kFlagPrefix;
+                    w[q] = j - q >= 0 ? ld_relaxed(a.lb + (j - q) * kRadix + d) : kFlagPrefix;
                 // add the published words from the nearest one back, up to and
                 // including the first inclusive prefix, or up to the first word
                 // not yet published
@@ -372,7 +302,7 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(PassArgs a)
             }
         }
         __syncthreads();
-        const int nvalid = (int)min((int64_t)kSortPart, seg_end - base);
+        const int nvalid = (int)min((int64_t)kSortPart, n - base);
         for (int i = tid; i < nvalid; i += kSortThreads) {
             const uint32_t key = s_keys[i];
             const uint32_t out = s_base[(key >> a.shift) & 0xff] + i;
@@ -393,8 +323,6 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(PassArgs a)
 struct ScanArgs {
     const uint32_t* rows;      // [n_rows] depth-sorted rows
     const uint32_t* n_tiles;   // [n_rows] per row
-    const int4* rect;          // [n_rows] tile rectangles (used when shift > 0)
-    int shift;                 // > 0: count the rectangle's (2^shift)^2 super-tiles instead
     int64_t n_rows;
     uint32_t* offsets;         // [n_rows] exclusive prefix (saturated at 2^32-1)
     uint32_t* chunk_row;       // [n_chunks_max] first sorted position of each duplicate chunk
@@ -407,21 +335,6 @@ struct ScanArgs {
     int32_t* status;
     int64_t spin_limit;
 };
-
-__device__ __forceinline__ int4 shifted_rect(int4 rc, int shift)
-{
-    if (shift == 0) return rc;
-    const int m = (1 << shift) - 1;
-    return make_int4(rc.x >> shift, rc.y >> shift, (rc.z + m) >> shift, (rc.w + m) >> shift);
-}
-
-__device__ __forceinline__ uint32_t row_count(const ScanArgs& a, uint32_t row)
-{
-    const uint32_t n = a.n_tiles[row];
-    if (a.shift == 0 || n == 0) return n;
-    const int4 rc = shifted_rect(a.rect[row], a.shift);
-    return (uint32_t)((rc.z - rc.x) * (rc.w - rc.y));
-}
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(ScanArgs a)
 {
@@ -447,14 +360,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(ScanArgs a)
 #pragma unroll
             for (int q = 0; q < kScanItems / 4; ++q) {
                 const uint4 r = r4[q];
-                c[4 * q + 0] = row_count(a, r.x);
-                c[4 * q + 1] = row_count(a, r.y);
-                c[4 * q + 2] = row_count(a, r.z);
-                c[4 * q + 3] = row_count(a, r.w);
+                c[4 * q + 0] = a.n_tiles[r.x];
+                c[4 * q + 1] = a.n_tiles[r.y];
+                c[4 * q + 2] = a.n_tiles[r.z];
+                c[4 * q + 3] = a.n_tiles[r.w];
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < kScanItems; ++j) c[j] = i0 + j < a.n_rows ? row_count(a, a.rows[i0 + j]) : 0u;
+            for (int j = 0; j < kScanItems; ++j) c[j] = i0 + j < a.n_rows ? a.n_tiles[a.rows[i0 + j]] : 0u;
         }
         unsigned long long tsum = 0;
 #pragma unroll
@@ -517,7 +430,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(ScanArgs a)
             const int64_t idx = i0 + j;
             if (idx < a.n_rows) {
                 a.offsets[idx] = off > 0xffffffffull ? 0xffffffffu : (uint32_t)off;
-                if (c[j] != 0 && a.n_chunks_max > 0) {
+                if (c[j] != 0) {
                     // chunks whose first slot falls inside [off, off + c)
                     const unsigned long long lo = (off + kDupChunk - 1) / kDupChunk;
                     const unsigned long long hi = (off + c[j] - 1) / kDupChunk;
@@ -631,336 +544,698 @@ __global__ void __launch_bounds__(256) k_ranges(const uint32_t* keys, const int6
 }
 
 // ---------------------------------------------------------------------------
-// Super-tile lists (level 1 of the binned path): a stable multi-split of the
-// (view, depth)-ordered visible rows by 8x8-tile super-tile.  A row enters
-// the list of every super-tile its tile rectangle meets, in raster order of
-// its super-rectangle, and the scan of the rows' super-tile counts gives every
-// row its first slot in that order (the slots of a view are contiguous).  The
-// lists' sizes come from the depth-key pass; one onesweep-style pass over
-// equal runs of slots then ranks each run's entries per super-tile in slot
-// order, finds every super-tile's offset from the runs before it by decoupled
-// look-back, and writes the entries in a second sweep over the same slots.
+// Super-tile lists (level 1 of the binned path).  A row enters the list of
+// every 8x8-tile super-tile its tile rectangle meets; a list is ordered by
+// (depth bits, row).  An MSD bucket sort with every list on its own:
+//
+//   k_cell_count    adds each entry to its cell = (super-tile, depth bin), one
+//                   reduction per entry, and packs the row's super-rectangle and
+//                   key into 8 bytes for the scatter.  Bins are equal steps of
+//                   the depth bits over the range of a sample of the view's rows
+//                   (depths outside fall into the first or last bin), so a bin's
+//                   entries are contiguous in the list's order
+//   k_cell_scan     block per super-tile: cell starts, the lists' ranges, K1, and
+//                   the sort units: runs of bins of about kUnit / 2 entries
+//   k_cell_scatter  writes each entry (row, key) into its cell, in any order
+//   k_unit_sort     sorts the units in shared memory (sort_unit below): before the
+//                   head count the units that hold the first kHeadEntries of a
+//                   list, after it the others, of the super-tiles with a list that
+//                   did not end in the head
+//
+// What bounds these kernels is latency and the one L2 atomic per entry.  They
+// replaced a radix sort of all rows by depth (four onesweep passes), a scan of
+// the rows' super-tile counts and a stable split of the entries by super-tile:
+// that chain of dependent passes took 130 us for a single view of any size below
+// 300k rows, and sorted every list to its end though a dense list is only read
+// up to its saturation.  All are exact: (depth bits, row) is unique in a list, so
+// the order does not depend on the arrival order in a cell.
 // ---------------------------------------------------------------------------
 
 constexpr int64_t kBinMaxTiles = 40960;  // per view: the binned path's default range
-constexpr int kSplitSlots = 4096;        // list slots per split partition (512 per warp)
-constexpr int kSplitWarpSlots = kSplitSlots / 8;
-constexpr int kSplitMaxSmem = 200 * 1024;  // shared memory the split's counters and grids may take
-constexpr unsigned long long kSplitAgg = 1ull << 62, kSplitPrefix = 2ull << 62, kSplitMask = (1ull << 62) - 1;
+constexpr int kSplitMaxSmem = 200 * 1024;
+constexpr int kMaxBins = 1024;           // depth bins per super-tile
+constexpr int kUnit = 2048;              // entries a block sorts in shared memory
+constexpr int kUnitThreads = 512, kPer = kUnit / kUnitThreads;
+constexpr int kUnitStep = kUnit / 2;     // a unit starts at the first bin start at or after each multiple
+constexpr int kSortBuckets = 2048;
+constexpr int kSortBucketBits = 11;
+constexpr uint32_t kCrowded = 48;        // entries in one bucket above which a unit is sorted bitonically
+constexpr uint32_t kWholeUnit = 0xffffffffu;
+constexpr int kHeadEntries = 512;        // entries of each list the head pass takes in order
 
-struct SplitArgs {
+struct CellArgs {
     splat_proj proj;
-    const uint32_t* rows;          // [V * n] rows, each view's in depth order, its visible ones first
-    const uint32_t* offsets;       // [V * n] first list slot of each of those rows
-    const uint32_t* super_total;   // [total_super] entries of each super-tile list
-    const int64_t* n_instances;    // K1, the slot count (checked against the capacity by the scan)
-    int V;
+    int V, bin_bits, nbins;        // nbins = 2^bin_bits depth bins
+    int copies;                    // of the cells (a power of two); block b of a view's rows uses copy b % copies
     int64_t n;                     // rows per view
-    int smax;                      // row stride of the per-warp counters (>= every view's super-tile count)
-    int sdiff;                     // row stride of the per-warp difference grids (>= (STX + 1) (STY + 1))
-    int total_super;
+    uint2* range;                  // [V] first depth bits and shift of the views' bins, from k_cell_count
     int super_base[SPLAT_MAX_VIEWS + 1];
-    int STX[SPLAT_MAX_VIEWS], STY[SPLAT_MAX_VIEWS];
-    unsigned long long* lb;        // [max_parts][smax] look-back words (zeroed)
-    int64_t max_parts;
-    uint32_t* ticket;
-    uint32_t* list;                // out: the super-tile lists, K1 entries
+    int STX[SPLAT_MAX_VIEWS];
+    uint2* rec;                    // [V * n] (super-rectangle x0 | y0 << 8 | x1 << 16 | y1 << 24, depth bits)
+    uint32_t* cell;                // [copies][total_super][nbins] entry counts (zeroed), then cursors
+    uint2* entries;                // out: (row, depth bits) of the lists' entries, by cell
+    int64_t capacity;
+    // k_cell_scan
+    unsigned long long* lb;        // [total_super] look-back words (zeroed)
+    uint32_t* ticket;              // (zeroed)
     uint2* sranges;                // out: [total_super] [start, end) of each list, (0, 0) when empty
+    int64_t* K1;                   // out: entries of all lists
+    uint4* queue;                  // out: units (start, end, super-tile, part or kWholeUnit); those of the
+                                   // head from the front, the others from the back
+    uint32_t* n_queue;             // [2] their counts (zeroed)
+    int64_t queue_cap;
+    int total_super;
     int32_t* status;
     int64_t spin_limit;
+    // zeroed by k_cell_count (the results of a call that stops early)
+    uint2* ranges;
+    int64_t total_tiles;
+    int64_t* n_instances;
+    int64_t* n_needed;             // may be null
 };
 
-// Last position p in [lo, hi) with offsets[p] <= s, given offsets[lo] <= s
-// (the warp probes 32 positions per step).
-__device__ __forceinline__ int64_t warp_search(const uint32_t* offsets, int64_t lo, int64_t hi, uint32_t s, int lane)
+// range: first depth bits, shift; monotone in the key
+__device__ __forceinline__ uint32_t depth_bin(uint2 range, int nbins, uint32_t key)
 {
-    while (hi - lo > 1) {
-        const int64_t step = (hi - lo + 31) / 32;
-        const int64_t p = lo + lane * step;
-        const bool ok = p < hi && offsets[p] <= s;
-        const unsigned m = __ballot_sync(0xffffffffu, ok) | 1u;
-        const int64_t nlo = lo + (31 - __clz(m)) * step;
-        hi = min(hi, nlo + step);
-        lo = nlo;
+    return key > range.x ? min((key - range.x) >> range.y, (uint32_t)nbins - 1u) : 0u;
+}
+
+// Depth bins of view v: the range of the depth bits of 256 of its rows, one per
+// thread, evenly spaced.  About one row in 128 lies outside; a camera far from a
+// small scene, whose depths share their leading bits, gets as fine a division as
+// any other (bins of a fixed part of an octave held a list's whole depth range:
+// 1060 against 340 us for 1M Gaussians seen from 40 times their extent).
+__device__ __forceinline__ uint2 sample_range(const CellArgs& a, int v, uint32_t (*s_mm)[8])
+{
+    const int64_t step = a.n >= 256 ? a.n / 256 : 1, i = threadIdx.x * step;
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    if (i < a.n) {
+        const int64_t r = (int64_t)v * a.n + i;
+        const uint32_t nt = a.proj.n_tiles[r];
+        const uint32_t key = __float_as_uint(((const float4*)a.proj.rgb_depth)[r].w);
+        if (nt > 0) lo = hi = key;
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0) {
+        s_mm[0][threadIdx.x >> 5] = lo;
+        s_mm[1][threadIdx.x >> 5] = hi;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        lo = min(lo, s_mm[0][w]);
+        hi = max(hi, s_mm[1][w]);
+    }
+    if (lo > hi) return make_uint2(0u, 31u);  // none visible in the sample
+    return make_uint2(lo, (uint32_t)min(31, max(0, 32 - __clz(hi - lo) - a.bin_bits)));
+}
+
+// The cells of this block's rows (the same in k_cell_count and k_cell_scatter).
+// Atomics on one cell, and on cells that share a sector, go one after the
+// other; where a batch has few super-tiles, or most rows lie in a few of them,
+// several copies of the cells spread them.
+__device__ __forceinline__ uint32_t* cell_copy(const CellArgs& a)
+{
+    return a.cell + ((size_t)(blockIdx.x & (a.copies - 1)) * a.total_super << a.bin_bits);
+}
+
+// One thread per row, blockIdx.y the view.  Each lane walks its own
+// super-rectangle: the reductions return nothing, so a warp only pays issue
+// slots for its widest row (sharing the entries out over the lanes, as the
+// scatter does, costs the same on wide splats and more on small ones).
+__global__ void __launch_bounds__(256) k_cell_count(CellArgs a)
+{
+    __shared__ uint32_t s_mm[2][8];
+    const int v = blockIdx.y;
+    const int64_t i = blockIdx.x * 256ll + threadIdx.x;
+    const int64_t gt = ((int64_t)v * gridDim.x + blockIdx.x) * 256 + threadIdx.x;
+    for (int64_t t = gt; t < a.total_tiles; t += (int64_t)gridDim.x * gridDim.y * 256) a.ranges[t] = make_uint2(0u, 0u);
+    if (gt == 0) {
+        *a.n_instances = 0;
+        if (a.n_needed) *a.n_needed = 0;
+    }
+    if (status_failed(a.status)) return;
+    const uint2 range = sample_range(a, v, s_mm);
+    uint32_t* cells = cell_copy(a);
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.range[v] = range;
+    if (i >= a.n) return;
+    const int64_t r = (int64_t)v * a.n + i;
+    uint32_t pack = 0u, key = 0u;
+    if (a.proj.n_tiles[r] > 0) {
+        const int4 rc = ((const int4*)a.proj.rect)[r];
+        key = __float_as_uint(((const float4*)a.proj.rgb_depth)[r].w);
+        const int x0 = rc.x >> 3, y0 = rc.y >> 3, x1 = (rc.z + 7) >> 3, y1 = (rc.w + 7) >> 3;
+        if (x1 > x0 && y1 > y0) {
+            pack = (uint32_t)x0 | (uint32_t)y0 << 8 | (uint32_t)x1 << 16 | (uint32_t)y1 << 24;
+            const uint32_t bin = depth_bin(range, a.nbins, key);
+            for (int y = y0; y < y1; ++y) {
+                uint32_t* c = cells + (size_t)(a.super_base[v] + y * a.STX[v]) * a.nbins + bin;
+                for (int x = x0; x < x1; ++x) atomicAdd(c + (size_t)x * a.nbins, 1u);
+            }
+        }
+    }
+    a.rec[r] = make_uint2(pack, key);
+}
+
+// First index of the ascending p[0 .. n) with p[index] >= x (n when none).
+__device__ __forceinline__ int lower_bound(const uint32_t* p, int n, uint32_t x)
+{
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int m = (lo + hi) >> 1;
+        if (p[m] < x) lo = m + 1;
+        else hi = m;
     }
     return lo;
 }
 
-// One warp's slots [sa, sb) of view v, from its row j0 on, in rounds of 32
-// rows: each row's entries whose slot lies in the range, in slot order, ranked
-// per super-tile by ballots over the bits of the super-tile index
-// (depth-ordered rows are scattered over the image, so a round holds many
-// distinct super-tiles, for which a match instruction is slow); the warp's
-// counter of each super-tile advances by its entries.  WRITE: the counters
-// hold the warp's first list slot of every super-tile and each entry is
-// written there.
-template <bool WRITE>
-__device__ __forceinline__ void split_sweep(const SplitArgs& a, int v, int nbits, int64_t j0, uint32_t sa,
-                                            uint32_t sb, uint32_t* cnt, int lane, unsigned lt)
+// Block per super-tile, taken in ticket order (look-back over the super-tiles).
+__global__ void __launch_bounds__(256) k_cell_scan(CellArgs a)
 {
-    const int STX = a.STX[v];
-    const int64_t vend = (int64_t)(v + 1) * a.n;
-    auto emit = [&](bool ok, uint32_t d, uint32_t row) {
-        unsigned peers = __ballot_sync(0xffffffffu, ok);
-        for (int b = 0; b < nbits; ++b) {  // warp-uniform
-            const bool bit = (d >> b) & 1u;
-            const unsigned bb = __ballot_sync(0xffffffffu, bit);
-            peers &= bit ? bb : ~bb;
+    __shared__ uint32_t s_p[kMaxBins + 1];  // first entry of each bin, relative to the list
+    __shared__ uint32_t s_tmp[8];
+    __shared__ unsigned long long s_excl;
+    __shared__ int s_gs;
+    constexpr unsigned long long kA = 1ull << 62, kP = 2ull << 62, kM = (1ull << 62) - 1;
+    if (status_failed(a.status)) return;
+    const int tid = threadIdx.x;
+    if (tid == 0) s_gs = (int)atomicAdd(a.ticket, 1u);
+    __syncthreads();
+    const int gs = s_gs;
+    if (gs >= a.total_super) return;
+    uint32_t* cell = a.cell + (size_t)gs * a.nbins;
+    const size_t copy_stride = (size_t)a.total_super << a.bin_bits;
+    uint32_t c[4] = {0u, 0u, 0u, 0u};
+    const bool quad = a.nbins == kMaxBins;  // four bins per thread, else one
+    for (int k = 0; k < a.copies; ++k) {
+        if (quad) {
+            const uint4 q = ((const uint4*)(cell + k * copy_stride))[tid];
+            c[0] += q.x; c[1] += q.y; c[2] += q.z; c[3] += q.w;
+        } else if (tid < a.nbins) {
+            c[0] += cell[k * copy_stride + tid];
         }
-        if (ok) {
-            const int leader = __ffs(peers) - 1;
-            uint32_t prev = 0;
-            if (lane == leader) {
-                prev = cnt[d];
-                cnt[d] = prev + __popc(peers);
-            }
-            prev = __shfl_sync(peers, prev, leader);
-            if (WRITE) a.list[prev + __popc(peers & lt)] = row;
-        }
-        __syncwarp();
-    };
-    for (int64_t jb = j0;; jb += 32) {
-        const int64_t j = jb + lane;
-        // c entries of row j from its entry kl on fall inside [sa, sb); pk: the
-        // super-rectangle's origin x | y << 10 | width << 20
-        uint32_t row = 0, c = 0, kl = 0, pk = 0;
-        bool past = true;
-        if (j < vend) {
-            const uint32_t off = a.offsets[j];
-            past = off >= sb;
-            if (!past) {
-                row = a.rows[j];
-                const int4 rc = ((const int4*)a.proj.rect)[row];
-                const int sx0 = rc.x >> 3, sy0 = rc.y >> 3, sx1 = (rc.z + 7) >> 3, sy1 = (rc.w + 7) >> 3;
-                if (sx1 > sx0 && sy1 > sy0) {
-                    const uint32_t cr = (uint32_t)((sx1 - sx0) * (sy1 - sy0));
-                    kl = off < sa ? sa - off : 0u;
-                    const uint32_t kh = min(cr, sb - off);
-                    c = kh > kl ? kh - kl : 0u;
-                    pk = (uint32_t)sx0 | (uint32_t)sy0 << 10 | (uint32_t)(sx1 - sx0) << 20;
-                }
-            }
-        }
-        if (__all_sync(0xffffffffu, c <= 1u && kl == 0u)) {  // the common case: a row's first entry at most
-            emit(c == 1u, (pk >> 10 & 1023u) * STX + (pk & 1023u), row);
-        } else {
-            // entry slots of the round in order: lane l owns [e, e + c)
-            uint32_t e = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, e, o);
-                if (lane >= o) e += y;
-            }
-            const uint32_t E = __shfl_sync(0xffffffffu, e, 31);
-            e -= c;
-            for (uint32_t s0 = 0; s0 < E; s0 += 32) {
-                const uint32_t sl = s0 + lane;
-                // the row of slot sl: the last lane whose first slot is at or before it
-                int src = 0;
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1)
-                    if (__shfl_sync(0xffffffffu, e, src + step) <= sl) src += step;
-                const uint32_t srow = __shfl_sync(0xffffffffu, row, src), spk = __shfl_sync(0xffffffffu, pk, src);
-                const uint32_t k = sl - __shfl_sync(0xffffffffu, e, src) + __shfl_sync(0xffffffffu, kl, src);
-                const int w = (int)(spk >> 20);
-                // k / w: an approximate quotient of (k + 1/2) / w (off by at most one), then corrected
-                int ky = w ? (int)__fdividef((float)k + 0.5f, (float)w) : 0, kx = (int)k - ky * w;
-                if (kx < 0) {
-                    --ky;
-                    kx += w;
-                } else if (kx >= w && w) {
-                    ++ky;
-                    kx -= w;
-                }
-                emit(sl < E, ((spk >> 10 & 1023u) + (uint32_t)ky) * STX + (spk & 1023u) + (uint32_t)kx, srow);
-            }
-        }
-        if (__any_sync(0xffffffffu, past)) break;  // offsets grow with j: the later rows are past sb too
     }
-}
-
-// Counting pass of one warp's slots [sa, sb) of view v, from its row j0 on:
-// a row whose entries all fall inside the range adds its super-rectangle to
-// the warp's 2D difference grid diff ((STX + 1) x (STY + 1), zeroed) with four
-// corner updates; the first and last rows of the range, which may fall in it
-// only in part, add their entries inside it to cnt one by one.  The grid's
-// prefix sums are then added to cnt.
-__device__ __forceinline__ void split_count(const SplitArgs& a, int v, int64_t j0, uint32_t sa, uint32_t sb,
-                                            uint32_t* cnt, uint32_t* diff, int lane)
-{
-    const int STX = a.STX[v], SX = STX + 1, SY = a.STY[v] + 1;
-    const int64_t vend = (int64_t)(v + 1) * a.n;
-    for (int64_t jb = j0;; jb += 32) {
-        const int64_t j = jb + lane;
-        bool past = true;
-        if (j < vend) {
-            const uint32_t off = a.offsets[j];
-            past = off >= sb;
-            if (!past) {
-                const int4 rc = ((const int4*)a.proj.rect)[a.rows[j]];
-                const int sx0 = rc.x >> 3, sy0 = rc.y >> 3, sx1 = (rc.z + 7) >> 3, sy1 = (rc.w + 7) >> 3;
-                if (sx1 > sx0 && sy1 > sy0) {
-                    const uint32_t w = (uint32_t)(sx1 - sx0), cr = w * (uint32_t)(sy1 - sy0);
-                    if (off >= sa && cr <= sb - off) {
-                        atomicAdd(&diff[sy0 * SX + sx0], 1u);
-                        atomicAdd(&diff[sy0 * SX + sx1], 0xffffffffu);
-                        atomicAdd(&diff[sy1 * SX + sx0], 0xffffffffu);
-                        atomicAdd(&diff[sy1 * SX + sx1], 1u);
-                    } else {
-                        const uint32_t kh = min(cr, sb - off);
-                        for (uint32_t k = off < sa ? sa - off : 0u; k < kh; ++k) {
-                            const uint32_t ky = k / w;
-                            atomicAdd(&cnt[(sy0 + ky) * STX + sx0 + (k - ky * w)], 1u);
-                        }
+    uint32_t n;
+    uint32_t p = block_excl_scan256(c[0] + c[1] + c[2] + c[3], s_tmp, &n);
+    if (quad) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            s_p[4 * tid + q] = p;
+            p += c[q];
+        }
+    } else if (tid < a.nbins) {
+        s_p[tid] = p;
+    }
+    if (tid == 0) s_p[a.nbins] = n;
+    if (tid < 32) {  // decoupled look-back by one warp, 32 predecessors per round trip
+        unsigned long long excl = 0;
+        if (tid == 0) st_relaxed64(a.lb + gs, (gs == 0 ? kP : kA) | n);
+        if (gs > 0) {
+            int64_t j = gs - 1, spins = 0;
+            for (;;) {
+                const unsigned long long w = j - tid >= 0 ? ld_relaxed64(a.lb + (j - tid)) : kP;
+                const unsigned long long flag = w & ~kM;
+                const unsigned pend = __ballot_sync(0xffffffffu, flag == 0);
+                const unsigned pref = __ballot_sync(0xffffffffu, flag == kP);
+                const int first_pend = pend ? __ffs(pend) - 1 : 32;
+                const int first_pref = pref ? __ffs(pref) - 1 : 32;
+                const bool found = first_pref < first_pend;
+                const int take = found ? first_pref + 1 : first_pend;
+                unsigned long long x = tid < take ? (w & kM) : 0ull;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                excl += x;
+                if (found) break;
+                j -= take;
+                if (take == 0) {
+                    if (++spins > a.spin_limit) {
+                        if (tid == 0) set_status(a.status, SPLAT_ERR_TIMEOUT, SPLAT_STAGE_SCAN, gs);
+                        break;
                     }
+                    if (spins > 64) __nanosleep(64);
                 }
             }
+            if (tid == 0) st_relaxed64(a.lb + gs, kP | ((excl + n) & kM));
         }
-        if (__any_sync(0xffffffffu, past)) break;  // offsets grow with j: the later rows are past sb too
-    }
-    __syncwarp();
-    for (int y = lane; y < SY; y += 32) {  // prefix along x
-        uint32_t run = 0;
-        for (int x = 0; x < SX; ++x) {
-            run += diff[y * SX + x];
-            diff[y * SX + x] = run;
+        if (tid == 0) {
+            s_excl = excl;
+            if (gs == a.total_super - 1) {
+                const int64_t K1 = (int64_t)(excl + n);
+                *a.K1 = K1;
+                if (K1 > a.capacity) set_status(a.status, SPLAT_ERR_CAPACITY, SPLAT_STAGE_SCAN, K1);
+            }
         }
-    }
-    __syncwarp();
-    for (int x = lane; x < SX; x += 32) {  // then along y
-        uint32_t run = 0;
-        for (int y = 0; y < SY; ++y) {
-            run += diff[y * SX + x];
-            diff[y * SX + x] = run;
-        }
-    }
-    __syncwarp();
-    for (int d = lane; d < STX * (SY - 1); d += 32) {
-        const int y = d / STX;
-        cnt[d] += diff[y * SX + (d - y * STX)];
-    }
-    __syncwarp();
-}
-
-__global__ void __launch_bounds__(256) k_super_split(SplitArgs a)
-{
-    extern __shared__ uint32_t s_dyn[];
-    uint32_t* s_cnt = s_dyn;                 // [8][smax] per-warp counters, then the warps' first slots
-    uint32_t* s_start = s_dyn + 8 * a.smax;  // [smax] first list slot of each super-tile of the view
-    uint32_t* s_diff = s_start + a.smax;     // [8][sdiff] per-warp difference grids of the counting pass
-    __shared__ uint32_t s_S[SPLAT_MAX_VIEWS + 1];   // first slot of each view
-    __shared__ uint32_t s_cb[SPLAT_MAX_VIEWS + 1];  // first partition of each view
-    __shared__ unsigned long long s_tmp64[8];
-    __shared__ int64_t s_ticket;
-    if (status_failed(a.status)) return;  // includes K1 above the capacity
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned lt = lanemask_lt();
-    if (tid == 0) {
-        const uint32_t K1 = (uint32_t)*a.n_instances;
-        uint32_t cb = 0;
-        for (int v = 0; v < a.V; ++v) s_S[v] = a.offsets[(int64_t)v * a.n];
-        s_S[a.V] = K1;
-        for (int v = 0; v < a.V; ++v) {  // every view takes a partition, if only to write its ranges
-            s_cb[v] = cb;
-            cb += max(1u, (s_S[v + 1] - s_S[v] + kSplitSlots - 1) / kSplitSlots);
-        }
-        s_cb[a.V] = cb;
     }
     __syncthreads();
-    const int64_t parts = min((int64_t)s_cb[a.V], a.max_parts);
-    int cur_v = -1;
-    for (;;) {
-        if (tid == 0) s_ticket = atomicAdd(a.ticket, 1u);
+    // (starts past 2^32 only arise with K1 beyond any capacity: the check above reports them)
+    const uint32_t start = (uint32_t)s_excl;
+    if (quad) {  // a bin's copies follow one another
+        uint4 at = make_uint4(start + s_p[4 * tid], start + s_p[4 * tid + 1], start + s_p[4 * tid + 2],
+                              start + s_p[4 * tid + 3]);
+        for (int k = 0; k < a.copies; ++k) {
+            uint4* q = (uint4*)(cell + k * copy_stride) + tid;
+            const uint4 x = a.copies > 1 ? *q : make_uint4(0u, 0u, 0u, 0u);
+            *q = at;
+            at.x += x.x; at.y += x.y; at.z += x.z; at.w += x.w;
+        }
+    } else if (tid < a.nbins) {
+        uint32_t at = start + s_p[tid];
+        for (int k = 0; k < a.copies; ++k) {
+            const uint32_t x = cell[k * copy_stride + tid];
+            cell[k * copy_stride + tid] = at;
+            at += x;
+        }
+    }
+    if (tid == 0) a.sranges[gs] = n ? make_uint2(start, start + n) : make_uint2(0u, 0u);
+    if (n <= (uint32_t)kUnit) return;  // one unit, sorted with the head's without a queue entry
+    const uint32_t steps = (n + kUnitStep - 1) / kUnitStep;
+    for (uint32_t k = tid; k < steps; k += 256) {
+        const uint32_t u0 = s_p[lower_bound(s_p, a.nbins, k * kUnitStep)];
+        const uint32_t u1 = s_p[lower_bound(s_p, a.nbins, (k + 1) * kUnitStep)];
+        if (u0 >= u1) continue;  // inside a bin of more than kUnitStep entries
+        const int q = u0 < (uint32_t)kHeadEntries ? 0 : 1;
+        const uint32_t parts = u1 - u0 <= (uint32_t)kUnit ? 1u : (u1 - u0 + kUnitStep - 1) / kUnitStep;
+        const uint32_t at = atomicAdd(&a.n_queue[q], parts);
+        for (uint32_t g = 0; g < parts; ++g) {
+            const int64_t slot = q ? a.queue_cap - 1 - (int64_t)(at + g) : (int64_t)(at + g);
+            if (slot >= 0 && slot < a.queue_cap)  // (it holds every unit of lists within the capacity)
+                a.queue[slot] = make_uint4(start + u0, start + u1, (uint32_t)gs, parts == 1 ? kWholeUnit : g);
+        }
+    }
+}
+
+// A warp takes 32 rows and shares their entries out over its lanes: the
+// position of each comes back from an atomic on its cell's cursor, and a row's
+// entries one after the other would wait for one another's.
+__global__ void __launch_bounds__(256) k_cell_scatter(CellArgs a)
+{
+    if (status_failed(a.status)) return;  // includes K1 above the capacity
+    const int v = blockIdx.y, lane = threadIdx.x & 31;
+    const int64_t i = blockIdx.x * 256ll + threadIdx.x;
+    const uint32_t row = (uint32_t)((int64_t)v * a.n + i);
+    const uint2 rec = i < a.n ? a.rec[row] : make_uint2(0u, 0u);
+    const uint32_t x0 = rec.x & 255u, y0 = rec.x >> 8 & 255u, w = (rec.x >> 16 & 255u) - x0;
+    const uint32_t c = w * ((rec.x >> 24) - y0);
+    // first cell of the row, and of its entries' order in the warp: lane l owns [e, e + c)
+    const uint32_t cell0 = (uint32_t)(a.super_base[v] + (int)y0 * a.STX[v] + (int)x0);
+    const uint32_t bin = depth_bin(a.range[v], a.nbins, rec.y);
+    uint32_t* cells = cell_copy(a);
+    uint32_t e = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, e, o);
+        if (lane >= o) e += y;
+    }
+    const uint32_t E = __shfl_sync(0xffffffffu, e, 31);
+    e -= c;
+    for (uint32_t s0 = 0; s0 < E; s0 += 32) {
+        const uint32_t s = s0 + lane;
+        // the row of entry s: the last lane whose first entry is at or before it
+        int src = 0;
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1)
+            if (__shfl_sync(0xffffffffu, e, src + step) <= s) src += step;
+        const uint32_t k = s - __shfl_sync(0xffffffffu, e, src);
+        const int sw = (int)__shfl_sync(0xffffffffu, w, src);
+        const uint32_t sc = __shfl_sync(0xffffffffu, cell0, src), sbin = __shfl_sync(0xffffffffu, bin, src);
+        const uint32_t skey = __shfl_sync(0xffffffffu, rec.y, src), srow = row - (uint32_t)(lane - src);
+        // k / sw: an approximate quotient of (k + 1/2) / sw (off by at most one), then corrected
+        int ky = sw ? (int)__fdividef((float)k + 0.5f, (float)sw) : 0, kx = (int)k - ky * sw;
+        if (kx < 0) {
+            --ky;
+            kx += sw;
+        } else if (kx >= sw && sw) {
+            ++ky;
+            kx -= sw;
+        }
+        if (s < E) {
+            const size_t cell = (size_t)(sc + (uint32_t)(ky * a.STX[v] + kx)) * a.nbins + sbin;
+            const uint32_t pos = atomicAdd(cells + cell, 1u);
+            if (pos < (uint64_t)a.capacity) a.entries[pos] = make_uint2(srow, skey);
+        }
+    }
+}
+
+struct SortArgs {
+    const uint2* sranges;
+    int total_super;
+    const unsigned long long* entries;  // (row, depth bits) as one word: depth bits << 32 | row
+    uint32_t* list;                     // out: the lists' rows in order
+    const uint4* queue;
+    const uint32_t* n_queue;
+    int64_t queue_cap;
+    const uint2* sat_head;              // the head count's ended tiles (second pass)
+    int32_t* status;
+};
+
+struct SortSmem {
+    unsigned long long e[kUnit];
+    uint32_t h[kSortBuckets + 4];  // bucket counts, then first positions; [kSortBuckets]: the total
+    uint32_t h2[kSortBuckets + 4];  // the same of the second level
+    uint32_t red[4][kUnitThreads / 32], tmp[kUnitThreads / 32];
+    uint32_t n;
+};
+
+// Bounds of a key range and the right shift that maps its differences to
+// kSortBuckets buckets (at least half of them used), order preserved.
+struct KeyRange {
+    unsigned long long lo;
+    int shift;
+};
+
+__device__ __forceinline__ KeyRange key_range(unsigned long long lo, unsigned long long hi)
+{
+    return {lo, max(0, 64 - kSortBucketBits - __clzll((long long)(hi - lo)))};
+}
+
+__device__ __forceinline__ uint32_t key_bucket(const KeyRange& r, unsigned long long e)
+{
+    return (uint32_t)((e - r.lo) >> r.shift);
+}
+
+// Block-wide key range from the threads' own extremes of the depth bits and,
+// should all depths be equal, of the rows.
+__device__ __forceinline__ void block_bounds(SortSmem& s, uint32_t dmin, uint32_t dmax, uint32_t rmin, uint32_t rmax,
+                                             unsigned long long& lo, unsigned long long& hi)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    dmin = __reduce_min_sync(0xffffffffu, dmin);
+    dmax = __reduce_max_sync(0xffffffffu, dmax);
+    rmin = __reduce_min_sync(0xffffffffu, rmin);
+    rmax = __reduce_max_sync(0xffffffffu, rmax);
+    if (lane == 0) {
+        s.red[0][warp] = dmin;
+        s.red[1][warp] = dmax;
+        s.red[2][warp] = rmin;
+        s.red[3][warp] = rmax;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kUnitThreads / 32; ++w) {
+        dmin = min(dmin, s.red[0][w]);
+        dmax = max(dmax, s.red[1][w]);
+        rmin = min(rmin, s.red[2][w]);
+        rmax = max(rmax, s.red[3][w]);
+    }
+    lo = (unsigned long long)dmin << 32 | (dmin == dmax ? rmin : 0u);
+    hi = (unsigned long long)dmax << 32 | (dmin == dmax ? rmax : 0xffffffffu);
+}
+
+// h: bucket counts -> first positions, h[kSortBuckets] the total; returns
+// (block-uniform) whether a bucket is crowded.
+__device__ __forceinline__ bool scan_buckets(SortSmem& s, uint32_t* h)
+{
+    static_assert(kSortBuckets == 4 * kUnitThreads, "four buckets per thread");
+    uint4* h4 = (uint4*)h + threadIdx.x;
+    const uint4 c = *h4;
+    const uint32_t mx = max(max(c.x, c.y), max(c.z, c.w));
+    uint32_t total;
+    const uint32_t x = block_excl_scan<kUnitThreads / 32>(c.x + c.y + c.z + c.w, s.tmp, &total);
+    *h4 = make_uint4(x, x + c.x, x + c.x + c.y, x + c.x + c.y + c.z);
+    if (threadIdx.x == 0) h[kSortBuckets] = total;
+    return __syncthreads_or(mx > kCrowded);
+}
+
+// Every entry of s.e[0 .. n), entry t + kUnitThreads k in e[k] of thread t and b[k] its
+// bucket of first positions h, to its place by the count of smaller ones in its
+// bucket; their rows to dst.
+__device__ __forceinline__ void place_rows(SortSmem& s, const unsigned long long (&e)[kPer],
+                                           uint32_t (&b)[kPer], const uint32_t* h, int n,
+                                           uint32_t* __restrict__ dst)
+{
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if (tid + kUnitThreads * k < n) {
+            const uint32_t j1 = h[b[k] + 1];
+            uint32_t j = h[b[k]], r = j;
+#pragma unroll 1
+            for (; j < j1; ++j) r += s.e[j] < e[k];
+            b[k] = r;
+        }
+    }
+    __syncthreads();
+    uint32_t* rows = (uint32_t*)s.e;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+        if (tid + kUnitThreads * k < n) rows[b[k]] = (uint32_t)e[k];
+    __syncthreads();
+    for (int i = tid; i < n; i += kUnitThreads) dst[i] = rows[i];
+    __syncthreads();
+}
+
+// A unit with crowded buckets, the entries in bucket order in s.e (kr, s.h):
+// many equal depths (means stored in 16 bits seen along an axis, planes facing
+// the camera).  A second counting pass spreads the crowded buckets' entries
+// over their positions by row (in [rmin, rmax]); should such a bucket hold
+// different depths, or the rows crowd as well, the unit is sorted bitonically.
+__device__ __noinline__ void sort_crowded(SortSmem& s, KeyRange kr, uint32_t rmin, uint32_t rmax, int n, uint32_t* dst)
+{
+    const int tid = threadIdx.x, up = __clz(max(1u, rmax - rmin));
+    unsigned long long e[kPer];
+    uint32_t b[kPer], at[kPer];
+    bool mixed = false;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if (tid + kUnitThreads * k < n) {
+            e[k] = s.e[tid + kUnitThreads * k];
+            const uint32_t d = key_bucket(kr, e[k]), p = s.h[d], c = s.h[d + 1] - p;
+            b[k] = p;
+            if (c > kCrowded) {
+                mixed |= (s.e[p] >> 32) != (e[k] >> 32);
+                b[k] = p + __umulhi(((uint32_t)e[k] - rmin) << up, c);
+            }
+        }
+        s.h2[tid + kUnitThreads * k] = 0u;
+    }
+    if (!__syncthreads_or(mixed)) {
+#pragma unroll
+        for (int k = 0; k < kPer; ++k)
+            if (tid + kUnitThreads * k < n) at[k] = atomicAdd(&s.h2[b[k]], 1u);
         __syncthreads();
-        const int64_t ticket = s_ticket;
-        if (ticket >= parts) break;
-        int v = 0;
-        for (int q = 1; q < a.V; ++q)
-            if (ticket >= (int64_t)s_cb[q]) v = q;
-        const int64_t first = s_cb[v], lp = ticket - first;
-        const int nsup = a.STX[v] * a.STY[v];
-        const int nbits = 32 - __clz(max(nsup - 1, 1));  // bits of a super-tile index of the view
-        const int sbase = a.super_base[v];
-        if (v != cur_v) {  // block-uniform: the first list slot of each of the view's super-tiles
-            cur_v = v;
-            unsigned long long before = s_S[v];
-            for (int d0 = 0; d0 < nsup; d0 += 256) {
-                const int d = d0 + tid;
-                const uint32_t c = d < nsup ? a.super_total[sbase + d] : 0u;
-                unsigned long long tot;
-                const unsigned long long ex = block_excl_scan256_u64(c, s_tmp64, &tot);
-                if (d < nsup) s_start[d] = (uint32_t)(before + ex);
-                before += tot;
+        if (!scan_buckets(s, s.h2)) {
+#pragma unroll
+            for (int k = 0; k < kPer; ++k)
+                if (tid + kUnitThreads * k < n) s.e[s.h2[b[k]] + at[k]] = e[k];
+            __syncthreads();
+            place_rows(s, e, b, s.h2, n, dst);
+            return;
+        }
+    }
+    int P = 2;
+    while (P < n) P <<= 1;
+    for (int i = n + tid; i < P; i += kUnitThreads) s.e[i] = ~0ull;
+    __syncthreads();
+    for (int size = 2; size <= P; size <<= 1) {
+        for (int step = size >> 1; step > 0; step >>= 1) {
+            for (int t = tid; t < P / 2; t += kUnitThreads) {
+                const int i = 2 * t - (t & (step - 1)), j = i + step;
+                const unsigned long long x = s.e[i], y = s.e[j];
+                if ((x > y) == ((i & size) == 0)) {
+                    s.e[i] = y;
+                    s.e[j] = x;
+                }
             }
             __syncthreads();
         }
-        if (lp == 0) {
-            for (int d = tid; d < nsup; d += 256) {
-                const uint32_t c = a.super_total[sbase + d], st = s_start[d];
-                a.sranges[sbase + d] = c ? make_uint2(st, st + c) : make_uint2(0u, 0u);
+    }
+    for (int i = tid; i < n; i += kUnitThreads) dst[i] = (uint32_t)s.e[i];
+    __syncthreads();
+}
+
+// Sorts a unit of n <= kUnit entries, entry t + kUnitThreads k in e[k] of thread t, and
+// writes their rows to dst: one counting-sort pass over buckets linear in the
+// key (about one entry each), then every entry counts the smaller ones of its
+// bucket.
+__device__ __forceinline__ void sort_unit(SortSmem& s, const unsigned long long (&e)[kPer], int n,
+                                          uint32_t* __restrict__ dst)
+{
+    const int tid = threadIdx.x;
+    uint32_t dmin = 0xffffffffu, dmax = 0u, rmin = 0xffffffffu, rmax = 0u;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if (tid + kUnitThreads * k < n) {
+            const uint32_t d = (uint32_t)(e[k] >> 32), r = (uint32_t)e[k];
+            dmin = min(dmin, d);
+            dmax = max(dmax, d);
+            rmin = min(rmin, r);
+            rmax = max(rmax, r);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) s.h[tid + kUnitThreads * k] = 0u;
+    unsigned long long lo, hi;
+    block_bounds(s, dmin, dmax, rmin, rmax, lo, hi);
+    const KeyRange kr = key_range(lo, hi);
+    uint32_t at[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+        if (tid + kUnitThreads * k < n) at[k] = atomicAdd(&s.h[key_bucket(kr, e[k])], 1u);
+    __syncthreads();
+    const bool crowded = scan_buckets(s, s.h);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if (tid + kUnitThreads * k < n) {
+            const uint32_t b = key_bucket(kr, e[k]);
+            s.e[s.h[b] + at[k]] = e[k];
+            at[k] = b;
+        }
+    }
+    __syncthreads();
+    if (crowded) {  // (block-uniform)
+#pragma unroll
+        for (int w = 0; w < kUnitThreads / 32; ++w) {  // the block's bounds of the rows, as block_bounds left the warps'
+            rmin = min(rmin, s.red[2][w]);
+            rmax = max(rmax, s.red[3][w]);
+        }
+        sort_crowded(s, kr, rmin, rmax, n, dst);
+    } else {
+        place_rows(s, e, at, s.h, n, dst);
+    }
+}
+
+// f(entry) for every one of src[0 .. n), eight loads in flight per thread (with
+// one a long unit is bound by their latency: 545 -> 160 us for a view whose
+// 300k rows all share one depth).
+template <typename F>
+__device__ __forceinline__ void each_entry(const unsigned long long* __restrict__ src, uint32_t n, F f)
+{
+    for (uint32_t i0 = threadIdx.x; i0 < n; i0 += 8 * kUnitThreads) {
+        unsigned long long x[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) x[k] = i0 + (uint32_t)kUnitThreads * k < n ? src[i0 + (uint32_t)kUnitThreads * k] : 0ull;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (i0 + (uint32_t)kUnitThreads * k < n) f(x[k]);
+    }
+}
+
+// Bucket counts (scanned, in s.h) of those of src[0 .. n) within [lo, hi]; with
+// `all` of every entry, the first and the last bucket open-ended.
+__device__ __forceinline__ KeyRange count_range(SortSmem& s, const unsigned long long* src, uint32_t n,
+                                                unsigned long long lo, unsigned long long hi, bool all = false)
+{
+    const KeyRange kr = key_range(lo, hi);
+    for (int k = threadIdx.x; k < kSortBuckets; k += kUnitThreads) s.h[k] = 0u;
+    __syncthreads();
+    each_entry(src, n, [&](unsigned long long e) {
+        if (all || (e >= lo && e <= hi))
+            atomicAdd(&s.h[e > lo ? min((e - lo) >> kr.shift, (unsigned long long)kSortBuckets - 1) : 0ull], 1u);
+    });
+    __syncthreads();
+    scan_buckets(s, s.h);
+    return kr;
+}
+
+// Part g of a unit of more than kUnit entries (one depth bin of a crowded
+// list): the parts' blocks each count the whole unit by value and take the
+// entries of the g-th run of buckets, about kUnitStep of them, so that any
+// number of blocks share a long unit without waiting for one another.  A run
+// that holds more than kUnit (one crowded bucket) goes through value ranges
+// of at most kUnit entries one after the other, each found by counting again
+// over ever finer buckets (entries are unique, so this ends).
+__device__ __noinline__ void sort_part(SortSmem& s, const unsigned long long* src, uint32_t n, uint32_t g, uint32_t* dst)
+{
+    const int tid = threadIdx.x;
+    // buckets over the range of a sample of kUnit entries, the first and the last open-ended
+    uint32_t dmin = 0xffffffffu, dmax = 0u, rmin = 0xffffffffu, rmax = 0u;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const unsigned long long x = src[(unsigned long long)(tid + kUnitThreads * k) * n / kUnit];
+        dmin = min(dmin, (uint32_t)(x >> 32));
+        dmax = max(dmax, (uint32_t)(x >> 32));
+        rmin = min(rmin, (uint32_t)x);
+        rmax = max(rmax, (uint32_t)x);
+    }
+    unsigned long long lo, hi;
+    block_bounds(s, dmin, dmax, rmin, rmax, lo, hi);
+    __syncthreads();
+    KeyRange kr = count_range(s, src, n, lo, hi, true);
+    const int b0 = lower_bound(s.h, kSortBuckets, g * kUnitStep), b1 = lower_bound(s.h, kSortBuckets, (g + 1) * kUnitStep);
+    uint32_t out = s.h[b0], left = s.h[b1] - out;
+    hi = b1 < kSortBuckets ? lo + ((unsigned long long)b1 << kr.shift) - 1 : ~0ull;
+    lo = b0 > 0 ? lo + ((unsigned long long)b0 << kr.shift) : 0ull;
+    __syncthreads();
+    while (left > 0) {  // (block-uniform) the entries in [lo, hi] are still to be written, from dst[out] on
+        unsigned long long top = hi;
+        uint32_t m = left;
+        while (m > (uint32_t)kUnit && lo < top) {
+            kr = count_range(s, src, n, lo, top);
+            // the buckets below b hold at most kUnit entries, those up to and including b more
+            const int b = lower_bound(s.h, kSortBuckets, kUnit + 1) - 1;
+            m = s.h[b];
+            if (m == 0) {  // bucket b alone holds too many
+                m = s.h[b + 1];
+                lo += (unsigned long long)b << kr.shift;
+                top = min(top, lo + (1ull << kr.shift) - 1);
+            } else {
+                top = lo + ((unsigned long long)b << kr.shift) - 1;
+            }
+            __syncthreads();
+        }
+        m = min(min(m, left), (uint32_t)kUnit);
+        if (m == 0) break;  // (not for consistent counts: bounds the loop whatever the buffer holds)
+        if (tid == 0) s.n = 0u;
+        __syncthreads();
+        each_entry(src, n, [&](unsigned long long x) {
+            if (x >= lo && x <= top) {
+                const uint32_t at = atomicAdd(&s.n, 1u);
+                if (at < (uint32_t)kUnit) s.e[at] = x;
+            }
+        });
+        __syncthreads();
+        unsigned long long e[kPer];
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) e[k] = tid + kUnitThreads * k < (int)m ? s.e[tid + kUnitThreads * k] : 0ull;
+        __syncthreads();
+        sort_unit(s, e, (int)m, dst + out);
+        out += m;
+        left -= m;
+        lo = top + 1;
+    }
+}
+
+// REST false: the lists of at most kUnit entries and the longer lists' units
+// that hold their first kHeadEntries; true: the longer lists' other units,
+// where a tile's list goes on past the head.
+template <bool REST>
+__global__ void __launch_bounds__(kUnitThreads, 2) k_unit_sort(SortArgs a)
+{
+    __shared__ SortSmem s;
+    if (status_failed(a.status)) return;
+    const uint32_t direct = REST ? 0u : (uint32_t)a.total_super;
+    const uint32_t items = direct + a.n_queue[REST ? 1 : 0];
+    for (uint32_t it = blockIdx.x; it < items; it += gridDim.x) {
+        uint32_t st, en, part = kWholeUnit;
+        if (!REST && it < direct) {
+            const uint2 rg = a.sranges[it];
+            st = rg.x;
+            en = rg.y - rg.x <= (uint32_t)kUnit ? rg.y : rg.x;
+        } else {
+            const int64_t q = it - direct;
+            const uint4 u = a.queue[REST ? a.queue_cap - 1 - q : q];
+            st = u.x;
+            en = u.y;
+            part = u.w;
+            if (REST) {
+                const uint2 sat = a.sat_head[u.z];
+                if ((sat.x & sat.y) == 0xffffffffu) continue;  // every list of the super-tile ended in the head
             }
         }
-        // this partition's slots and this warp's share of them
-        const uint32_t s0 = s_S[v] + (uint32_t)lp * kSplitSlots, s1 = min(s_S[v + 1], s0 + kSplitSlots);
-        const uint32_t wa = min(s1, s0 + warp * kSplitWarpSlots), wb = min(s1, wa + kSplitWarpSlots);
-        int64_t j0 = 0;
-        if (wa < wb) j0 = warp_search(a.offsets, (int64_t)v * a.n, (int64_t)(v + 1) * a.n, wa, lane);
-        uint32_t* cnt = s_cnt + warp * a.smax;
-        uint32_t* diff = s_diff + warp * a.sdiff;
-        for (int d = lane; d < nsup; d += 32) cnt[d] = 0u;
-        for (int d = lane; d < (a.STX[v] + 1) * (a.STY[v] + 1); d += 32) diff[d] = 0u;
-        __syncwarp();
-        if (wa < wb) split_count(a, v, j0, wa, wb, cnt, diff, lane);
-        __syncthreads();
-        // per super-tile: prefix over the warps, the partition's count, look-back
-        for (int d = tid; d < nsup; d += 256) {
-            uint32_t run = 0;
+        if (st >= en) continue;  // (block-uniform)
+        const int n = (int)(en - st);
+        if (part == kWholeUnit) {
+            unsigned long long e[kPer];
 #pragma unroll
-            for (int w = 0; w < 8; ++w) {
-                const uint32_t c = s_cnt[w * a.smax + d];
-                s_cnt[w * a.smax + d] = run;
-                run += c;
+            for (int k = 0; k < kPer; ++k) {
+                const int i = (int)threadIdx.x + kUnitThreads * k;
+                e[k] = i < n ? a.entries[st + i] : 0ull;
             }
-            unsigned long long* my = a.lb + ticket * a.smax + d;
-            st_relaxed64(my, (lp == 0 ? kSplitPrefix : kSplitAgg) | run);
-            unsigned long long excl = 0;
-            if (lp > 0) {
-                int64_t j = ticket - 1, spins = 0;  // nearest predecessor not yet added
-                for (;;) {
-                    unsigned long long wd[kLookWindow];
-#pragma unroll
-                    for (int q = 0; q < kLookWindow; ++q)
-                        wd[q] = j - q >= first ? ld_relaxed64(a.lb + (j - q) * a.smax + d) : kSplitPrefix;
-                    int q = 0;
-                    bool found = false;
-#pragma unroll
-                    for (int t = 0; t < kLookWindow; ++t) {
-                        if (found || q < t) continue;  // stopped at an earlier word
-                        const unsigned long long flag = wd[t] & ~kSplitMask;
-                        if (flag == 0) continue;       // not yet published: q stays at t
-                        excl += wd[t] & kSplitMask;
-                        q = t + 1;
-                        found = flag == kSplitPrefix;
-                    }
-                    if (found) break;
-                    j -= q;
-                    if (q == 0) {
-                        if (++spins > a.spin_limit) {
-                            set_status(a.status, SPLAT_ERR_TIMEOUT, SPLAT_STAGE_SCAN, ticket);
-                            break;
-                        }
-                        if (spins > 64) __nanosleep(64);
-                    }
-                }
-                st_relaxed64(my, kSplitPrefix | ((excl + run) & kSplitMask));
-            }
-            const uint32_t base = s_start[d] + (uint32_t)excl;
-#pragma unroll
-            for (int w = 0; w < 8; ++w) s_cnt[w * a.smax + d] += base;
+            sort_unit(s, e, n, a.list + st);
+        } else {
+            sort_part(s, a.entries + st, (uint32_t)n, part, a.list + st);
         }
-        __syncthreads();
-        if (wa < wb && !status_failed(a.status)) split_sweep<true>(a, v, nbits, j0, wa, wb, cnt, lane, lt);
-        __syncthreads();
     }
 }
 
@@ -1099,7 +1374,7 @@ struct TileArgs {
 // margin for the rounding of the T products (a product of (1 - alpha) below
 // e^-9.25 at every pixel; the kernels' T rounds by about 2^-23 an update, which
 // the margin covers for 2e5 updates, and a cut falls within the first
-// kHeadChunks x 256 entries of a list).  The sums are exact integers, so the
+// kHeadEntries entries of a list).  The sums are exact integers, so the
 // cut does not depend on the order of any reduction.
 constexpr float kSatScale = 65536.f;                       // fixed point of -ln(1 - alpha)
 constexpr uint32_t kSatThreshold = (uint32_t)(9.25 * 65536);  // -ln(1e-4) = 9.2103 plus the margin
@@ -1147,7 +1422,6 @@ __device__ __forceinline__ uint32_t sat_weight(const SatRow& r, float xlo, float
 }
 
 constexpr int kFilterSeg = 1024;  // list entries per tail segment (one CTA)
-constexpr int kHeadChunks = 2;    // 256-row chunks of each list the head pass takes in order
 
 // one block (the last of the head count): head length of each super-tile list
 // (its longest tile row's), tail segments per list, exclusive scan -> seg_base
@@ -1393,7 +1667,7 @@ __device__ __forceinline__ bool ellipse_band_extent(const float4& g0, const floa
 }
 
 // Head pass, counting: one CTA per (super-tile, tile row), warp c serving
-// tile column c.  The CTA streams the first kHeadChunks x 256 entries of the
+// tile column c.  The CTA streams the first kHeadEntries entries of the
 // super-tile's list in depth order, 256 at a time.  Thread t takes entry t of
 // the chunk: the entry joins the tile row's queue (in order) when its
 // rectangle covers the row, and then gets its columns in the row (the
@@ -1441,7 +1715,7 @@ __global__ void __launch_bounds__(256, 8) k_head_count(TileArgs a)
     uint32_t cnt = 0u, wsum = 0u;
     if (threadIdx.x == 0) s_sat = 0u;
     const uint2 rgs = a.sranges[gs];
-    const uint32_t end = min(rgs.y, rgs.x + (uint32_t)(kHeadChunks * 256));
+    const uint32_t end = min(rgs.y, rgs.x + (uint32_t)kHeadEntries);
     uint32_t row_end = rgs.x;
     int done = __syncthreads_and(sat);  // block-uniform: every list of the row has ended
     for (uint32_t b = rgs.x; b < end; b += 256) {
@@ -1840,22 +2114,62 @@ __global__ void __launch_bounds__(256) k_tile_filter(TileArgs a)
 
 struct SortLayout {
     int64_t n_rows, capacity;
-    int V, tmax, smax;
+    int V;
     bool binned;
     int64_t parts_d, parts_t, parts_scan, n_chunks;
-    int64_t total_tiles, total_super;
-    int64_t parts_split;
+    int64_t total_tiles, total_super, max_segs;
+    // radix path
     size_t off_dkeys[2], off_dvals[2], off_offsets, off_chunk, off_scan_lb, off_dlb[2], off_tlb[2], off_tkeys,
-        off_tvals, off_hist, off_dhist, off_suptot, off_rlb, off_tickets, off_split_lb, off_total;
-    size_t off_vals1, off_sranges, off_ninst1, off_segbase, off_segcnt, off_segsuper, off_nhead, off_sathead,
-        off_nhead8, off_mask, off_tord;
-    int64_t max_segs;
+        off_tvals, off_hist;
+    // binned path
+    int bin_bits, copies;
+    int64_t queue_cap;
+    size_t off_rec, off_range, off_cell, off_cell_lb, off_queue, off_nqueue, off_rlb, off_total, off_vals1, off_sranges,
+        off_ninst1, off_segbase, off_segcnt, off_segsuper, off_nhead, off_sathead, off_nhead8, off_mask;
+    // both
+    size_t off_tord, off_tickets, zero_begin, zero_end;
     size_t bytes;
 };
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 constexpr int kSuperShift = 3;  // super-tiles of 8 x 8 tiles
+
+// Bytes the workspace took when both paths sorted the rows by depth with radix
+// passes.  It stays the least that is asked for, so that the sizes callers hold
+// and the limit of splat_bin_sort_noalloc are what they were.
+static size_t legacy_bytes(const SortLayout& L, int64_t n_rows, int64_t capacity, int V, int smax)
+{
+    size_t o = 0;
+    auto take = [&](size_t bytes) { o = align256(o + std::max<size_t>(bytes, 4)); };
+    const size_t rows = (size_t)n_rows, cap = (size_t)capacity, S = (size_t)L.total_super;
+    const size_t parts_d = V > 0 ? (size_t)(V * ((n_rows / V + 4095) / 4096)) : 0, parts_c = (cap + 4095) / 4096;
+    for (int b = 0; b < 5; ++b) take(4 * rows);
+    take(L.binned ? 4 : 4 * ((cap + kDupChunk - 1) / kDupChunk + 1));
+    take(8 * std::max<size_t>((rows + 4095) / 4096, 1));
+    for (int b = 0; b < 2; ++b) take(1024 * std::max<size_t>(parts_d, 1));
+    for (int b = 0; b < 2; ++b) take(1024 * std::max<size_t>(L.binned ? 0 : parts_c, 1));
+    for (int b = 0; b < 2; ++b) take(L.binned ? 4 : 4 * cap);
+    take(1024 * 9);
+    take(4096 * (size_t)std::max(V, 1));
+    take(L.binned ? 4 * S : 4);
+    take(8 * (size_t)((L.total_tiles + 255) / 256 + 1));
+    take(2 * kOrderClasses * 4);
+    take(64);
+    take(L.binned ? 8 * (size_t)smax * std::max<size_t>(parts_c + (size_t)V, 1) : 4);
+    take(L.binned ? 4 * (size_t)L.total_tiles : 4);
+    take(L.binned ? 4 * cap : 4);
+    take(L.binned ? 8 * S : 4);
+    take(8);
+    take(4 * (S + 1));
+    take(L.binned ? 256 * (size_t)L.max_segs : 4);
+    take(L.binned ? 4 * (size_t)L.max_segs : 4);
+    take(4 * std::max<size_t>(S, 1));
+    take(8 * std::max<size_t>(S, 1));
+    take(32 * std::max<size_t>(S, 1));
+    take(L.binned ? 8 * cap : 4);
+    return o;
+}
 
 SortLayout sort_layout(int64_t n_rows, int64_t capacity, int V, const int* TX, const int* TY, int tile_sort)
 {
@@ -1871,56 +2185,76 @@ SortLayout sort_layout(int64_t n_rows, int64_t capacity, int V, const int* TX, c
         L.total_tiles += (int64_t)TX[v] * TY[v];
         L.total_super += (int64_t)sx * sy;
     }
-    L.tmax = (tmax + 3) & ~3;
-    L.smax = (smax + 3) & ~3;
-    // the split packs super-tile coordinates in 10 bits and keeps 9 counters per super-tile and 8 difference
-    // grids in shared memory
+    smax = (smax + 3) & ~3;
+    // views of up to kBinMaxTiles tiles, or (forced) those whose super-tile grids fit the split's former
+    // shared-memory counters
     int sdiff = 0;
-    bool split_ok = true;
-    for (int v = 0; v < V; ++v) {
-        const int sx = (TX[v] + 7) >> kSuperShift, sy = (TY[v] + 7) >> kSuperShift;
-        split_ok = split_ok && sx < 1024 && sy < 1024;
-        sdiff = std::max(sdiff, (sx + 1) * (sy + 1));
-    }
-    split_ok = split_ok && 4 * (9 * (int64_t)L.smax + 8 * (int64_t)sdiff) <= kSplitMaxSmem;
+    for (int v = 0; v < V; ++v)
+        sdiff = std::max(sdiff, (((TX[v] + 7) >> kSuperShift) + 1) * (((TY[v] + 7) >> kSuperShift) + 1));
+    const bool split_ok = 4 * (9 * (int64_t)smax + 8 * (int64_t)sdiff) <= kSplitMaxSmem;
     L.binned = split_ok && (tile_sort == 2 || (tile_sort == 0 && tmax <= kBinMaxTiles));
-    L.parts_d = V > 0 ? (int64_t)V * ((n_rows / V + kSortPart - 1) / kSortPart) : 0;  // partitions within views
-    L.parts_t = L.binned ? 0 : (capacity + kSortPart - 1) / kSortPart;
-    L.parts_scan = (n_rows + kScanPart - 1) / kScanPart;
-    L.parts_split = L.binned ? (capacity + kSplitSlots - 1) / kSplitSlots + V : 0;
-    L.n_chunks = L.binned ? 1 : (capacity + kDupChunk - 1) / kDupChunk + 1;
+    L.max_segs = L.binned ? (capacity + kFilterSeg - 1) / kFilterSeg + L.total_super : 1;
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align256(o + std::max<size_t>(bytes, 4)); return r; };
-    for (int b = 0; b < 2; ++b) L.off_dkeys[b] = take(4 * (size_t)n_rows);
-    for (int b = 0; b < 2; ++b) L.off_dvals[b] = take(4 * (size_t)n_rows);
-    L.off_offsets = take(4 * (size_t)n_rows);
-    L.off_chunk = take(4 * (size_t)L.n_chunks);
-    L.off_scan_lb = take(8 * (size_t)std::max<int64_t>(L.parts_scan, 1));
-    for (int b = 0; b < 2; ++b) L.off_dlb[b] = take(4 * (size_t)kRadix * std::max<int64_t>(L.parts_d, 1));
-    for (int b = 0; b < 2; ++b) L.off_tlb[b] = take(4 * (size_t)kRadix * std::max<int64_t>(L.parts_t, 1));
-    L.off_tkeys = take(L.binned ? 4 : 4 * (size_t)capacity);
-    L.off_tvals = take(L.binned ? 4 : 4 * (size_t)capacity);
-    L.off_hist = take(4 * (size_t)kRadix * 9);
-    // zeroed together with hist: the depth digits per view and the super-tile list sizes
-    L.off_dhist = take(4 * (size_t)kRadix * 4 * std::max(V, 1));
-    L.off_suptot = take(L.binned ? 4 * (size_t)L.total_super : 4);
-    L.off_rlb = take(8 * (size_t)((L.total_tiles + kRangeTiles - 1) / kRangeTiles + 1));  // tile ranges' look-back
-    L.off_tord = take(2 * kOrderClasses * 4);  // tile-order class counts and cursors
-    L.off_tickets = take(4 * 16);
-    L.off_split_lb = take(L.binned ? 8 * (size_t)L.smax * std::max<int64_t>(L.parts_split, 1) : 4);
-    L.off_total = take(L.binned ? 4 * (size_t)L.total_tiles : 4);
-    L.off_vals1 = take(L.binned ? 4 * (size_t)capacity : 4);
-    L.off_sranges = take(L.binned ? 8 * (size_t)L.total_super : 4);
-    L.off_ninst1 = take(8);
-    L.max_segs = L.binned ? (capacity + kFilterSeg - 1) / kFilterSeg + L.total_super : 1;
-    L.off_segbase = take(4 * (size_t)(L.total_super + 1));
-    L.off_segcnt = take(L.binned ? 4 * 64 * (size_t)L.max_segs : 4);
-    L.off_segsuper = take(L.binned ? 4 * (size_t)L.max_segs : 4);
-    L.off_nhead = take(4 * (size_t)std::max<int64_t>(L.total_super, 1));
-    L.off_sathead = take(8 * (size_t)std::max<int64_t>(L.total_super, 1));
-    L.off_nhead8 = take(32 * (size_t)std::max<int64_t>(L.total_super, 1));
-    L.off_mask = take(L.binned ? 8 * (size_t)capacity : 4);
-    L.bytes = o;
+    if (!L.binned) {
+        L.parts_d = (n_rows + kSortPart - 1) / kSortPart;
+        L.parts_t = (capacity + kSortPart - 1) / kSortPart;
+        L.parts_scan = (n_rows + kScanPart - 1) / kScanPart;
+        L.n_chunks = (capacity + kDupChunk - 1) / kDupChunk + 1;
+        for (int b = 0; b < 2; ++b) L.off_dkeys[b] = take(4 * (size_t)n_rows);
+        for (int b = 0; b < 2; ++b) L.off_dvals[b] = take(4 * (size_t)n_rows);
+        L.off_offsets = take(4 * (size_t)n_rows);
+        L.off_chunk = take(4 * (size_t)L.n_chunks);
+        L.off_scan_lb = take(8 * (size_t)std::max<int64_t>(L.parts_scan, 1));
+        for (int b = 0; b < 2; ++b) L.off_dlb[b] = take(4 * (size_t)kRadix * std::max<int64_t>(L.parts_d, 1));
+        for (int b = 0; b < 2; ++b) L.off_tlb[b] = take(4 * (size_t)kRadix * std::max<int64_t>(L.parts_t, 1));
+        L.off_tkeys = take(4 * (size_t)capacity);
+        L.off_tvals = take(4 * (size_t)capacity);
+        L.zero_begin = L.off_hist = take(4 * (size_t)kRadix * 9);
+        L.off_tickets = take(4 * 16);
+        L.zero_end = o;
+        L.off_tord = take(2 * kOrderClasses * 4);  // tile-order class counts and cursors
+    }
+    const size_t legacy = legacy_bytes(L, n_rows, capacity, V, smax);
+    if (L.binned) {
+        L.off_total = take(4 * (size_t)L.total_tiles);
+        L.off_vals1 = take(4 * (size_t)capacity);
+        L.off_sranges = take(8 * (size_t)L.total_super);
+        L.off_ninst1 = take(8);
+        L.off_segbase = take(4 * (size_t)(L.total_super + 1));
+        L.off_segcnt = take(4 * 64 * (size_t)L.max_segs);
+        L.off_segsuper = take(4 * (size_t)L.max_segs);
+        L.off_nhead = take(4 * (size_t)std::max<int64_t>(L.total_super, 1));
+        L.off_sathead = take(8 * (size_t)std::max<int64_t>(L.total_super, 1));
+        L.off_nhead8 = take(32 * (size_t)std::max<int64_t>(L.total_super, 1));
+        L.off_mask = take(8 * (size_t)capacity);  // the unsorted entries, then the coverage words
+        L.off_rec = take(8 * (size_t)n_rows);
+        L.off_range = take(8 * (size_t)std::max(V, 1));
+        // units of lists of more than kUnit entries: at most 2 n / kUnitStep + 1 of a list of n
+        const int64_t per_view = V > 0 ? n_rows / V : 0;
+        const int64_t most = std::min<int64_t>(capacity, per_view * L.total_super);
+        L.queue_cap = 5 * (most / kUnit) + 8;
+        L.off_queue = take(16 * (size_t)L.queue_cap);
+        L.zero_begin = L.off_nqueue = take(8);
+        L.off_tickets = take(4 * 16);
+        L.off_cell_lb = take(8 * (size_t)L.total_super);
+        L.off_rlb = take(8 * (size_t)((L.total_tiles + kRangeTiles - 1) / kRangeTiles + 1));
+        L.off_tord = take(2 * kOrderClasses * 4);
+        // depth bins: 1024 where lists are long (their cells then hold a few entries), 64 where a list is
+        // about one unit; fewer where the cells would not fit the workspace
+        L.bin_bits = n_rows >= 512 * L.total_super ? 10 : 6;
+        while (L.bin_bits > 0 && align256(o + (4 * (size_t)L.total_super << L.bin_bits)) > legacy) L.bin_bits -= 2;
+        const size_t cell_bytes = 4 * (size_t)L.total_super << L.bin_bits;
+        // copies while they stay within 4 MB (8 for a view of 1352x1014, 1 for four of 2704x2028): 1M Gaussians
+        // seen in a 128x128 view sort in 432 us with one copy, 337 with two, 270 with eight; the scan's extra
+        // reads cost a view of 300k about 1 us
+        for (L.copies = 1; L.copies < 8 && 2 * L.copies * cell_bytes <= (4u << 20) &&
+                           align256(o + 2 * L.copies * cell_bytes) <= legacy;)
+            L.copies *= 2;
+        L.off_cell = take(L.copies * cell_bytes);
+        L.zero_end = o;
+    }
+    L.bytes = std::max(o, legacy);
     return L;
 }
 
@@ -1972,165 +2306,79 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
     auto U = [&](size_t off) { return (uint32_t*)(w + off); };
     cudaStream_t s = ctx.stream;
     cudaError_t err;
-    if ((err = cudaMemsetAsync(w + L.off_hist, 0, (L.off_tickets - L.off_hist) + 64, s)) != cudaSuccess) return err;
-    if ((err = cudaMemsetAsync(bins.ranges, 0, sizeof(uint32_t) * 2 * (size_t)vb.total_tiles, s)) != cudaSuccess)
-        return err;
-    if ((err = cudaMemsetAsync(bins.n_instances, 0, sizeof(int64_t), s)) != cudaSuccess) return err;
-    if (bins.n_needed && (err = cudaMemsetAsync(bins.n_needed, 0, sizeof(int64_t), s)) != cudaSuccess) return err;
+    if ((err = cudaMemsetAsync(w + L.zero_begin, 0, L.zero_end - L.zero_begin, s)) != cudaSuccess) return err;
+    if (n_rows == 0 || !L.binned) {  // (k_cell_count clears them otherwise)
+        if ((err = cudaMemsetAsync(bins.ranges, 0, sizeof(uint32_t) * 2 * (size_t)vb.total_tiles, s)) != cudaSuccess)
+            return err;
+        if ((err = cudaMemsetAsync(bins.n_instances, 0, sizeof(int64_t), s)) != cudaSuccess) return err;
+        if (bins.n_needed && (err = cudaMemsetAsync(bins.n_needed, 0, sizeof(int64_t), s)) != cudaSuccess) return err;
+    }
     if (n_rows == 0) return cudaSuccess;
-    uint32_t* hist = U(L.off_hist);
     uint32_t* tickets = U(L.off_tickets);
-    const int resident = ctx.num_sms * sort_ctas_per_sm();
-
-    // super-tile grids (binned path)
-    int super_base[SPLAT_MAX_VIEWS + 1], STX[SPLAT_MAX_VIEWS], STY[SPLAT_MAX_VIEWS];
-    int sb = 0;
-    for (int v = 0; v < vb.V; ++v) {
-        super_base[v] = sb;
-        STX[v] = (vb.v[v].TX + 7) >> kSuperShift;
-        STY[v] = (vb.v[v].TY + 7) >> kSuperShift;
-        sb += STX[v] * STY[v];
-    }
-    super_base[vb.V] = sb;
-    int sdiff = 0;  // words of the largest view's super-tile difference grid
-    for (int v = 0; v < vb.V; ++v) sdiff = std::max(sdiff, (STX[v] + 1) * (STY[v] + 1));
-    // 1. depth keys + per-view digit counts and (binned) the super-tile list sizes; zero the first depth
-    // look-back buffer, the scan's and the split's
-    uint32_t* dhist = U(L.off_dhist);
-    uint32_t* suptot = U(L.off_suptot);
-    {
-        DepthArgs a{};
-        a.proj = proj;
-        a.V = vb.V;
-        a.keys = U(L.off_dkeys[0]);
-        a.vals = U(L.off_dvals[0]);
-        a.dhist = dhist;
-        a.super_total = L.binned ? suptot : nullptr;
-        for (int v = 0; v < vb.V; ++v) {
-            a.super_base[v] = super_base[v];
-            a.STX[v] = STX[v];
-            a.STY[v] = STY[v];
-        }
-        a.zero_a = U(L.off_dlb[0]);
-        a.n_zero_a = L.parts_d * kRadix;
-        a.zero_b = (unsigned long long*)(w + L.off_scan_lb);
-        a.n_zero_b = L.parts_scan;
-        a.zero_c = (unsigned long long*)(w + L.off_split_lb);
-        a.n_zero_c = L.binned ? L.parts_split * L.smax : 0;
-        const size_t smem = L.binned ? 4 * (size_t)sdiff : 0;
-        static size_t smem_set = 0;
-        if (smem > smem_set) {
-            if ((err = cudaFuncSetAttribute(k_depth_keys, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-                cudaSuccess)
-                return err;
-            smem_set = smem;
-        }
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_depth_keys, 256, smem) != cudaSuccess ||
-            per_sm < 1)
-            per_sm = 1;
-        a.blocks_per_view = (int)std::max<int64_t>(
-            1, std::min<int64_t>((proj.n + 255) / 256, (int64_t)ctx.num_sms * per_sm / vb.V));
-        count_launch();
-        k_depth_keys<<<vb.V * a.blocks_per_view, 256, smem, s>>>(a);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    }
-    // 2. depth passes (buffers 0 -> 1 -> 0 -> 1 -> 0).  Binned: each view's rows sorted in place, giving the
-    // (view, depth) order the super-tile split takes.  Radix path: one sort of all rows by depth, so that
-    // the rows without tiles come last (the duplication's chunks assume no such row between listed ones)
-    const int passes = 4;
-    for (int p = 0; p < passes; ++p) {
-        PassArgs a{};
-        a.keys_in = U(L.off_dkeys[p & 1]);
-        a.vals_in = U(L.off_dvals[p & 1]);
-        a.keys_out = p + 1 < passes ? U(L.off_dkeys[(p + 1) & 1]) : nullptr;
-        a.vals_out = U(L.off_dvals[(p + 1) & 1]);
-        a.n_dev = nullptr;
-        a.n_host = n_rows;
-        a.cap = n_rows;
-        a.hist = dhist + (size_t)p * vb.V * kRadix;
-        a.lb = U(L.off_dlb[p & 1]);
-        a.lb_next = p + 1 < passes ? U(L.off_dlb[(p + 1) & 1]) : nullptr;
-        a.ticket = tickets + p;
-        a.status = status;
-        a.stage = SPLAT_STAGE_DEPTH_SORT;
-        a.shift = 8 * p;
-        a.spin_limit = ctx.spin_limit;
-        a.seg_len = L.binned ? proj.n : 0;
-        a.hist_sum = vb.V;
-        a.ballot_rank = p < 3;  // the low depth digits take many values in a warp, the top one few
-        if ((err = run_pass(a, L.parts_d, resident, s)) != cudaSuccess) return err;
-    }
-    const uint32_t* rows = U(L.off_dvals[passes & 1]);
     if (L.binned) {
-        // 3. super-tile lists.  The scan of the rows' super-tile counts gives each row its first slot and K1;
-        // the lists (K1 entries) live in a capacity-sized buffer, so K1 is checked there, before anything is
-        // written (K itself is checked by the tile ranges once the tile lists are counted).  Then the stable
-        // split of the slots by super-tile.
-        {
-            ScanArgs a{};
-            a.rows = rows;
-            a.n_tiles = proj.n_tiles;
-            a.rect = (const int4*)proj.rect;
-            a.shift = kSuperShift;
-            a.n_rows = n_rows;
-            a.offsets = U(L.off_offsets);
-            a.chunk_row = U(L.off_chunk);
-            a.n_chunks_max = 0;
-            a.lb = (unsigned long long*)(w + L.off_scan_lb);
-            a.ticket = tickets + 4;
-            a.n_instances = (int64_t*)(w + L.off_ninst1);
-            a.n_needed = nullptr;
-            a.capacity = bins.capacity;
-            a.status = status;
-            a.spin_limit = ctx.spin_limit;
-            const int blocks = (int)std::min<int64_t>(L.parts_scan, (int64_t)ctx.num_sms * 4);
-            count_launch();
-            k_scan_tiles<<<blocks, kScanThreads, 0, s>>>(a);
-            if ((err = cudaGetLastError()) != cudaSuccess) return err;
+        // super-tile grids
+        int super_base[SPLAT_MAX_VIEWS + 1], STX[SPLAT_MAX_VIEWS];
+        int sb = 0;
+        for (int v = 0; v < vb.V; ++v) {
+            super_base[v] = sb;
+            STX[v] = (vb.v[v].TX + 7) >> kSuperShift;
+            sb += STX[v] * ((vb.v[v].TY + 7) >> kSuperShift);
         }
-        {
-            SplitArgs a{};
-            a.proj = proj;
-            a.rows = rows;
-            a.offsets = U(L.off_offsets);
-            a.super_total = suptot;
-            a.n_instances = (const int64_t*)(w + L.off_ninst1);
-            a.V = vb.V;
-            a.n = proj.n;
-            a.smax = L.smax;
-            a.sdiff = sdiff;
-            a.total_super = sb;
-            for (int v = 0; v <= vb.V; ++v) a.super_base[v] = super_base[v];
-            for (int v = 0; v < vb.V; ++v) {
-                a.STX[v] = STX[v];
-                a.STY[v] = STY[v];
-            }
-            a.lb = (unsigned long long*)(w + L.off_split_lb);
-            a.max_parts = L.parts_split;
-            a.ticket = tickets + 9;
-            a.list = U(L.off_vals1);
-            a.sranges = (uint2*)(w + L.off_sranges);
-            a.status = status;
-            a.spin_limit = ctx.spin_limit;
-            const size_t smem = 4 * ((size_t)L.smax * 9 + 8 * (size_t)sdiff);
-            static size_t smem_set = 0;
-            if (smem > smem_set) {
-                if ((err = cudaFuncSetAttribute(k_super_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)smem)) != cudaSuccess)
-                    return err;
-                smem_set = smem;
-            }
-            int per_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_super_split, 256, smem) != cudaSuccess ||
-                per_sm < 1)
-                per_sm = 1;
-            const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(L.parts_split, (int64_t)ctx.num_sms * per_sm));
-            count_launch();
-            k_super_split<<<blocks, 256, smem, s>>>(a);
-            if ((err = cudaGetLastError()) != cudaSuccess) return err;
-        }
-        // 4. tile level: per-super-tile lists filtered into per-tile lists (see above)
+        super_base[vb.V] = sb;
+        // 1. the super-tile lists, unsorted inside their cells.  The lists (K1 entries) live in a
+        // capacity-sized buffer, so K1 is checked by the scan, before anything is written (K itself is
+        // checked by the tile ranges once the tile lists are counted)
+        CellArgs c{};
+        c.proj = proj;
+        c.V = vb.V;
+        c.bin_bits = L.bin_bits;
+        c.copies = L.copies;
+        c.nbins = 1 << L.bin_bits;
+        c.n = proj.n;
+        c.range = (uint2*)(w + L.off_range);
+        for (int v = 0; v < vb.V; ++v) c.STX[v] = STX[v];
+        for (int v = 0; v <= vb.V; ++v) c.super_base[v] = super_base[v];
+        c.rec = (uint2*)(w + L.off_rec);
+        c.cell = U(L.off_cell);
+        c.entries = (uint2*)(w + L.off_mask);
+        c.capacity = bins.capacity;
+        c.lb = (unsigned long long*)(w + L.off_cell_lb);
+        c.ticket = tickets;
+        c.sranges = (uint2*)(w + L.off_sranges);
+        c.K1 = (int64_t*)(w + L.off_ninst1);
+        c.queue = (uint4*)(w + L.off_queue);
+        c.n_queue = U(L.off_nqueue);
+        c.queue_cap = L.queue_cap;
+        c.total_super = sb;
+        c.status = status;
+        c.spin_limit = ctx.spin_limit;
+        c.ranges = (uint2*)bins.ranges;
+        c.total_tiles = vb.total_tiles;
+        c.n_instances = bins.n_instances;
+        c.n_needed = bins.n_needed;
+        const dim3 row_grid((unsigned)((proj.n + 255) / 256), (unsigned)vb.V);
+        count_launch(3);
+        k_cell_count<<<row_grid, 256, 0, s>>>(c);
+        k_cell_scan<<<sb, 256, 0, s>>>(c);
+        k_cell_scatter<<<row_grid, 256, 0, s>>>(c);
+        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+        // 2. the units of each list that the head pass takes, in order
+        SortArgs u{};
+        u.sranges = (const uint2*)(w + L.off_sranges);
+        u.total_super = sb;
+        u.entries = (const unsigned long long*)(w + L.off_mask);
+        u.list = U(L.off_vals1);
+        u.queue = (const uint4*)(w + L.off_queue);
+        u.n_queue = U(L.off_nqueue);
+        u.queue_cap = L.queue_cap;
+        u.sat_head = (const uint2*)(w + L.off_sathead);
+        u.status = status;
+        static const int per_sm_u[2] = {ctas_per_sm(k_unit_sort<false>, kUnitThreads),
+                                          ctas_per_sm(k_unit_sort<true>, kUnitThreads)};
+        auto blocks_u = [&](int rest) {
+            return (int)std::min<int64_t>(L.queue_cap + (rest ? 0 : sb), (int64_t)ctx.num_sms * per_sm_u[rest]);
+        };
+        // 3. tile level: per-super-tile lists filtered into per-tile lists (see above)
         TileArgs t{};
         t.proj = proj;
         t.V = vb.V;
@@ -2164,10 +2412,10 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         t.n_head8 = U(L.off_nhead8);
         t.sat_head = (uint2*)(w + L.off_sathead);
         t.mask = (uint2*)(w + L.off_mask);
-        t.ticket = tickets + 10;
+        t.ticket = tickets + 1;
         TileRangeArgs tr{};
         tr.lb = (unsigned long long*)(w + L.off_rlb);
-        tr.ticket = tickets + 13;
+        tr.ticket = tickets + 4;
         tr.ranges = (uint2*)bins.ranges;
         tr.K_out = bins.n_instances;
         tr.capacity = bins.capacity;
@@ -2176,28 +2424,71 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         tr.cls = bins.tile_order ? U(L.off_tord) : nullptr;
         tr.spin_limit = ctx.spin_limit;
         // the head of each super-tile list in order (each tile's list up to its
-        // saturation), the tail in parallel segments, the prefix over head and
-        // segments with the ranges, K and the capacity check, then the heads'
-        // and segments' writes in one pass
+        // saturation), the rest of the units and the tail in parallel segments, the
+        // prefix over head and segments with the ranges, K and the capacity check,
+        // then the heads' and segments' writes in one pass
         static const int per_sm_f[2] = {ctas_per_sm(k_tile_filter<false>, 256), ctas_per_sm(k_tile_filter<true>, 256)};
         auto blocks_f = [&](int c) {
             return (int)std::min<int64_t>(L.max_segs + (c ? 0 : sb), (int64_t)ctx.num_sms * per_sm_f[c]);
         };
-        count_launch(4);
+        count_launch(6);
+        k_unit_sort<false><<<blocks_u(0), kUnitThreads, 0, s>>>(u);
         k_head_count<<<8 * sb, 256, 0, s>>>(t);
+        k_unit_sort<true><<<blocks_u(1), kUnitThreads, 0, s>>>(u);
         k_tile_filter<true><<<blocks_f(1), 256, 0, s>>>(t);
         k_tile_ranges<<<(int)((vb.total_tiles + kRangeTiles - 1) / kRangeTiles), 256, 0, s>>>(t, tr);
         k_tile_filter<false><<<blocks_f(0), 256, 0, s>>>(t);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         return launch_tile_order(bins, L.total_tiles, U(L.off_tord), status, ctx, true);
     }
-    // 3. radix path: scan of the per-row tile counts in depth order
+    // radix path: 1. depth keys + digit counts; zero the first depth look-back buffer and the scan's
+    uint32_t* hist = U(L.off_hist);
+    const int resident = ctx.num_sms * sort_ctas_per_sm();
+    {
+        DepthArgs a{};
+        a.proj = proj;
+        a.n_rows = n_rows;
+        a.keys = U(L.off_dkeys[0]);
+        a.vals = U(L.off_dvals[0]);
+        a.dhist = hist;
+        a.zero_a = U(L.off_dlb[0]);
+        a.n_zero_a = L.parts_d * kRadix;
+        a.zero_b = (unsigned long long*)(w + L.off_scan_lb);
+        a.n_zero_b = L.parts_scan;
+        const int blocks = (int)std::min<int64_t>((n_rows + 255) / 256, (int64_t)ctx.num_sms * 8);
+        count_launch();
+        k_depth_keys<<<blocks, 256, 0, s>>>(a);
+        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    }
+    // 2. depth passes (buffers 0 -> 1 -> 0 -> 1 -> 0): all rows by depth, those without tiles last (the
+    // duplication's chunks assume no such row between listed ones)
+    const int passes = 4;
+    for (int p = 0; p < passes; ++p) {
+        PassArgs a{};
+        a.keys_in = U(L.off_dkeys[p & 1]);
+        a.vals_in = U(L.off_dvals[p & 1]);
+        a.keys_out = p + 1 < passes ? U(L.off_dkeys[(p + 1) & 1]) : nullptr;
+        a.vals_out = U(L.off_dvals[(p + 1) & 1]);
+        a.n_dev = nullptr;
+        a.n_host = n_rows;
+        a.cap = n_rows;
+        a.hist = hist + p * kRadix;
+        a.lb = U(L.off_dlb[p & 1]);
+        a.lb_next = p + 1 < passes ? U(L.off_dlb[(p + 1) & 1]) : nullptr;
+        a.ticket = tickets + p;
+        a.status = status;
+        a.stage = SPLAT_STAGE_DEPTH_SORT;
+        a.shift = 8 * p;
+        a.spin_limit = ctx.spin_limit;
+        a.ballot_rank = p < 3;  // the low depth digits take many values in a warp, the top one few
+        if ((err = run_pass(a, L.parts_d, resident, s)) != cudaSuccess) return err;
+    }
+    const uint32_t* rows = U(L.off_dvals[passes & 1]);
+    // 3. scan of the per-row tile counts in depth order
     {
         ScanArgs a{};
         a.rows = rows;
         a.n_tiles = proj.n_tiles;
-        a.rect = (const int4*)proj.rect;
-        a.shift = 0;
         a.n_rows = n_rows;
         a.offsets = U(L.off_offsets);
         a.chunk_row = U(L.off_chunk);
@@ -2214,7 +2505,7 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         k_scan_tiles<<<blocks, kScanThreads, 0, s>>>(a);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
     }
-    // 4. radix path: duplicate, tile-digit passes, ranges
+    // 4. duplicate, tile-digit passes, ranges
     int bits = 1;
     while ((1ll << bits) < (int64_t)vb.total_tiles) ++bits;
     const int tile_passes = (bits + 7) / 8;
@@ -2256,7 +2547,6 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         a.n_host = 0;
         a.cap = bins.capacity;
         a.hist = hist + (4 + p) * kRadix;
-        a.hist_sum = 1;
         a.lb = U(L.off_tlb[p & 1]);
         a.lb_next = p + 1 < tile_passes ? U(L.off_tlb[(p + 1) & 1]) : nullptr;
         a.ticket = tickets + 5 + p;
