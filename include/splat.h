@@ -541,7 +541,8 @@ void splat_set_spin_limit(int64_t iterations);
 /*
  * Tuning knob of the compositing kernels: pixels each lane owns (2, 4 or 8,
  * evaluated in pairs; one warp covers 32 x that many pixels of a 16x16
- * tile).  Other values are ignored.  Default 8 / 8.  Host-side global (the library default
+ * tile).  Other values are ignored.  Until it is called each launch chooses by
+ * its number of tiles.  Host-side global (the library default
  * of splat_options.pixels_per_lane_*); the results do not depend
  * on it beyond floating-point summation order of the gradients.
  */

@@ -84,7 +84,7 @@ size_t densify_workspace(int64_t n3, int64_t cap3, int64_t n4, int64_t cap4, int
 // overrides them field by field.
 static std::atomic<int64_t> g_spin_limit{1ll << 22};
 std::atomic<int64_t> g_launches{0};
-static std::atomic<int> g_ppl_fwd{8}, g_ppl_bwd{8};
+static std::atomic<int> g_ppl_fwd{0}, g_ppl_bwd{0};  // 0: by the number of tiles
 static std::atomic<int> g_tile_sort{0}, g_tile_cull{1};
 static std::atomic<unsigned long long*> g_stats{nullptr};
 static int g_num_sms[64];

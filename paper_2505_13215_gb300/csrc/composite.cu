@@ -204,13 +204,13 @@ constexpr float kClampFree = 0.989f;
 // skipped for it there as here).  Every pair is blended in straight-line code,
 // a skipped pixel with alpha = 0 (no effect): few listed Gaussians reach no
 // pixel of the band, and a block of independent pairs keeps the pipes fed.
-// The saturation stop is rare and handled behind a vote.  No test result
+// The saturation stop is handled behind a vote.  No test result
 // is kept across the pairs (the skip test is one compare, redone where
 // needed), which keeps the predicate registers free.
 template <int NP, bool CLAMP, bool STATS>
 __device__ __forceinline__ bool fwd_gaussian(const Feat& f, const ColTerms& ct, float2 (&T)[NP],
-                                             float2 (&nC)[NP][3], float2 (&nrow)[NP], int (&last)[2 * NP],
-                                             unsigned& done, int pos, unsigned& n_eval, unsigned& n_blend)
+                                             float2 (&nC)[NP][3], float2 (&nrow)[NP], int (*last)[32],
+                                             unsigned& done, int pos, int lane, unsigned& n_eval, unsigned& n_blend)
 {
     float2 np2[NP];
 #pragma unroll
@@ -243,14 +243,14 @@ __device__ __forceinline__ bool fwd_gaussian(const Feat& f, const ColTerms& ct, 
                 nrow[p].x = -kOffRow;
                 nw[p].x = 0.f;
                 tT[p].x = T[p].x;
-                last[2 * p] = pos - 1;
+                last[2 * p][lane] = pos - 1;
             }
             if (tT[p].y < kTMin) {
                 done |= 2u << (2 * p);
                 nrow[p].y = -kOffRow;
                 nw[p].y = 0.f;
                 tT[p].y = T[p].y;
-                last[2 * p + 1] = pos - 1;
+                last[2 * p + 1][lane] = pos - 1;
             }
         }
         finished = __all_sync(0xffffffffu, done == (1u << (2 * NP)) - 1);
@@ -266,14 +266,19 @@ __device__ __forceinline__ bool fwd_gaussian(const Feat& f, const ColTerms& ct, 
     return finished;
 }
 
-// Resident one-warp CTAs per SM the forward is compiled for.  The register
-// file is split among the four schedulers, so occupancy moves in steps of four
-// warps: PPL = 8 at 24 (80 registers, 8 bytes spilled) measured 0.329 ->
-// 0.317 ms per 4-view step against 20 at 92 registers (28 at 72 registers:
-// 0.321, 32 at 64: 0.337); the smaller variants fit 32 in 64 registers.
+// Resident one-warp CTAs per SM the forward is compiled for, and the Gaussians
+// it takes as a group.  The register file is split among the four schedulers, so
+// occupancy moves in steps of four warps.  A group's alphas do not depend on T:
+// computing them together gives the scheduler independent work, and one stop
+// test on the last T serves them all, since T never grows.  Measured (us, 4 views
+// of 1352x1014 and 8 of the 500k arc, PPL = 8): one Gaussian at a time at 24
+// CTAs 351 and 542, groups of 2 at 24 (80 registers) 322 and 504, at 20 325 and
+// 510, at 28 343 and 548, groups of 3 335 and 544; PPL = 4 (one 1352x1014 view):
+// 105 one at a time, 92 in groups of 4 at 28 CTAs; PPL = 2 (128x128): 23 and 14.
 template <int PPL>
 struct FwdOccupancy {
-    static constexpr int kMinBlocks = PPL >= 8 ? 24 : 32;
+    static constexpr int kMinBlocks = PPL >= 8 ? 24 : (PPL == 4 ? 28 : 32);
+    static constexpr int kGroup = PPL >= 8 ? 2 : 4;
 };
 
 // STATS: also count, per warp, the pixel-Gaussian pairs evaluated (power
@@ -290,6 +295,9 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
     __shared__ float4 s_feat[kCompWarps][32][kFeat];
     __shared__ RawRows s_raw[kCompWarps];
     __shared__ float s_target[kCompWarps][3 * PPL][32];  // the fused loss's target at the lane's pixels
+    // end of each pixel's walk: the list length unless it saturates (touched only where a pixel does, so it
+    // need not hold registers)
+    __shared__ int s_last[kCompWarps][PPL][32];
     if (status_failed(status)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t unit = (int64_t)blockIdx.x * kCompWarps + warp;
@@ -310,23 +318,23 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
     // saturated).  nC: minus the accumulated colour.
     const uint2 rg = ranges[tile];
     float2 T[NP], nC[NP][3], nrow[NP];
-    int last[PPL];  // end of the walk: the list length unless the pixel saturates
+    int (*last)[32] = s_last[warp];
     unsigned done = 0;
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
         T[p] = make_float2(1.f, 1.f);
         nC[p][0] = nC[p][1] = nC[p][2] = make_float2(0.f, 0.f);
         nrow[p] = make_float2(-(float)(y0 + 4 * p), -(float)(y0 + 4 * p + 2));
-        last[2 * p] = last[2 * p + 1] = (int)(rg.y - rg.x);
+        last[2 * p][lane] = last[2 * p + 1][lane] = (int)(rg.y - rg.x);
         if (u >= vp.W || y0 + 4 * p >= vp.H) {
             done |= 1u << (2 * p);
             nrow[p].x = -kOffRow;
-            last[2 * p] = 0;
+            last[2 * p][lane] = 0;
         }
         if (u >= vp.W || y0 + 4 * p + 2 >= vp.H) {
             done |= 2u << (2 * p);
             nrow[p].y = -kOffRow;
-            last[2 * p + 1] = 0;
+            last[2 * p + 1][lane] = 0;
         }
     }
     const unsigned all_done = (1u << PPL) - 1;
@@ -367,16 +375,112 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
         const int pos0 = (int)(b - rg.x) + 1;
         // every lane walks the batch (finished pixels fail every test) so that
         // the votes inside see the whole warp
-        for (int j = 0; j < n; ++j) {
+        const bool clamp_batch = __any_sync(0xffffffffu, lane < n && sf[lane * kFeat + 2].w >= kClampFree);
+        auto one = [&](auto clamp_tag, int j) {  // true once every pixel of the warp is done
             Feat f;
             load_feat(sf + j * kFeat, f);
             const ColTerms ct = col_terms(f, nu);
-            const bool finished =
-                f.op < kClampFree  // same Gaussian on every lane
-                    ? fwd_gaussian<NP, false, STATS>(f, ct, T, nC, nrow, last, done, pos0 + j, n_eval, n_blend)
-                    : fwd_gaussian<NP, true, STATS>(f, ct, T, nC, nrow, last, done, pos0 + j, n_eval, n_blend);
-            if (finished) break;  // warp-uniform
-        }
+            return fwd_gaussian<NP, decltype(clamp_tag)::value, STATS>(f, ct, T, nC, nrow, last, done, pos0 + j, lane,
+                                                                       n_eval, n_blend);
+        };
+        auto walk = [&](auto clamp_tag) {
+            constexpr bool CL = decltype(clamp_tag)::value;
+            constexpr int GS = STATS ? 1 : FwdOccupancy<PPL>::kGroup;
+            int j = 0;
+            if constexpr (GS > 1) {
+                for (; j + GS <= n; j += GS) {
+                    float2 nw[GS][NP], t[NP];
+#pragma unroll
+                    for (int q = 0; q < GS; ++q) {  // -alpha of each: independent of T
+                        Feat f;
+                        load_feat(sf + (j + q) * kFeat, f);
+                        const ColTerms ct = col_terms(f, nu);
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) {
+                            const float2 np2 = pair_npower(f, ct, add2(f.py, nrow[p]));
+                            float2 a = pair_alpha(np2);
+                            if (CL) {
+                                a.x = fminf(a.x, kAlphaClamp);
+                                a.y = fminf(a.y, kAlphaClamp);
+                            }
+                            nw[q][p].x = __float_as_uint(np2.x) <= kLimBits ? -a.x : 0.f;
+                            nw[q][p].y = __float_as_uint(np2.y) <= kLimBits ? -a.y : 0.f;
+                        }
+                    }
+                    bool stop = false;
+#pragma unroll
+                    for (int p = 0; p < NP; ++p) {
+                        t[p] = T[p];
+#pragma unroll
+                        for (int q = 0; q < GS; ++q) {
+                            nw[q][p] = mul2(nw[q][p], t[p]);  // -alpha T
+                            t[p] = add2(t[p], nw[q][p]);
+                        }
+                        stop |= (t[p].x < kTMin) | (t[p].y < kTMin);
+                    }
+                    bool finished = false;
+                    if (__any_sync(0xffffffffu, stop)) {
+                        // a pixel saturates inside the group: T again along its chain, nothing blended from
+                        // the Gaussian that would take it below the limit on
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) {
+                            if (t[p].x < kTMin) {
+                                float tx = T[p].x;
+                                bool over = false;
+#pragma unroll
+                                for (int q = 0; q < GS; ++q) {
+                                    const float tq = tx + nw[q][p].x;
+                                    if (!over && tq < kTMin) {
+                                        over = true;
+                                        last[2 * p][lane] = pos0 + j + q - 1;
+                                    }
+                                    nw[q][p].x = over ? 0.f : nw[q][p].x;
+                                    tx = over ? tx : tq;
+                                }
+                                t[p].x = tx;
+                                done |= 1u << (2 * p);
+                                nrow[p].x = -kOffRow;
+                            }
+                            if (t[p].y < kTMin) {
+                                float ty = T[p].y;
+                                bool over = false;
+#pragma unroll
+                                for (int q = 0; q < GS; ++q) {
+                                    const float tq = ty + nw[q][p].y;
+                                    if (!over && tq < kTMin) {
+                                        over = true;
+                                        last[2 * p + 1][lane] = pos0 + j + q - 1;
+                                    }
+                                    nw[q][p].y = over ? 0.f : nw[q][p].y;
+                                    ty = over ? ty : tq;
+                                }
+                                t[p].y = ty;
+                                done |= 2u << (2 * p);
+                                nrow[p].y = -kOffRow;
+                            }
+                        }
+                        finished = __all_sync(0xffffffffu, done == all_done);
+                    }
+#pragma unroll
+                    for (int q = 0; q < GS; ++q) {
+                        const float4 f1 = sf[(j + q) * kFeat + 1], f2 = sf[(j + q) * kFeat + 2];
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) {
+                            nC[p][0] = fma2(make_float2(f1.x, f1.y), nw[q][p], nC[p][0]);
+                            nC[p][1] = fma2(make_float2(f1.z, f1.w), nw[q][p], nC[p][1]);
+                            nC[p][2] = fma2(make_float2(f2.x, f2.y), nw[q][p], nC[p][2]);
+                        }
+                    }
+#pragma unroll
+                    for (int p = 0; p < NP; ++p) T[p] = t[p];
+                    if (finished) return;  // warp-uniform
+                }
+            }
+            for (; j < n; ++j)
+                if (one(clamp_tag, j)) return;  // warp-uniform
+        };
+        if (clamp_batch) walk(std::integral_constant<bool, true>());
+        else walk(std::integral_constant<bool, false>());
         __syncwarp();
     }
     cp_async_wait_all();  // no copy may land in shared memory after the CTA has left
@@ -402,7 +506,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
 #pragma unroll
         for (int ch = 0; ch < 3; ++ch) rgb[ch * HW + p] = out[ch];
         img.final_T[vp.pix_base + p] = Tk;
-        img.last[vp.pix_base + p] = last[k];
+        img.last[vp.pix_base + p] = last[k][lane];
         if (l1.target) {  // same for every lane
             const int64_t q = 3 * vp.pix_base + p;
 #pragma unroll
@@ -437,8 +541,9 @@ constexpr int kRedBatch = 7;
 constexpr int kRedGroups = 16;
 // resident one-warp CTAs per SM the backward is compiled for: 16 leave
 // PPL = 8 its 128 registers (20, at 96 registers, spill in the loop and
-// measured slower: 0.615 -> 0.641 ms per 4-view step), 20 give the smaller
-// variants 96
+// measured slower: 0.615 -> 0.641 ms per 4-view step; with the walks' ends in shared
+// memory they fit in 96, but the reduction's shared memory then has to shrink to
+// groups of 5: 679 -> 702 us), 20 give the smaller variants 96
 template <int PPL>
 struct BwdOccupancy {
     static constexpr int kMinBlocks = PPL >= 8 ? 16 : 20;
@@ -453,7 +558,7 @@ __device__ __forceinline__ void flush_group(const float4* red, int nq, unsigned 
     __syncwarp();
     const int gi = lane >> 1, h = lane & 1;
     float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
-    if (gi < 2 * nq || gi == 14 || (gi == 15 && nq > 4)) {
+    if (gi < 2 * nq || gi == 2 * kRedBatch || (gi == 2 * kRedBatch + 1 && nq > 4)) {
         const float4* col = red + gi * 32 + 16 * h;
         const int x = lane & 7;
 #pragma unroll
@@ -468,7 +573,7 @@ __device__ __forceinline__ void flush_group(const float4* red, int nq, unsigned 
     s1.x += __shfl_xor_sync(0xffffffffu, s1.x, 1);
     s1.y += __shfl_xor_sync(0xffffffffu, s1.y, 1);
     const int q = h ? gi : gi >> 1;
-    const int bl = 28 + 2 * (q >> 2);
+    const int bl = 4 * kRedBatch + 2 * (q >> 2);
     const float b0 = __shfl_sync(0xffffffffu, s0.x, bl & 31), b1 = __shfl_sync(0xffffffffu, s0.y, bl & 31);
     const float b2 = __shfl_sync(0xffffffffu, s1.x, bl & 31), b3 = __shfl_sync(0xffffffffu, s1.y, bl & 31);
     if (q < nq && ((used >> q) & 1u)) {
@@ -500,6 +605,17 @@ __device__ __forceinline__ void flush_group(const float4* red, int nq, unsigned 
 struct BwdSums {
     float2 W0, W1, W2, r, g, b;
 };
+
+// The lane's sums of a Gaussian into its reduction slot q.
+__device__ __forceinline__ void store_sums(const BwdSums& S, float dx, float4* red, int q, int lane)
+{
+    const float W0 = S.W0.x + S.W0.y, W1 = S.W1.x + S.W1.y;
+    float4* slot = red + 2 * q * 32 + lane;
+    const float dxW0 = dx * W0;
+    slot[0] = make_float4(dxW0, W1, dx * dxW0, dx * W1);
+    slot[32] = make_float4(S.W2.x + S.W2.y, W0, S.r.x + S.r.y, S.g.x + S.g.y);
+    ((float*)(red + (2 * kRedBatch + (q >> 2)) * 32 + lane))[q & 3] = S.b.x + S.b.y;
+}
 
 // The backward's work for one staged Gaussian on all pixel pairs of the lane,
 // in straight-line code (a skipped pixel with alpha = 0, no effect).  Returns
@@ -576,6 +692,10 @@ __global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks
     __shared__ uint32_t s_row[kCompWarps][32];
     __shared__ float4 s_red[kCompWarps][kRedGroups][32];
     __shared__ RawRows s_raw[kCompWarps];
+    // ends of the pixels' walks, read only where one switches on: in shared memory for PPL = 8, whose registers
+    // bound it; the smaller variants' shared memory bounds how many of their CTAs fit
+    constexpr bool kLastShared = PPL >= 8;
+    __shared__ int s_last[kCompWarps][kLastShared ? PPL : 1][32];
     if (status_failed(status)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t unit = (int64_t)blockIdx.x * kCompWarps + warp;
@@ -618,7 +738,8 @@ __global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks
             q = -(g0 * vp.bg[0] + g1 * vp.bg[1] + g2 * vp.bg[2]);
             maxlast = max(maxlast, lk);
         }
-        last[k] = lk;
+        if (kLastShared) s_last[warp][kLastShared ? k : 0][lane] = lk;
+        else last[k] = lk;
         if (k & 1) {
             T[k >> 1].y = t; nQ[k >> 1].y = q; G[k >> 1][0].y = g0; G[k >> 1][1].y = g1; G[k >> 1][2].y = g2;
             nrow[k >> 1].y = -kOffRow;
@@ -671,48 +792,55 @@ __global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks
         const int n = (int)min(32u, end - b);
         // one vote per batch: does any staged Gaussian reach the 0.99 clamp
         const bool clamp_batch = __any_sync(0xffffffffu, lane < n && sf[lane * kFeat + 2].w >= kClampFree);
+        // pixels whose last contributor is at li or later switch on (warp-uniform)
+        auto switch_on = [&](int li) {
+            int nxt = -1;
+#pragma unroll
+            for (int k = 0; k < PPL; ++k) {
+                const float nr = -(y0f + (float)(2 * k));
+                const int lk = kLastShared ? s_last[warp][kLastShared ? k : 0][lane] : last[k];
+                if (li < lk) {
+                    if (k & 1) nrow[k >> 1].y = nr;
+                    else nrow[k >> 1].x = nr;
+                } else {
+                    nxt = max(nxt, lk - 1);
+                }
+            }
+            act = __reduce_max_sync(0xffffffffu, nxt);
+        };
+        // Gaussian j into reduction slot q; returns whether its sums are to be added
+        auto one = [&](auto clamp_tag, int j, int q) {
+            if (STATS) {
+#pragma unroll
+                for (int k = 0; k < PPL; ++k)
+                    n_eval += 32 * bi + j < (kLastShared ? s_last[warp][kLastShared ? k : 0][lane] : last[k]);
+            }
+            Feat f;
+            load_feat(sf + j * kFeat, f);
+            const ColTerms ct = col_terms(f, nu);
+            BwdSums S;
+            const bool any = bwd_gaussian<NP, decltype(clamp_tag)::value, STATS>(f, ct, T, nQ, G, nrow, S, n_blend);
+            store_sums(S, ct.dx, red, q, lane);
+            return any;
+        };
         auto walk = [&](auto clamp_tag) {
-            constexpr bool CL = decltype(clamp_tag)::value;
             // groups of kRedBatch consecutive Gaussians, back to front; Gaussian
             // j0 - q of a group sums into reduction slot q
             for (int j0 = n - 1; j0 >= 0; j0 -= kRedBatch) {
                 unsigned used = 0;
+                if (32 * bi + j0 <= act) switch_on(32 * bi + j0);
+                if (!STATS && j0 >= kRedBatch - 1 && act < 32 * bi + j0 - (kRedBatch - 1)) {
+                    // (nearly all) a whole group in which no pixel switches on: straight-line code
 #pragma unroll
-                for (int q = 0; q < kRedBatch; ++q) {
-                    const int j = j0 - q;
-                    if (j < 0) break;  // warp-uniform: the last group of a batch may be short
-                    const int li = 32 * bi + j;  // position in the tile list
-                    if (li <= act) {  // (warp-uniform) pixels whose last contributor is at li or later switch on
-                        int nxt = -1;
-#pragma unroll
-                        for (int k = 0; k < PPL; ++k) {
-                            const float nr = -(y0f + (float)(2 * k));
-                            const int lk = last[k];
-                            if (li < lk) {
-                                if (k & 1) nrow[k >> 1].y = nr;
-                                else nrow[k >> 1].x = nr;
-                            } else {
-                                nxt = max(nxt, lk - 1);
-                            }
-                        }
-                        act = __reduce_max_sync(0xffffffffu, nxt);
+                    for (int q = 0; q < kRedBatch; ++q) one(clamp_tag, j0 - q, q);
+                    used = (1u << kRedBatch) - 1u;
+                } else {
+#pragma unroll 1
+                    for (int q = 0; q < min(kRedBatch, j0 + 1); ++q) {
+                        const int li = 32 * bi + j0 - q;  // position in the tile list
+                        if (li <= act) switch_on(li);
+                        used |= (unsigned)one(clamp_tag, j0 - q, q) << q;
                     }
-                    if (STATS) {
-#pragma unroll
-                        for (int k = 0; k < PPL; ++k) n_eval += li < last[k];
-                    }
-                    Feat f;
-                    load_feat(sf + j * kFeat, f);
-                    const ColTerms ct = col_terms(f, nu);
-                    BwdSums S;
-                    const bool any = bwd_gaussian<NP, CL, STATS>(f, ct, T, nQ, G, nrow, S, n_blend);
-                    used |= (unsigned)any << q;
-                    const float W0 = S.W0.x + S.W0.y, W1 = S.W1.x + S.W1.y;
-                    float4* slot = red + 2 * q * 32 + lane;
-                    const float dx = ct.dx, dxW0 = dx * W0;
-                    slot[0] = make_float4(dxW0, W1, dx * dxW0, dx * W1);
-                    slot[32] = make_float4(S.W2.x + S.W2.y, W0, S.r.x + S.r.y, S.g.x + S.g.y);
-                    ((float*)(red + (14 + (q >> 2)) * 32 + lane))[q & 3] = S.b.x + S.b.y;
                 }
                 if (used) flush_group(red, min(kRedBatch, j0 + 1), used, j0, sf, s_row[warp], dproj, lane);
             }
@@ -801,10 +929,28 @@ static void bwd_launch(int ppl, int blocks, cudaStream_t st, const splat_proj& p
     }
 }
 
+// Pixels per lane where the caller leaves them open (0): as many as keep the
+// chip full.  Eight share the per-Gaussian work best, but a batch with few tiles
+// leaves warp slots empty and is as slow as its longest walk, which fewer pixels
+// per lane make shorter.  Forward + backward us at 8 / 4 / 2 pixels per lane:
+//   64 tiles (128x128):     fwd 27 / 19 / 14    bwd 49 / 44 / 38
+//   300 tiles:              fwd 42 / 27 / 21    bwd 80 / 66 / 63
+//   600 tiles:              fwd 42 / 30 / 27    bwd 80 / 72 / 74
+//   1376 tiles (677x507):   fwd 55 / 39 / 37    bwd 98 / 91 / 96
+//   2451 tiles:             fwd 71 / 51 / 55    bwd 125 / 123 / 146
+//   5440 tiles (1352x1014): fwd 100 / 86 / 120  bwd 196 / 211 / 339
+//   10880 tiles:            fwd 163 / 166 / 238 bwd 356 / 420 / 683
+static int auto_ppl(int ppl, int tiles, int num_sms, int two, int four)
+{
+    if (ppl) return ppl;
+    return tiles <= two * num_sms ? 2 : (tiles <= four * num_sms ? 4 : 8);
+}
+
 cudaError_t launch_composite_fwd(const splat_proj& proj, const splat_bins& bins, const ViewBatch& vb,
                                  const splat_image& img, const L1Fuse* l1p, int32_t* status, int ppl,
                                  unsigned long long* stats, const LaunchCtx& ctx)
 {
+    ppl = auto_ppl(ppl, vb.total_tiles, ctx.num_sms, 4, 40);
     const L1Fuse l1 = l1p ? *l1p : L1Fuse{nullptr, 0.f, nullptr, nullptr};
     if (l1.loss) {
         const cudaError_t e = cudaMemsetAsync(l1.loss, 0, sizeof(float), ctx.stream);
@@ -825,6 +971,7 @@ cudaError_t launch_composite_bwd(const splat_proj& proj, const splat_bins& bins,
                                  unsigned long long* stats, const LaunchCtx& ctx)
 {
     if (vb.total_tiles == 0) return cudaSuccess;
+    ppl = auto_ppl(ppl, vb.total_tiles, ctx.num_sms, 2, 10);
     const int bands = 8 / ppl;
     const int64_t units = (int64_t)vb.total_tiles * bands;
     const int blocks = (int)((units + kCompWarps - 1) / kCompWarps);

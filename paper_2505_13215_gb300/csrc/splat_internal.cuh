@@ -296,7 +296,7 @@ struct LaunchCtx {
     int64_t spin_limit;
     int tile_sort;   // 0 automatic, 1 radix passes, 2 binned partition
     int tile_cull;   // binned path: footprint culling and the saturation cut
-    int ppl_fwd, ppl_bwd;
+    int ppl_fwd, ppl_bwd;  // 0: by the number of tiles
     unsigned long long* stats;
 };
 LaunchCtx launch_ctx(void* stream, const splat_options* opt = nullptr);

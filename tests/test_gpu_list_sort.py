@@ -67,7 +67,7 @@ def _check(views, n, rects, z, visible, cap=None):
     assert (rg[~some] == 0).all()
 
 
-@pytest.mark.parametrize("n", [1, 31, 32, 33, 511, 512, 513, 545, 1536, 1537, 2047, 2048, 2049, 5000])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 511, 512, 513, 545, 1536, 1537, 2047, 2048, 2049, 4096, 4097, 5000])
 def test_one_super_tile(n):
     rng = np.random.default_rng(n)
     views = [scenes.identity_view(128, 128, 128.0, 0.5)]
