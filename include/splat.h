@@ -520,6 +520,17 @@ splat_status splat_composite_fwd_l1_opts(const splat_proj *proj, const splat_bin
                                          int V, splat_image *img, const float *target, float scale, float *dL_drgb,
                                          float *loss, int32_t *status, const splat_options *opt, void *stream);
 
+/*
+ * splat_composite_fwd_l1_opts with scratch for the loss: workspace (device,
+ * 4-byte aligned; any splat_workspace_size() buffer that no running call uses)
+ * holds partial sums, so that the float sum of a large batch keeps FP32
+ * accuracy.  NULL or fewer than 4096 bytes: one running sum, as there.
+ */
+splat_status splat_composite_fwd_l1_ws(const splat_proj *proj, const splat_bins *bins, const splat_view *views, int V,
+                                       splat_image *img, const float *target, float scale, float *dL_drgb,
+                                       float *loss, int32_t *status, void *workspace, size_t workspace_bytes,
+                                       const splat_options *opt, void *stream);
+
 /* splat_composite_bwd with per-call options (pixels_per_lane_bwd, stats). */
 splat_status splat_composite_bwd_opts(const splat_proj *proj, const splat_bins *bins, const splat_view *views, int V,
                                       const splat_image *img, const float *dL_drgb, const splat_g3 *g3,

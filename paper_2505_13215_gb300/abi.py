@@ -155,6 +155,9 @@ EXPORTS = {
     "splat_composite_fwd_l1_opts": (C.c_int, [_P(splat_proj), _P(splat_bins), _P(splat_view), C.c_int,
                                               _P(splat_image), C.c_void_p, C.c_float, C.c_void_p, C.c_void_p,
                                               C.c_void_p, _P(splat_options), C.c_void_p]),
+    "splat_composite_fwd_l1_ws": (C.c_int, [_P(splat_proj), _P(splat_bins), _P(splat_view), C.c_int,
+                                            _P(splat_image), C.c_void_p, C.c_float, C.c_void_p, C.c_void_p,
+                                            C.c_void_p, C.c_void_p, C.c_size_t, _P(splat_options), C.c_void_p]),
     "splat_composite_bwd_opts": (C.c_int, [_P(splat_proj), _P(splat_bins), _P(splat_view), C.c_int, _P(splat_image),
                                            C.c_void_p, _P(splat_g3), _P(splat_g4), _P(splat_grads3),
                                            _P(splat_grads4), C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p,
@@ -331,6 +334,11 @@ def splat_composite_fwd_opts(proj, bins, views, V, img, status, opt, stream):
 
 def splat_composite_fwd_l1_opts(proj, bins, views, V, img, target, scale, dL, loss, status, opt, stream):
     return lib().splat_composite_fwd_l1_opts(proj, bins, views, V, img, target, scale, dL, loss, status, opt, stream)
+
+
+def splat_composite_fwd_l1_ws(proj, bins, views, V, img, target, scale, dL, loss, status, ws, ws_bytes, opt, stream):
+    return lib().splat_composite_fwd_l1_ws(proj, bins, views, V, img, target, scale, dL, loss, status, ws, ws_bytes,
+                                           opt, stream)
 
 
 def splat_composite_bwd_opts(proj, bins, views, V, img, dL, g3, g4, dg3, dg4, dproj, flags, status, ws, ws_bytes, opt,

@@ -380,6 +380,15 @@ splat_status splat_composite_fwd_l1_opts(const splat_proj* proj, const splat_bin
                                          int V, splat_image* img, const float* target, float scale, float* dL_drgb,
                                          float* loss, int32_t* status, const splat_options* opt, void* stream)
 {
+    return splat_composite_fwd_l1_ws(proj, bins, views, V, img, target, scale, dL_drgb, loss, status, nullptr, 0, opt,
+                                     stream);
+}
+
+splat_status splat_composite_fwd_l1_ws(const splat_proj* proj, const splat_bins* bins, const splat_view* views, int V,
+                                       splat_image* img, const float* target, float scale, float* dL_drgb, float* loss,
+                                       int32_t* status, void* workspace, size_t workspace_bytes,
+                                       const splat_options* opt, void* stream)
+{
     if (!valid_views(views, V) || !valid_proj(proj, V) || !bins || !img || !status || !valid_options(opt))
         return SPLAT_ERR_INVALID_ARG;
     if (!img->rgb || !img->final_T || !img->last || !bins->ranges || (bins->capacity > 0 && !bins->vals))
@@ -387,7 +396,10 @@ splat_status splat_composite_fwd_l1_opts(const splat_proj* proj, const splat_bin
     if (!target || !dL_drgb || !loss || !std::isfinite(scale)) return SPLAT_ERR_INVALID_ARG;
     const LaunchCtx ctx = launch_ctx(stream, opt);
     const ViewBatch vb = make_batch(views, V);
-    const L1Fuse l1{target, scale, dL_drgb, loss};
+    float* partial = workspace && workspace_bytes >= kLossParts * sizeof(float) && aligned(workspace, 4)
+                         ? (float*)workspace
+                         : nullptr;
+    const L1Fuse l1{target, scale, dL_drgb, loss, partial};
     return cuda_status(launch_composite_fwd(*proj, *bins, vb, *img, &l1, status, ctx.ppl_fwd, ctx.stats, ctx));
 }
 

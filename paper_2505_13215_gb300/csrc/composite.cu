@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
     if (l1.target) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) l1sum += __shfl_xor_sync(0xffffffffu, l1sum, o);
-        if (lane == 0) atomicAdd(l1.loss, l1sum);
+        if (lane == 0) atomicAdd(l1.partial ? l1.partial + (unit & (kLossParts - 1)) : l1.loss, l1sum);
     }
 }
 
@@ -903,6 +903,24 @@ cudaError_t launch_l1_loss(const float* img, const float* target, int64_t n, flo
     return cudaGetLastError();
 }
 
+// *loss = the sum of the kLossParts partial sums
+__global__ void __launch_bounds__(256) k_loss_sum(const float* __restrict__ partial, float* loss)
+{
+    float acc = 0.f;
+#pragma unroll
+    for (int i = 0; i < kLossParts / 256; ++i) acc += partial[threadIdx.x + 256 * i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    __shared__ float s_acc[8];
+    if ((threadIdx.x & 31) == 0) s_acc[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.f;
+        for (int w = 0; w < 8; ++w) t += s_acc[w];
+        *loss = t;
+    }
+}
+
 template <bool ST>
 static void fwd_launch(int ppl, int blocks, cudaStream_t st, const splat_proj& proj, const splat_bins& bins,
                        const ViewBatch& vb, const splat_image& img, const L1Fuse& l1, int32_t* status,
@@ -951,18 +969,24 @@ cudaError_t launch_composite_fwd(const splat_proj& proj, const splat_bins& bins,
                                  unsigned long long* stats, const LaunchCtx& ctx)
 {
     ppl = auto_ppl(ppl, vb.total_tiles, ctx.num_sms, 4, 40);
-    const L1Fuse l1 = l1p ? *l1p : L1Fuse{nullptr, 0.f, nullptr, nullptr};
+    L1Fuse l1 = l1p ? *l1p : L1Fuse{nullptr, 0.f, nullptr, nullptr, nullptr};
+    const int bands = 8 / ppl;
+    const int64_t units = (int64_t)vb.total_tiles * bands;
+    if (units <= 512) l1.partial = nullptr;  // few shares: within 5e-7, and one launch less
     if (l1.loss) {
-        const cudaError_t e = cudaMemsetAsync(l1.loss, 0, sizeof(float), ctx.stream);
+        const cudaError_t e = l1.partial ? cudaMemsetAsync(l1.partial, 0, kLossParts * sizeof(float), ctx.stream)
+                                         : cudaMemsetAsync(l1.loss, 0, sizeof(float), ctx.stream);
         if (e != cudaSuccess) return e;
     }
     if (vb.total_tiles == 0) return cudaSuccess;
-    const int bands = 8 / ppl;
-    const int64_t units = (int64_t)vb.total_tiles * bands;
     const int blocks = (int)((units + kCompWarps - 1) / kCompWarps);
     count_launch();
     if (stats) fwd_launch<true>(ppl, blocks, ctx.stream, proj, bins, vb, img, l1, status, stats);
     else fwd_launch<false>(ppl, blocks, ctx.stream, proj, bins, vb, img, l1, status, nullptr);
+    if (l1.partial) {
+        count_launch();
+        k_loss_sum<<<1, 256, 0, ctx.stream>>>(l1.partial, l1.loss);
+    }
     return cudaGetLastError();
 }
 

@@ -279,13 +279,18 @@ extern std::atomic<int64_t> g_launches;  // kernels launched or captured (diagno
 inline void count_launch(int n = 1) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 // L1 loss fused into the forward compositing (all null when not fused):
 // *loss += sum |rgb - target|, dL = scale * sign(rgb - target), per pixel as
-// its colour is written.
+// its colour is written.  With partial (kLossParts floats) a warp adds its share
+// to one of them and they are summed at the end: FP32 additions of tens of
+// thousands of shares to one number lose 2e-8 sqrt(shares) of it (3e-6 for 4
+// views of 1352x1014), more than the kernels' other errors.
 struct L1Fuse {
     const float* target;
     float scale;
     float* dL;
     float* loss;
+    float* partial;
 };
+constexpr int kLossParts = 1024;
 
 // Per-call launch context: the stream, the device's SM count and the tuning
 // of this call (the library-wide splat_set_* settings, or a caller's

@@ -297,10 +297,10 @@ class Rasterizer:
         """Composite all views with the L1 loss fused in (the same image, loss and
         pixel gradient as composite() followed by l1_loss(); asynchronous)."""
         n = self.rgb.numel()
-        abi.check(abi.splat_composite_fwd_l1_opts(C.byref(self.cproj), C.byref(self.cbins), self.cviews, self.V,
-                                                  C.byref(self.cimg), _ptr(target), 1.0 / max(1, n), _ptr(self.dL),
-                                                  _ptr(self.loss), _ptr(self.status), C.byref(self.options),
-                                                  _stream(stream)), "splat_composite_fwd_l1")
+        abi.check(abi.splat_composite_fwd_l1_ws(C.byref(self.cproj), C.byref(self.cbins), self.cviews, self.V,
+                                                C.byref(self.cimg), _ptr(target), 1.0 / max(1, n), _ptr(self.dL),
+                                                _ptr(self.loss), _ptr(self.status), _ptr(self.ws), self.ws_bytes,
+                                                C.byref(self.options), _stream(stream)), "splat_composite_fwd_l1")
         return self.loss
 
     STAGES = ("slice_project", "bin_sort", "composite_fwd", "loss", "composite_bwd", "adjoint")
