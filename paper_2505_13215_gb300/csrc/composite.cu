@@ -129,6 +129,53 @@ __device__ __forceinline__ void stage_feat(const RawRows& raw, int lane, float4*
     s[3] = make_float4(na2, nb2, ml, 0.f);
 }
 
+// Whether the lane's gathered Gaussian can reach rows [y, y + rows - 1] of a unit
+// with columns [x, x + 15]: the rows its footprint spans inside the columns.  The
+// squared radius is enlarged for the rounding of the kernels' power: 1e-4 of
+// itself and 2e-3 as for the lists, and 2e-6 ac / (ac - b^2) of itself for the
+// cancellation of its terms on nearly singular conics (their absolute sum is at
+// most about 4 ac / (ac - b^2) times the power on the footprint), so that every
+// pixel of a unit left out fails the alpha test.  Bands skip a quarter of the
+// entries of scenes whose footprints are small against a tile and few of scenes
+// with large ones.  us without -> with: 128x128 (PPL = 2) backward 38 -> 32,
+// 677x507 (PPL = 4) forward 59 -> 55, backward 135 -> 122, but one 1352x1014
+// view of the wide-footprint scene (PPL = 4) forward 94 -> 97.  Inside a unit
+// the same test per half, with a branch around its pairs, cost far more than it
+// skipped (PPL = 8 backward 673 -> 868 on 4 views of 1352x1014): the branches
+// part the straight-line code that keeps the pipes fed.
+__device__ __forceinline__ bool reaches_unit(const RawRows& raw, int lane, float x, float y, int rows)
+{
+    const float2 xy = raw.xy[lane];
+    const float4 co = raw.co[lane];
+    const float ac = co.x * co.z;
+    const float R2 = -2.f * __logf(__fdividef(kAlphaMin, co.w)) *
+                         (1.0001f + 2e-6f * __fdividef(ac, ac - co.y * co.y)) + 2e-3f;
+    // rows and columns exchanged: the extent along y inside a band of x
+    float4 g0, g1;
+    ellipse_consts(xy.y, xy.x, co.z, co.y, co.x, R2, g0, g1);
+    float lo, hi;
+    return ellipse_band_extent(g0, g1, x, x + (float)(kTile - 1), lo, hi) && !(hi < y) &&
+           !(lo > y + (float)(rows - 1));
+}
+
+// The staged Gaussians of a batch in walking order, front to back (Forward) or
+// back to front.  A unit that is a band of a tile (PPL < 8) walks only those that
+// reach the band (a bit mask), a whole tile all n: its list holds no others.
+template <bool BANDS, bool FORWARD>
+struct Batch {
+    uint32_t bits;  // BANDS: those still to walk
+    int at, n;
+    __device__ __forceinline__ Batch(uint32_t reach, int n_) : bits(reach), at(FORWARD ? 0 : n_ - 1), n(n_) {}
+    __device__ __forceinline__ int left() const { return BANDS ? __popc(bits) : (FORWARD ? n - at : at + 1); }
+    __device__ __forceinline__ int next()
+    {
+        if (!BANDS) return FORWARD ? at++ : at--;
+        const int j = FORWARD ? __ffs(bits) - 1 : 31 - __clz(bits);
+        bits &= ~(1u << (j & 31));
+        return j;
+    }
+};
+
 __device__ __forceinline__ int find_view(const ViewBatch& vb, int tile)
 {
     int v = 0;
@@ -310,7 +357,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
     const int local = tile - vp.tile_base;
     const int ty = local / vp.TX, tx = local - ty * vp.TX;
     const int u = tx * kTile + (lane & 15);
-    const int y0 = ty * kTile + band * (2 * PPL) + (lane >> 4);
+    const int ybase = ty * kTile + band * (2 * PPL), y0 = ybase + (lane >> 4);
     const float2 nu = make_float2(-(float)u, -(float)u);
     const int64_t HW = (int64_t)vp.W * vp.H;
     // pair p holds pixels k = 2p, 2p + 1 (rows y0 + 4p, y0 + 4p + 2).  nrow:
@@ -365,7 +412,11 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
         const uint32_t idx = b + lane;
         if (b == rg.x) cp_async_wait_one();  // batch 0's rows (the target may still be in flight)
         else cp_async_wait_all();
+        uint32_t reach = 0xffffffffu;  // bit j: Gaussian j of the batch reaches the unit
         if (idx < rg.y) stage_feat(raw, lane, sf + lane * kFeat);
+        if (BANDS > 1)
+            reach = __ballot_sync(0xffffffffu, idx < rg.y && (STATS || reaches_unit(raw, lane, (float)(tx * kTile),
+                                                                                    (float)ybase, 2 * PPL)));
         __syncwarp();
         // the next batch's rows land while this one is composited
         if (idx + 32 < rg.y) gather_rows(proj, next_row, raw, lane);
@@ -384,16 +435,19 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
                                                                        n_eval, n_blend);
         };
         auto walk = [&](auto clamp_tag) {
-            constexpr bool CL = decltype(clamp_tag)::value;
+            [[maybe_unused]] constexpr bool CL = decltype(clamp_tag)::value;
             constexpr int GS = STATS ? 1 : FwdOccupancy<PPL>::kGroup;
-            int j = 0;
+            Batch<(BANDS > 1), true> batch(reach, n);
             if constexpr (GS > 1) {
-                for (; j + GS <= n; j += GS) {
+                while (batch.left() >= GS) {
+                    int jq[GS];
+#pragma unroll
+                    for (int q = 0; q < GS; ++q) jq[q] = batch.next();
                     float2 nw[GS][NP], t[NP];
 #pragma unroll
                     for (int q = 0; q < GS; ++q) {  // -alpha of each: independent of T
                         Feat f;
-                        load_feat(sf + (j + q) * kFeat, f);
+                        load_feat(sf + jq[q] * kFeat, f);
                         const ColTerms ct = col_terms(f, nu);
 #pragma unroll
                         for (int p = 0; p < NP; ++p) {
@@ -432,7 +486,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
                                     const float tq = tx + nw[q][p].x;
                                     if (!over && tq < kTMin) {
                                         over = true;
-                                        last[2 * p][lane] = pos0 + j + q - 1;
+                                        last[2 * p][lane] = pos0 + jq[q] - 1;
                                     }
                                     nw[q][p].x = over ? 0.f : nw[q][p].x;
                                     tx = over ? tx : tq;
@@ -449,7 +503,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
                                     const float tq = ty + nw[q][p].y;
                                     if (!over && tq < kTMin) {
                                         over = true;
-                                        last[2 * p + 1][lane] = pos0 + j + q - 1;
+                                        last[2 * p + 1][lane] = pos0 + jq[q] - 1;
                                     }
                                     nw[q][p].y = over ? 0.f : nw[q][p].y;
                                     ty = over ? ty : tq;
@@ -463,7 +517,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
                     }
 #pragma unroll
                     for (int q = 0; q < GS; ++q) {
-                        const float4 f1 = sf[(j + q) * kFeat + 1], f2 = sf[(j + q) * kFeat + 2];
+                        const float4 f1 = sf[jq[q] * kFeat + 1], f2 = sf[jq[q] * kFeat + 2];
 #pragma unroll
                         for (int p = 0; p < NP; ++p) {
                             nC[p][0] = fma2(make_float2(f1.x, f1.y), nw[q][p], nC[p][0]);
@@ -476,8 +530,8 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
                     if (finished) return;  // warp-uniform
                 }
             }
-            for (; j < n; ++j)
-                if (one(clamp_tag, j)) return;  // warp-uniform
+            while (batch.left() > 0)
+                if (one(clamp_tag, batch.next())) return;  // warp-uniform
         };
         if (clamp_batch) walk(std::integral_constant<bool, true>());
         else walk(std::integral_constant<bool, false>());
@@ -549,10 +603,10 @@ struct BwdOccupancy {
     static constexpr int kMinBlocks = PPL >= 8 ? 16 : 20;
 };
 
-// Reduction of a group of consecutive staged Gaussians j0, j0 - 1, ..,
-// j0 - nq + 1 held in slots 0 .. nq - 1; slot q is added to dproj when bit q of
-// `used` is set.
-__device__ __forceinline__ void flush_group(const float4* red, int nq, unsigned used, int j0, const float4* sf,
+// Reduction of a group of staged Gaussians, the next nq of `group`, held in slots
+// 0 .. nq - 1; slot q is added to dproj when bit q of `used` is set.
+template <typename B>
+__device__ __forceinline__ void flush_group(const float4* red, int nq, unsigned used, B group, const float4* sf,
                                             const uint32_t* srow, float* dproj, int lane)
 {
     __syncwarp();
@@ -577,7 +631,8 @@ __device__ __forceinline__ void flush_group(const float4* red, int nq, unsigned 
     const float b0 = __shfl_sync(0xffffffffu, s0.x, bl & 31), b1 = __shfl_sync(0xffffffffu, s0.y, bl & 31);
     const float b2 = __shfl_sync(0xffffffffu, s1.x, bl & 31), b3 = __shfl_sync(0xffffffffu, s1.y, bl & 31);
     if (q < nq && ((used >> q) & 1u)) {
-        const int jv = j0 - q;
+        int jv = group.next();
+        for (int k = 0; k < q; ++k) jv = group.next();
         const uint32_t row = srow[jv];
         if (h == 0) {
             const float4 f3 = sf[jv * kFeat + 3];
@@ -708,7 +763,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks
     const int local = tile - vp.tile_base;
     const int ty = local / vp.TX, tx = local - ty * vp.TX;
     const int u = tx * kTile + (lane & 15);
-    const int y0 = ty * kTile + band * (2 * PPL) + (lane >> 4);
+    const int ybase = ty * kTile + band * (2 * PPL), y0 = ybase + (lane >> 4);
     const float2 nu = make_float2(-(float)u, -(float)u);
     const int64_t HW = (int64_t)vp.W * vp.H;
     // Per pixel: T = T_{j+1} (replayed transmittance behind the current Gaussian j),
@@ -779,10 +834,14 @@ __global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks
         const uint32_t b = rg.x + 32u * bi;
         const uint32_t idx = b + lane;
         cp_async_wait_all();
+        uint32_t reach = 0xffffffffu;  // bit j: Gaussian j of the batch reaches the unit
         if (idx < end) {
             s_row[warp][lane] = cur_row;
             stage_feat(raw, lane, sf + lane * kFeat);
         }
+        if (BANDS > 1)
+            reach = __ballot_sync(0xffffffffu, idx < end && (STATS || reaches_unit(raw, lane, (float)(tx * kTile),
+                                                                                   (float)ybase, 2 * PPL)));
         __syncwarp();
         // the previous batch's rows land while this one is walked
         if (bi >= 1) gather_rows(proj, next_row, raw, lane);
@@ -824,25 +883,32 @@ __global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks
             return any;
         };
         auto walk = [&](auto clamp_tag) {
-            // groups of kRedBatch consecutive Gaussians, back to front; Gaussian
-            // j0 - q of a group sums into reduction slot q
-            for (int j0 = n - 1; j0 >= 0; j0 -= kRedBatch) {
-                unsigned used = 0;
-                if (32 * bi + j0 <= act) switch_on(32 * bi + j0);
-                if (!STATS && j0 >= kRedBatch - 1 && act < 32 * bi + j0 - (kRedBatch - 1)) {
-                    // (nearly all) a whole group in which no pixel switches on: straight-line code
+            // groups of kRedBatch Gaussians, back to front, the q-th of a group
+            // summed into reduction slot q
+            Batch<(BANDS > 1), false> batch(reach, n);
+            while (batch.left() > 0) {
+                const Batch<(BANDS > 1), false> group = batch;
+                const int cnt = min(kRedBatch, batch.left());
+                int jq[kRedBatch];
 #pragma unroll
-                    for (int q = 0; q < kRedBatch; ++q) one(clamp_tag, j0 - q, q);
+                for (int q = 0; q < kRedBatch; ++q) jq[q] = batch.next();  // (negative from cnt on)
+                unsigned used = 0;
+                if (32 * bi + jq[0] <= act) switch_on(32 * bi + jq[0]);
+                if (!STATS && cnt == kRedBatch && act < 32 * bi + jq[kRedBatch - 1]) {
+                    // a whole group in which no pixel switches on: straight-line code
+#pragma unroll
+                    for (int q = 0; q < kRedBatch; ++q) one(clamp_tag, jq[q], q);
                     used = (1u << kRedBatch) - 1u;
                 } else {
+                    Batch<(BANDS > 1), false> b = group;
 #pragma unroll 1
-                    for (int q = 0; q < min(kRedBatch, j0 + 1); ++q) {
-                        const int li = 32 * bi + j0 - q;  // position in the tile list
+                    for (int q = 0; q < cnt; ++q) {
+                        const int j = b.next(), li = 32 * bi + j;  // li: position in the tile list
                         if (li <= act) switch_on(li);
-                        used |= (unsigned)one(clamp_tag, j0 - q, q) << q;
+                        used |= (unsigned)one(clamp_tag, j, q) << q;
                     }
                 }
-                if (used) flush_group(red, min(kRedBatch, j0 + 1), used, j0, sf, s_row[warp], dproj, lane);
+                if (used) flush_group(red, cnt, used, group, sf, s_row[warp], dproj, lane);
             }
         };
         if (clamp_batch) walk(std::integral_constant<bool, true>());

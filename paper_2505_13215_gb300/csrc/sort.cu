@@ -1609,74 +1609,6 @@ __global__ void __launch_bounds__(256) k_tile_ranges(TileArgs a, TileRangeArgs r
     }
 }
 
-// Opacity footprint of one projected Gaussian: the ellipse {power >= pcut},
-// power = -(a dx^2 + 2 b dx dy + c dy^2) / 2 with dx = px - u, dy = py - v,
-// i.e. q(dx, dy) <= R2 = -2 pcut (R2 enlarged by the caller).  Constants per
-// Gaussian, computed once: g0 = (px, py, R2, Y) with Y the |dy| reach,
-// g1 = (X, yr, b/a, det/a) with X the |dx| reach and yr the dy of the rightmost
-// point, g2.x = 1/a.  Degenerate conics keep the whole band (Y = inf).
-// Square root by the PTX approximation (a few ulp): the footprint's squared
-// radius carries a margin of 1e-4 of itself, far above that error.
-__device__ __forceinline__ float sqrt_approx(float x)
-{
-    float y;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ void ellipse_consts(float px, float py, float a, float b, float c, float R2, float4& g0,
-                                               float4& g1)
-{
-    const float det = a * c - b * b;
-    if (!(det > 0.f) || !(a > 0.f) || !(c > 0.f)) {
-        g0 = make_float4(px, py, 0.f, __int_as_float(0x7f800000));
-        g1 = make_float4(0.f, 0.f, 0.f, 0.f);
-        return;
-    }
-    // approximate quotients and roots (relative errors of a few 1e-7, inside
-    // the squared radius' 1e-4 margin)
-    const float ia = __fdividef(1.f, a), idet = __fdividef(1.f, det);
-    const float X = sqrt_approx(R2 * c * idet);
-    // g0 = (centre, R2 / a, reach in y); g1 = (reach in x, dy of the rightmost
-    // point, b / a, det / a^2)
-    g0 = make_float4(px, py, R2 * ia, sqrt_approx(R2 * a * idet));
-    g1 = make_float4(X, -__fdividef(b, c) * X, b * ia, det * ia * ia);
-}
-
-// Horizontal pixel extent [ul, ur] of the footprint inside the pixel band
-// v in [vlo, vhi]; false when the footprint misses the band.  At offset dy the
-// footprint spans dx = -(b/a) dy +- sqrt(R2/a - (det/a^2) dy^2).
-__device__ __forceinline__ bool ellipse_band_extent(const float4& g0, const float4& g1, float vlo, float vhi,
-                                                    float& ul, float& ur)
-{
-    const float px = g0.x, py = g0.y, Ra = g0.z, Y = g0.w;
-    if (isinf(Y)) {
-        ul = -3.0e38f;
-        ur = 3.0e38f;
-        return true;
-    }
-    const float e0 = fmaxf(py - vhi, -Y), e1 = fminf(py - vlo, Y);  // dy range of the band inside the reach
-    if (e0 > e1) return false;
-    const float X = g1.x, yr = g1.y, ba = g1.z, hq = g1.w;
-    float dxmax, dxmin;
-    if (yr >= e0 && yr <= e1) {
-        dxmax = X;
-    } else {
-        const float dy = fminf(fmaxf(yr, e0), e1);
-        dxmax = -ba * dy + sqrt_approx(fmaxf(0.f, Ra - hq * dy * dy));
-    }
-    const float yl = -yr;  // leftmost point
-    if (yl >= e0 && yl <= e1) {
-        dxmin = -X;
-    } else {
-        const float dy = fminf(fmaxf(yl, e0), e1);
-        dxmin = -ba * dy - sqrt_approx(fmaxf(0.f, Ra - hq * dy * dy));
-    }
-    ul = px - dxmax;
-    ur = px - dxmin;
-    return true;
-}
-
 // Tile columns [lo, hi) of the super-tile's tile row with pixel rows
 // [vlo, vlo + 15] that an entry is listed in, as bits: its rectangle's columns
 // [x0, x1), with culling on narrowed to the tiles its opacity footprint reaches.

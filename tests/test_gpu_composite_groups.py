@@ -14,12 +14,12 @@ from paper_2505_13215_gb300 import raster, scenes
 pytestmark = pytest.mark.gpu
 
 
-def _stack(n, logit, seed, W=37, H=21, spread=0.0):
-    """n wide Gaussians behind one another in front of a small image."""
+def _stack(n, logit, seed, W=37, H=21, spread=0.0, scales=(-1.5, 0.5)):
+    """n Gaussians (wide ones by default) behind one another in front of a small image."""
     rng = np.random.default_rng(seed)
     means = np.stack([rng.uniform(-spread, spread, n), rng.uniform(-spread, spread, n), 2.0 + 0.01 * np.arange(n)], 1)
     s = scenes.random_scene(rng, n, 0, means, np.zeros((0, 3)))
-    s.log_scale3[:] = rng.uniform(-1.5, 0.5, (n, 3)).astype(np.float32)
+    s.log_scale3[:] = rng.uniform(*scales, (n, 3)).astype(np.float32)
     s.opacity3[:] = np.asarray(logit, np.float32)
     return s, [scenes.identity_view(W, H, 40.0, 0.5)]
 
@@ -27,7 +27,16 @@ def _stack(n, logit, seed, W=37, H=21, spread=0.0):
 @pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 7, 31, 33, 66])
 @pytest.mark.parametrize("logit", [-2.0, 0.5, 3.0, 9.0])
 def test_groups_agree_with_single_steps(n, logit):
-    scene, views = _stack(n, logit, 100 * n + int(10 * logit), spread=0.2)
+    _agree(*_stack(n, logit, 100 * n + int(10 * logit), spread=0.2))
+
+
+@pytest.mark.parametrize("scales", [(-5.0, -3.5), (-3.5, -2.5), (-6.0, 0.5)])
+def test_bands_leave_out_only_what_they_do_not_reach(scales):
+    """Footprints smaller than a band of a tile, about a tile, and needles across it (nearly singular conics)."""
+    _agree(*_stack(700, 2.0, 5, W=61, H=67, spread=1.2, scales=scales))
+
+
+def _agree(scene, views):
     G = raster.Gaussians.from_scene(scene, "cuda")
     counters = torch.zeros(8, dtype=torch.int64, device="cuda")
     out = []
