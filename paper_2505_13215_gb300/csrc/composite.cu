@@ -337,6 +337,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
                                                                    splat_image img, L1Fuse l1, int32_t* status,
                                                                    unsigned long long* stats)
 {
+    wait_for_previous_kernel();
     static_assert(PPL == 2 || PPL == 4 || PPL == 8, "pixels per lane come in pairs");
     constexpr int BANDS = 8 / PPL, NP = PPL / 2;
     __shared__ float4 s_feat[kCompWarps][32][kFeat];
@@ -741,6 +742,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks
                                                                    float* dproj, int32_t* status,
                                                                    unsigned long long* stats)
 {
+    wait_for_previous_kernel();
     static_assert(PPL == 2 || PPL == 4 || PPL == 8, "pixels per lane come in pairs");
     constexpr int BANDS = 8 / PPL, NP = PPL / 2;
     __shared__ float4 s_feat[kCompWarps][32][kFeat];
@@ -931,6 +933,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks
 __global__ void __launch_bounds__(256) k_l1_loss(const float* __restrict__ img, const float* __restrict__ target,
                                                  int64_t n, float scale, float* __restrict__ dL, float* loss)
 {
+    wait_for_previous_kernel();
     float acc = 0.f;
     const int64_t n4 = n / 4;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
@@ -965,13 +968,14 @@ cudaError_t launch_l1_loss(const float* img, const float* target, int64_t n, flo
     const int64_t want = (n / 4 + 255) / 256 + 1;
     const int blocks = (int)(want < (int64_t)ctx.num_sms * 8 ? want : (int64_t)ctx.num_sms * 8);
     count_launch();
-    k_l1_loss<<<blocks, 256, 0, ctx.stream>>>(img, target, n, scale, dL, loss);
+    launch_kernel(k_l1_loss, blocks, 256, 0, ctx.stream, img, target, n, scale, dL, loss);
     return cudaGetLastError();
 }
 
 // *loss = the sum of the kLossParts partial sums
 __global__ void __launch_bounds__(256) k_loss_sum(const float* __restrict__ partial, float* loss)
 {
+    wait_for_previous_kernel();
     float acc = 0.f;
 #pragma unroll
     for (int i = 0; i < kLossParts / 256; ++i) acc += partial[threadIdx.x + 256 * i];
@@ -994,9 +998,9 @@ static void fwd_launch(int ppl, int blocks, cudaStream_t st, const splat_proj& p
 {
     const uint2* rg = (const uint2*)bins.ranges;
     switch (ppl) {
-    case 8: k_composite_fwd<8, ST><<<blocks, kCompWarps * 32, 0, st>>>(proj, bins.vals, rg, bins.tile_order, vb, img, l1, status, stats); break;
-    case 4: k_composite_fwd<4, ST><<<blocks, kCompWarps * 32, 0, st>>>(proj, bins.vals, rg, bins.tile_order, vb, img, l1, status, stats); break;
-    default: k_composite_fwd<2, ST><<<blocks, kCompWarps * 32, 0, st>>>(proj, bins.vals, rg, bins.tile_order, vb, img, l1, status, stats); break;
+    case 8: launch_kernel(k_composite_fwd<8, ST>, blocks, kCompWarps * 32, 0, st, proj, bins.vals, rg, bins.tile_order, vb, img, l1, status, stats); break;
+    case 4: launch_kernel(k_composite_fwd<4, ST>, blocks, kCompWarps * 32, 0, st, proj, bins.vals, rg, bins.tile_order, vb, img, l1, status, stats); break;
+    default: launch_kernel(k_composite_fwd<2, ST>, blocks, kCompWarps * 32, 0, st, proj, bins.vals, rg, bins.tile_order, vb, img, l1, status, stats); break;
     }
 }
 
@@ -1007,9 +1011,9 @@ static void bwd_launch(int ppl, int blocks, cudaStream_t st, const splat_proj& p
 {
     const uint2* rg = (const uint2*)bins.ranges;
     switch (ppl) {
-    case 8: k_composite_bwd<8, ST><<<blocks, kCompWarps * 32, 0, st>>>(proj, bins.vals, rg, bins.tile_order, vb, img, dL, dproj, status, stats); break;
-    case 4: k_composite_bwd<4, ST><<<blocks, kCompWarps * 32, 0, st>>>(proj, bins.vals, rg, bins.tile_order, vb, img, dL, dproj, status, stats); break;
-    default: k_composite_bwd<2, ST><<<blocks, kCompWarps * 32, 0, st>>>(proj, bins.vals, rg, bins.tile_order, vb, img, dL, dproj, status, stats); break;
+    case 8: launch_kernel(k_composite_bwd<8, ST>, blocks, kCompWarps * 32, 0, st, proj, bins.vals, rg, bins.tile_order, vb, img, dL, dproj, status, stats); break;
+    case 4: launch_kernel(k_composite_bwd<4, ST>, blocks, kCompWarps * 32, 0, st, proj, bins.vals, rg, bins.tile_order, vb, img, dL, dproj, status, stats); break;
+    default: launch_kernel(k_composite_bwd<2, ST>, blocks, kCompWarps * 32, 0, st, proj, bins.vals, rg, bins.tile_order, vb, img, dL, dproj, status, stats); break;
     }
 }
 
@@ -1051,7 +1055,7 @@ cudaError_t launch_composite_fwd(const splat_proj& proj, const splat_bins& bins,
     else fwd_launch<false>(ppl, blocks, ctx.stream, proj, bins, vb, img, l1, status, nullptr);
     if (l1.partial) {
         count_launch();
-        k_loss_sum<<<1, 256, 0, ctx.stream>>>(l1.partial, l1.loss);
+        launch_kernel(k_loss_sum, 1, 256, 0, ctx.stream, l1.partial, l1.loss);
     }
     return cudaGetLastError();
 }

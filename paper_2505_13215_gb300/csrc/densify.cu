@@ -45,6 +45,7 @@ struct StatArgs {
 
 __global__ void __launch_bounds__(256) k_dens_stats(StatArgs a)
 {
+    wait_for_previous_kernel();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.N; i += (int64_t)gridDim.x * blockDim.x) {
         float acc = 0.f, cnt = 0.f;
         for (int v = 0; v < a.V; ++v) {
@@ -67,7 +68,7 @@ cudaError_t launch_dens_stats(const StatArgs& a, const LaunchCtx& ctx)
     if (a.N == 0) return cudaSuccess;
     const int blocks = (int)std::min<int64_t>((a.N + 255) / 256, (int64_t)ctx.num_sms * 8);
     count_launch();
-    k_dens_stats<<<blocks, 256, 0, ctx.stream>>>(a);
+    launch_kernel(k_dens_stats, blocks, 256, 0, ctx.stream, a);
     return cudaGetLastError();
 }
 

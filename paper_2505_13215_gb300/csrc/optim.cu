@@ -58,6 +58,7 @@ __device__ __forceinline__ float adam_one(const OptArgs& a, float lr, float g, f
 template <int DT>
 __global__ void __launch_bounds__(kOptThreads) k_adam(OptArgs a)
 {
+    wait_for_previous_kernel();
     if (status_failed(a.status)) return;
     const OptSeg s = a.seg[blockIdx.y];
     const int64_t n4 = s.n / 4;
@@ -120,9 +121,9 @@ cudaError_t launch_adam(const OptArgs& a, const LaunchCtx& ctx)
     const dim3 grid(opt_blocks(a, ctx), a.nseg);
     count_launch();
     switch (a.dtype) {
-    case SPLAT_F32: k_adam<SPLAT_F32><<<grid, kOptThreads, 0, ctx.stream>>>(a); break;
-    case SPLAT_BF16: k_adam<SPLAT_BF16><<<grid, kOptThreads, 0, ctx.stream>>>(a); break;
-    default: k_adam<SPLAT_F16><<<grid, kOptThreads, 0, ctx.stream>>>(a); break;
+    case SPLAT_F32: launch_kernel(k_adam<SPLAT_F32>, grid, kOptThreads, 0, ctx.stream, a); break;
+    case SPLAT_BF16: launch_kernel(k_adam<SPLAT_BF16>, grid, kOptThreads, 0, ctx.stream, a); break;
+    default: launch_kernel(k_adam<SPLAT_F16>, grid, kOptThreads, 0, ctx.stream, a); break;
     }
     return cudaGetLastError();
 }

@@ -267,6 +267,7 @@ template <int DT>
 __global__ void __launch_bounds__(128, 7) k_slice_project(splat_g3 g3, splat_g4 g4, ViewBatch vb, splat_proj out,
                                                        int32_t* status)
 {
+    wait_for_previous_kernel();
     const int64_t N = out.n;
     const int64_t n4 = g4.n;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
@@ -472,6 +473,7 @@ __global__ void __launch_bounds__(kAdjThreads, 6) k_adjoint(splat_g3 g3, splat_g
                                                  const float* __restrict__ dproj, splat_grads3 dg3,
                                                  splat_grads4 dg4, int32_t* status)
 {
+    wait_for_previous_kernel();
     static_assert(L == 1 || L == 2 || L == 4 || L == 8 || L == 16, "lanes per Gaussian");
     constexpr int KPL = 16 / L;  // SH functions whose gradient a lane writes
     constexpr int GPS = 32 / L;  // Gaussians per sub-batch of a warp
@@ -815,9 +817,9 @@ cudaError_t launch_slice_project(const splat_g3& g3, const splat_g4& g4, const V
     const int blocks = (int)(want < (int64_t)ctx.num_sms * 64 ? want : (int64_t)ctx.num_sms * 64);
     count_launch();
     switch (dtype) {
-    case SPLAT_F32: k_slice_project<SPLAT_F32><<<blocks, threads, 0, ctx.stream>>>(g3, g4, vb, out, status); break;
-    case SPLAT_BF16: k_slice_project<SPLAT_BF16><<<blocks, threads, 0, ctx.stream>>>(g3, g4, vb, out, status); break;
-    default: k_slice_project<SPLAT_F16><<<blocks, threads, 0, ctx.stream>>>(g3, g4, vb, out, status); break;
+    case SPLAT_F32: launch_kernel(k_slice_project<SPLAT_F32>, blocks, threads, 0, ctx.stream, g3, g4, vb, out, status); break;
+    case SPLAT_BF16: launch_kernel(k_slice_project<SPLAT_BF16>, blocks, threads, 0, ctx.stream, g3, g4, vb, out, status); break;
+    default: launch_kernel(k_slice_project<SPLAT_F16>, blocks, threads, 0, ctx.stream, g3, g4, vb, out, status); break;
     }
     return cudaGetLastError();
 }
@@ -827,7 +829,7 @@ static void adjoint_launch(int blocks, cudaStream_t st, const splat_g3& g3, cons
                            const splat_proj& proj, const float* dproj, const splat_grads3& dg3,
                            const splat_grads4& dg4, int32_t* status)
 {
-    k_adjoint<DT, L><<<blocks, kAdjThreads, 0, st>>>(g3, g4, vb, proj, dproj, dg3, dg4, status);
+    launch_kernel(k_adjoint<DT, L>, blocks, kAdjThreads, 0, st, g3, g4, vb, proj, dproj, dg3, dg4, status);
 }
 
 template <int DT>

@@ -667,6 +667,7 @@ __device__ __forceinline__ uint32_t* cell_copy(const CellArgs& a)
 // scatter does, costs the same on wide splats and more on small ones).
 __global__ void __launch_bounds__(256) k_cell_count(CellArgs a)
 {
+    wait_for_previous_kernel();
     __shared__ uint32_t s_mm[2][8];
     const int v = blockIdx.y;
     const int64_t i = blockIdx.x * 256ll + threadIdx.x;
@@ -717,6 +718,7 @@ __device__ __forceinline__ int lower_bound(const uint32_t* p, int n, uint32_t x)
 // Block per super-tile, taken in ticket order (look-back over the super-tiles).
 __global__ void __launch_bounds__(256) k_cell_scan(CellArgs a)
 {
+    wait_for_previous_kernel();
     __shared__ uint32_t s_p[kMaxBins + 1];  // first entry of each bin, relative to the list
     __shared__ uint32_t s_tmp[8];
     __shared__ unsigned long long s_excl;
@@ -834,6 +836,7 @@ __global__ void __launch_bounds__(256) k_cell_scan(CellArgs a)
 // entries one after the other would wait for one another's.
 __global__ void __launch_bounds__(256) k_cell_scatter(CellArgs a)
 {
+    wait_for_previous_kernel();
     if (status_failed(a.status)) return;  // includes K1 above the capacity
     const int v = blockIdx.y, lane = threadIdx.x & 31;
     const int64_t i = blockIdx.x * 256ll + threadIdx.x;
@@ -1213,6 +1216,7 @@ __device__ __noinline__ void sort_part(SortSmem& s, const unsigned long long* sr
 template <bool REST>
 __global__ void __launch_bounds__(kUnitThreads, 2) k_unit_sort(SortArgs a)
 {
+    wait_for_previous_kernel();
     __shared__ SortSmem s;
     if (status_failed(a.status)) return;
     const uint32_t direct = REST ? 0u : (uint32_t)a.total_super;
@@ -1280,6 +1284,7 @@ template <bool SCATTER>
 __global__ void __launch_bounds__(256) k_tile_order(const uint2* ranges, int n, uint32_t* cls, uint32_t* order,
                                                     int32_t* status)
 {
+    wait_for_previous_kernel();
     __shared__ uint32_t s_start[kOrderClasses];
     __shared__ uint32_t s_tmp[8];
     if (status_failed(status)) return;
@@ -1322,10 +1327,10 @@ static cudaError_t launch_tile_order(const splat_bins& bins, int64_t total_tiles
         cudaError_t e = cudaMemsetAsync(cls, 0, 2 * kOrderClasses * sizeof(uint32_t), ctx.stream);
         if (e != cudaSuccess) return e;
         count_launch();
-        k_tile_order<false><<<blocks, 256, 0, ctx.stream>>>((const uint2*)bins.ranges, n, cls, bins.tile_order, status);
+        launch_kernel(k_tile_order<false>, blocks, 256, 0, ctx.stream, (const uint2*)bins.ranges, n, cls, bins.tile_order, status);
     }
     count_launch();
-    k_tile_order<true><<<blocks, 256, 0, ctx.stream>>>((const uint2*)bins.ranges, n, cls, bins.tile_order, status);
+    launch_kernel(k_tile_order<true>, blocks, 256, 0, ctx.stream, (const uint2*)bins.ranges, n, cls, bins.tile_order, status);
     return cudaGetLastError();
 }
 
@@ -1505,6 +1510,7 @@ struct TileRangeArgs {
 
 __global__ void __launch_bounds__(256) k_tile_ranges(TileArgs a, TileRangeArgs r)
 {
+    wait_for_previous_kernel();
     __shared__ unsigned long long s_tmp64[8];
     __shared__ unsigned long long s_excl;
     __shared__ int64_t s_ticket;
@@ -1670,6 +1676,7 @@ __device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane)
 // on 1M Gaussians at 4 x 2704x2028, 50 us on 300k at 4 x 1352x1014.
 __global__ void __launch_bounds__(kHeadEntries, 2) k_head_count(TileArgs a)
 {
+    wait_for_previous_kernel();
     constexpr int kGroups = kHeadEntries / 32;
     __shared__ uint32_t s_sum[kGroups][32];  // saturation weights of each (group, tile)
     __shared__ uint32_t s_word[kGroups][32];
@@ -1773,6 +1780,7 @@ __global__ void __launch_bounds__(kHeadEntries, 2) k_head_count(TileArgs a)
 // Gaussians at 4 x 2704x2028.
 __global__ void __launch_bounds__(256) k_tail_count(TileArgs a)
 {
+    wait_for_previous_kernel();
     __shared__ uint32_t s_cnt[8][64];
     __shared__ uint32_t s_g;
     __shared__ int s_gs;
@@ -1859,6 +1867,7 @@ constexpr int kSparse = 6;
 
 __global__ void __launch_bounds__(256) k_tile_write(TileArgs a)
 {
+    wait_for_previous_kernel();
     __shared__ uint32_t s_row[kFilterSeg];
     __shared__ uint32_t s_buf[8][32 * kSparse];
     __shared__ uint32_t s_tk;
@@ -2218,9 +2227,9 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         c.n_needed = bins.n_needed;
         const dim3 row_grid((unsigned)((proj.n + 255) / 256), (unsigned)vb.V);
         count_launch(3);
-        k_cell_count<<<row_grid, 256, 0, s>>>(c);
-        k_cell_scan<<<sb, 256, 0, s>>>(c);
-        k_cell_scatter<<<row_grid, 256, 0, s>>>(c);
+        launch_kernel(k_cell_count, row_grid, 256, 0, s, c);
+        launch_kernel(k_cell_scan, sb, 256, 0, s, c);
+        launch_kernel(k_cell_scatter, row_grid, 256, 0, s, c);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         // 2. the units of each list that the head pass takes, in order
         SortArgs u{};
@@ -2290,12 +2299,12 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
             return (int)std::min<int64_t>(L.max_segs + (write ? sb : 0), (int64_t)ctx.num_sms * per_sm_f[write]);
         };
         count_launch(6);
-        k_unit_sort<false><<<blocks_u(0), kUnitThreads, 0, s>>>(u);
-        k_head_count<<<2 * sb, kHeadEntries, 0, s>>>(t);
-        k_unit_sort<true><<<blocks_u(1), kUnitThreads, 0, s>>>(u);
-        k_tail_count<<<blocks_f(0), 256, 0, s>>>(t);
-        k_tile_ranges<<<(int)((vb.total_tiles + kRangeTiles - 1) / kRangeTiles), 256, 0, s>>>(t, tr);
-        k_tile_write<<<blocks_f(1), 256, 0, s>>>(t);
+        launch_kernel(k_unit_sort<false>, blocks_u(0), kUnitThreads, 0, s, u);
+        launch_kernel(k_head_count, 2 * sb, kHeadEntries, 0, s, t);
+        launch_kernel(k_unit_sort<true>, blocks_u(1), kUnitThreads, 0, s, u);
+        launch_kernel(k_tail_count, blocks_f(0), 256, 0, s, t);
+        launch_kernel(k_tile_ranges, (int)((vb.total_tiles + kRangeTiles - 1) / kRangeTiles), 256, 0, s, t, tr);
+        launch_kernel(k_tile_write, blocks_f(1), 256, 0, s, t);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         return launch_tile_order(bins, L.total_tiles, U(L.off_tord), status, ctx, true);
     }
