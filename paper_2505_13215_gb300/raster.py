@@ -440,14 +440,19 @@ class HybridRasterize(torch.autograd.Function):
     def backward(ctx, grad_rgb):
         R, G = ctx.R, ctx.G
         R.backward(G, grad_rgb.contiguous())
-        out = [None, None]
-        for k in FIELDS3:
-            g = torch.zeros_like(G.t[k], dtype=torch.float32)
-            g[: G.n3] = R.grads[k]
-            out.append(g.to(G.t[k].dtype))
-        for k in FIELDS4:
-            out.append(R.grads[k].clone().to(G.t[k].dtype))
-        return tuple(out)
+        # the gradients leave R's buffers in one multi-tensor copy (rounded to the storage
+        # type); 3D rows past n3 have none
+        out, dst = [], []
+        for k in FIELDS3 + FIELDS4:
+            rows = G.capacity3 if k in FIELDS3 else R.n4
+            g = torch.empty((rows,) + tuple(R.grads[k].shape[1:]), dtype=G.t[k].dtype, device=G.t[k].device)
+            n = R.grads[k].shape[0]
+            if rows > n:
+                g[n:].zero_()
+            out.append(g)
+            dst.append(g if rows == n else g[:n])
+        torch._foreach_copy_(dst, [R.grads[k] for k in FIELDS3 + FIELDS4])
+        return (None, None, *out)
 
 
 def render(G: Gaussians, views, capacity=None) -> List[torch.Tensor]:
