@@ -575,7 +575,7 @@ constexpr int64_t kBinMaxTiles = 40960;  // per view: the binned path's default 
 constexpr int kSplitMaxSmem = 200 * 1024;
 constexpr int kMaxBins = 1024;           // depth bins per super-tile
 constexpr int kUnit = 2048;              // entries a block sorts in shared memory
-constexpr int kUnitThreads = 512, kPer = kUnit / kUnitThreads;
+constexpr int kUnitThreads = 256, kPer = kUnit / kUnitThreads;
 constexpr int kUnitStep = kUnit / 2;     // a unit starts at the first bin start at or after each multiple
 constexpr int kSortBuckets = 2048;
 constexpr int kSortBucketBits = 11;
@@ -907,6 +907,7 @@ struct SortSmem {
     unsigned long long e[kUnit];
     uint32_t h[kSortBuckets + 4];  // bucket counts, then first positions; [kSortBuckets]: the total
     uint32_t h2[kSortBuckets + 4];  // the same of the second level
+    uint16_t at[kUnit];            // arrival in a second-level bucket
     uint32_t red[4][kUnitThreads / 32], tmp[kUnitThreads / 32];
     uint32_t n;
 };
@@ -960,108 +961,37 @@ __device__ __forceinline__ void block_bounds(SortSmem& s, uint32_t dmin, uint32_
 // (block-uniform) whether a bucket is crowded.
 __device__ __forceinline__ bool scan_buckets(SortSmem& s, uint32_t* h)
 {
-    static_assert(kSortBuckets == 4 * kUnitThreads, "four buckets per thread");
-    uint4* h4 = (uint4*)h + threadIdx.x;
-    const uint4 c = *h4;
-    const uint32_t mx = max(max(c.x, c.y), max(c.z, c.w));
+    static_assert(kSortBuckets == 8 * kUnitThreads, "eight buckets per thread");
+    uint4* h4 = (uint4*)h + 2 * threadIdx.x;
+    const uint4 c = h4[0], d = h4[1];
+    const uint32_t mx = max(max(max(c.x, c.y), max(c.z, c.w)), max(max(d.x, d.y), max(d.z, d.w)));
+    const uint32_t sc = c.x + c.y + c.z + c.w;
     uint32_t total;
-    const uint32_t x = block_excl_scan<kUnitThreads / 32>(c.x + c.y + c.z + c.w, s.tmp, &total);
-    *h4 = make_uint4(x, x + c.x, x + c.x + c.y, x + c.x + c.y + c.z);
+    const uint32_t x = block_excl_scan<kUnitThreads / 32>(sc + d.x + d.y + d.z + d.w, s.tmp, &total), y = x + sc;
+    h4[0] = make_uint4(x, x + c.x, x + c.x + c.y, x + c.x + c.y + c.z);
+    h4[1] = make_uint4(y, y + d.x, y + d.x + d.y, y + d.x + d.y + d.z);
     if (threadIdx.x == 0) h[kSortBuckets] = total;
     return __syncthreads_or(mx > kCrowded);
 }
 
-// Every entry of s.e[0 .. n), entry t + kUnitThreads k in e[k] of thread t and b[k] its
-// bucket of first positions h, to its place by the count of smaller ones in its
-// bucket; their rows to dst.
-__device__ __forceinline__ void place_rows(SortSmem& s, const unsigned long long (&e)[kPer],
-                                           uint32_t (&b)[kPer], const uint32_t* h, int n,
-                                           uint32_t* __restrict__ dst)
+// The second-level position of entry e, whose bucket is b: the bucket's first
+// position, in a crowded bucket plus a share of its length linear in the row.
+__device__ __forceinline__ uint32_t second_level(const SortSmem& s, uint32_t b, uint32_t row, uint32_t rmin, int up)
 {
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        if (tid + kUnitThreads * k < n) {
-            const uint32_t j1 = h[b[k] + 1];
-            uint32_t j = h[b[k]], r = j;
-#pragma unroll 1
-            for (; j < j1; ++j) r += s.e[j] < e[k];
-            b[k] = r;
-        }
-    }
-    __syncthreads();
-    uint32_t* rows = (uint32_t*)s.e;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k)
-        if (tid + kUnitThreads * k < n) rows[b[k]] = (uint32_t)e[k];
-    __syncthreads();
-    for (int i = tid; i < n; i += kUnitThreads) dst[i] = rows[i];
-    __syncthreads();
+    const uint32_t p = s.h[b], c = s.h[b + 1] - p;
+    return c > kCrowded ? p + __umulhi((row - rmin) << up, c) : p;
 }
 
-// A unit with crowded buckets, the entries in bucket order in s.e (kr, s.h):
-// many equal depths (means stored in 16 bits seen along an axis, planes facing
-// the camera).  A second counting pass spreads the crowded buckets' entries
-// over their positions by row (in [rmin, rmax]); should such a bucket hold
-// different depths, or the rows crowd as well, the unit is sorted bitonically.
-__device__ __noinline__ void sort_crowded(SortSmem& s, KeyRange kr, uint32_t rmin, uint32_t rmax, int n, uint32_t* dst)
-{
-    const int tid = threadIdx.x, up = __clz(max(1u, rmax - rmin));
-    unsigned long long e[kPer];
-    uint32_t b[kPer], at[kPer];
-    bool mixed = false;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        if (tid + kUnitThreads * k < n) {
-            e[k] = s.e[tid + kUnitThreads * k];
-            const uint32_t d = key_bucket(kr, e[k]), p = s.h[d], c = s.h[d + 1] - p;
-            b[k] = p;
-            if (c > kCrowded) {
-                mixed |= (s.e[p] >> 32) != (e[k] >> 32);
-                b[k] = p + __umulhi(((uint32_t)e[k] - rmin) << up, c);
-            }
-        }
-        s.h2[tid + kUnitThreads * k] = 0u;
-    }
-    if (!__syncthreads_or(mixed)) {
-#pragma unroll
-        for (int k = 0; k < kPer; ++k)
-            if (tid + kUnitThreads * k < n) at[k] = atomicAdd(&s.h2[b[k]], 1u);
-        __syncthreads();
-        if (!scan_buckets(s, s.h2)) {
-#pragma unroll
-            for (int k = 0; k < kPer; ++k)
-                if (tid + kUnitThreads * k < n) s.e[s.h2[b[k]] + at[k]] = e[k];
-            __syncthreads();
-            place_rows(s, e, b, s.h2, n, dst);
-            return;
-        }
-    }
-    int P = 2;
-    while (P < n) P <<= 1;
-    for (int i = n + tid; i < P; i += kUnitThreads) s.e[i] = ~0ull;
-    __syncthreads();
-    for (int size = 2; size <= P; size <<= 1) {
-        for (int step = size >> 1; step > 0; step >>= 1) {
-            for (int t = tid; t < P / 2; t += kUnitThreads) {
-                const int i = 2 * t - (t & (step - 1)), j = i + step;
-                const unsigned long long x = s.e[i], y = s.e[j];
-                if ((x > y) == ((i & size) == 0)) {
-                    s.e[i] = y;
-                    s.e[j] = x;
-                }
-            }
-            __syncthreads();
-        }
-    }
-    for (int i = tid; i < n; i += kUnitThreads) dst[i] = (uint32_t)s.e[i];
-    __syncthreads();
-}
-
-// Sorts a unit of n <= kUnit entries, entry t + kUnitThreads k in e[k] of thread t, and
-// writes their rows to dst: one counting-sort pass over buckets linear in the
-// key (about one entry each), then every entry counts the smaller ones of its
-// bucket.
+// Sorts a unit of n <= kUnit entries, entry t + kUnitThreads k in e[k] of thread
+// t, and writes their rows to dst: one counting-sort pass over buckets linear in
+// the key (about one entry each), then every entry counts the smaller ones of its
+// bucket.  Where a bucket is crowded (many equal depths: means stored in 16 bits
+// seen along an axis, planes facing the camera), a second counting pass spreads
+// the crowded buckets' entries over their positions by row; should such a bucket
+// hold different depths, or the rows crowd as well, the unit is sorted
+// bitonically.  (The second pass keeps its arrivals in shared memory: in
+// registers they made the common path spill, 78 -> 118 us for the rest of the
+// lists of 1M Gaussians at 4 x 2704x2028.)
 __device__ __forceinline__ void sort_unit(SortSmem& s, const unsigned long long (&e)[kPer], int n,
                                           uint32_t* __restrict__ dst)
 {
@@ -1093,20 +1023,90 @@ __device__ __forceinline__ void sort_unit(SortSmem& s, const unsigned long long 
         if (tid + kUnitThreads * k < n) {
             const uint32_t b = key_bucket(kr, e[k]);
             s.e[s.h[b] + at[k]] = e[k];
-            at[k] = b;
         }
     }
     __syncthreads();
-    if (crowded) {  // (block-uniform)
+    if (!crowded) {
 #pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            if (tid + kUnitThreads * k < n) {
+                const uint32_t b = key_bucket(kr, e[k]), j1 = s.h[b + 1];
+                uint32_t j = s.h[b], r = j;
+                for (; j < j1; ++j) r += s.e[j] < e[k];
+                at[k] = r;
+            }
+        }
+        __syncthreads();
+        uint32_t* rows = (uint32_t*)s.e;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k)
+            if (tid + kUnitThreads * k < n) rows[at[k]] = (uint32_t)e[k];
+        __syncthreads();
+        for (int i = tid; i < n; i += kUnitThreads) dst[i] = rows[i];
+    } else {
+        rmin = 0xffffffffu;
+        rmax = 0u;
         for (int w = 0; w < kUnitThreads / 32; ++w) {  // the block's bounds of the rows, as block_bounds left the warps'
             rmin = min(rmin, s.red[2][w]);
             rmax = max(rmax, s.red[3][w]);
         }
-        sort_crowded(s, kr, rmin, rmax, n, dst);
-    } else {
-        place_rows(s, e, at, s.h, n, dst);
+        const int up = __clz(max(1u, rmax - rmin));
+        for (int i = tid; i < kSortBuckets; i += kUnitThreads) s.h2[i] = 0u;
+        __syncthreads();
+        bool mixed = false;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            if (tid + kUnitThreads * k < n) {
+                const uint32_t b = key_bucket(kr, e[k]);
+                const uint32_t p = second_level(s, b, (uint32_t)e[k], rmin, up);
+                mixed |= s.h[b + 1] - s.h[b] > kCrowded && (s.e[s.h[b]] >> 32) != (e[k] >> 32);
+                s.at[tid + kUnitThreads * k] = (uint16_t)atomicAdd(&s.h2[p], 1u);
+            }
+        }
+        mixed = __syncthreads_or(mixed);
+        if (!mixed) mixed = scan_buckets(s, s.h2);
+        if (!mixed) {
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                if (tid + kUnitThreads * k < n) {
+                    const uint32_t p = second_level(s, key_bucket(kr, e[k]), (uint32_t)e[k], rmin, up);
+                    s.e[s.h2[p] + s.at[tid + kUnitThreads * k]] = e[k];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                if (tid + kUnitThreads * k < n) {
+                    const uint32_t p = second_level(s, key_bucket(kr, e[k]), (uint32_t)e[k], rmin, up);
+                    const uint32_t j1 = s.h2[p + 1];
+                    uint32_t j = s.h2[p], r = j;
+#pragma unroll 1
+                    for (; j < j1; ++j) r += s.e[j] < e[k];
+                    dst[r] = (uint32_t)e[k];
+                }
+            }
+        } else {
+            int P = 2;
+            while (P < n) P <<= 1;
+            for (int i = n + tid; i < P; i += kUnitThreads) s.e[i] = ~0ull;
+            __syncthreads();
+            for (int size = 2; size <= P; size <<= 1) {
+                for (int step = size >> 1; step > 0; step >>= 1) {
+                    for (int t = tid; t < P / 2; t += kUnitThreads) {
+                        const int i = 2 * t - (t & (step - 1)), j = i + step;
+                        const unsigned long long x = s.e[i], y = s.e[j];
+                        if ((x > y) == ((i & size) == 0)) {
+                            s.e[i] = y;
+                            s.e[j] = x;
+                        }
+                    }
+                    __syncthreads();
+                }
+            }
+            for (int i = tid; i < n; i += kUnitThreads) dst[i] = (uint32_t)s.e[i];
+        }
     }
+    __syncthreads();
 }
 
 // f(entry) for every one of src[0 .. n), eight loads in flight per thread (with
@@ -1145,11 +1145,11 @@ __device__ __forceinline__ KeyRange count_range(SortSmem& s, const unsigned long
 // Part g of a unit of more than kUnit entries (one depth bin of a crowded
 // list): the parts' blocks each count the whole unit by value and take the
 // entries of the g-th run of buckets, about kUnitStep of them, so that any
-// number of blocks share a long unit without waiting for one another.  A run
-// that holds more than kUnit (one crowded bucket) goes through value ranges
-// of at most kUnit entries one after the other, each found by counting again
-// over ever finer buckets (entries are unique, so this ends).
-__device__ __noinline__ void sort_part(SortSmem& s, const unsigned long long* src, uint32_t n, uint32_t g, uint32_t* dst)
+// number of blocks share a long unit without waiting for one another.
+// Sets the value range [lo, hi] of the part, the number of its entries and their
+// first position in the unit.
+__device__ __noinline__ void part_range(SortSmem& s, const unsigned long long* src, uint32_t n, uint32_t g,
+                                        unsigned long long& lo, unsigned long long& hi, uint32_t& left, uint32_t& out)
 {
     const int tid = threadIdx.x;
     // buckets over the range of a sample of kUnit entries, the first and the last open-ended
@@ -1162,59 +1162,61 @@ __device__ __noinline__ void sort_part(SortSmem& s, const unsigned long long* sr
         rmin = min(rmin, (uint32_t)x);
         rmax = max(rmax, (uint32_t)x);
     }
-    unsigned long long lo, hi;
     block_bounds(s, dmin, dmax, rmin, rmax, lo, hi);
     __syncthreads();
-    KeyRange kr = count_range(s, src, n, lo, hi, true);
+    const KeyRange kr = count_range(s, src, n, lo, hi, true);
     const int b0 = lower_bound(s.h, kSortBuckets, g * kUnitStep), b1 = lower_bound(s.h, kSortBuckets, (g + 1) * kUnitStep);
-    uint32_t out = s.h[b0], left = s.h[b1] - out;
+    out = s.h[b0];
+    left = s.h[b1] - out;
     hi = b1 < kSortBuckets ? lo + ((unsigned long long)b1 << kr.shift) - 1 : ~0ull;
     lo = b0 > 0 ? lo + ((unsigned long long)b0 << kr.shift) : 0ull;
     __syncthreads();
-    while (left > 0) {  // (block-uniform) the entries in [lo, hi] are still to be written, from dst[out] on
-        unsigned long long top = hi;
-        uint32_t m = left;
-        while (m > (uint32_t)kUnit && lo < top) {
-            kr = count_range(s, src, n, lo, top);
-            // the buckets below b hold at most kUnit entries, those up to and including b more
-            const int b = lower_bound(s.h, kSortBuckets, kUnit + 1) - 1;
-            m = s.h[b];
-            if (m == 0) {  // bucket b alone holds too many
-                m = s.h[b + 1];
-                lo += (unsigned long long)b << kr.shift;
-                top = min(top, lo + (1ull << kr.shift) - 1);
-            } else {
-                top = lo + ((unsigned long long)b << kr.shift) - 1;
-            }
-            __syncthreads();
+}
+
+// The first up to kUnit entries by value of a part's `left` ones in [lo, hi] into
+// s.e: returns their number and the value top up to which they go (0: none).  A
+// part that holds more than kUnit (one crowded bucket) goes through several of
+// these, each found by counting again over ever finer buckets (entries are unique,
+// so this ends).
+__device__ __noinline__ uint32_t take_range(SortSmem& s, const unsigned long long* src, uint32_t n, uint32_t left,
+                                            unsigned long long& lo, unsigned long long hi, unsigned long long& top)
+{
+    const int tid = threadIdx.x;
+    top = hi;
+    uint32_t m = left;
+    while (m > (uint32_t)kUnit && lo < top) {
+        const KeyRange kr = count_range(s, src, n, lo, top);
+        // the buckets below b hold at most kUnit entries, those up to and including b more
+        const int b = lower_bound(s.h, kSortBuckets, kUnit + 1) - 1;
+        m = s.h[b];
+        if (m == 0) {  // bucket b alone holds too many
+            m = s.h[b + 1];
+            lo += (unsigned long long)b << kr.shift;
+            top = min(top, lo + (1ull << kr.shift) - 1);
+        } else {
+            top = lo + ((unsigned long long)b << kr.shift) - 1;
         }
-        m = min(min(m, left), (uint32_t)kUnit);
-        if (m == 0) break;  // (not for consistent counts: bounds the loop whatever the buffer holds)
-        if (tid == 0) s.n = 0u;
         __syncthreads();
-        each_entry(src, n, [&](unsigned long long x) {
-            if (x >= lo && x <= top) {
-                const uint32_t at = atomicAdd(&s.n, 1u);
-                if (at < (uint32_t)kUnit) s.e[at] = x;
-            }
-        });
-        __syncthreads();
-        unsigned long long e[kPer];
-#pragma unroll
-        for (int k = 0; k < kPer; ++k) e[k] = tid + kUnitThreads * k < (int)m ? s.e[tid + kUnitThreads * k] : 0ull;
-        __syncthreads();
-        sort_unit(s, e, (int)m, dst + out);
-        out += m;
-        left -= m;
-        lo = top + 1;
     }
+    m = min(min(m, left), (uint32_t)kUnit);
+    if (m == 0) return 0u;  // (not for consistent counts: bounds the loop whatever the buffer holds)
+    if (tid == 0) s.n = 0u;
+    __syncthreads();
+    each_entry(src, n, [&](unsigned long long x) {
+        if (x >= lo && x <= top) {
+            const uint32_t at = atomicAdd(&s.n, 1u);
+            if (at < (uint32_t)kUnit) s.e[at] = x;
+        }
+    });
+    __syncthreads();
+    return m;
 }
 
 // REST false: the lists of at most kUnit entries and the longer lists' units
-// that hold their first kHeadEntries; true: the longer lists' other units,
+// that hold their head's entries; true: the longer lists' other units,
 // where a tile's list goes on past the head.
 template <bool REST>
-__global__ void __launch_bounds__(kUnitThreads, 2) k_unit_sort(SortArgs a)
+__global__ void __launch_bounds__(kUnitThreads, 4) k_unit_sort(SortArgs a)
 {
     wait_for_previous_kernel();
     __shared__ SortSmem s;
@@ -1239,17 +1241,34 @@ __global__ void __launch_bounds__(kUnitThreads, 2) k_unit_sort(SortArgs a)
             }
         }
         if (st >= en) continue;  // (block-uniform)
-        const int n = (int)(en - st);
-        if (part == kWholeUnit) {
+        const uint32_t n = en - st;
+        unsigned long long lo = 0ull, hi = ~0ull;
+        uint32_t left = n, out = 0u;
+        if (part != kWholeUnit) part_range(s, a.entries + st, n, part, lo, hi, left, out);
+        while (left > 0) {  // (block-uniform) once for a whole unit
+            uint32_t m = left;
+            unsigned long long top = hi;
             unsigned long long e[kPer];
+            if (part == kWholeUnit) {
 #pragma unroll
-            for (int k = 0; k < kPer; ++k) {
-                const int i = (int)threadIdx.x + kUnitThreads * k;
-                e[k] = i < n ? a.entries[st + i] : 0ull;
+                for (int k = 0; k < kPer; ++k) {
+                    const uint32_t i = threadIdx.x + kUnitThreads * k;
+                    e[k] = i < n ? a.entries[st + i] : 0ull;
+                }
+            } else {
+                m = take_range(s, a.entries + st, n, left, lo, hi, top);
+                if (m == 0) break;
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    const uint32_t i = threadIdx.x + kUnitThreads * k;
+                    e[k] = i < m ? s.e[i] : 0ull;
+                }
+                __syncthreads();
             }
-            sort_unit(s, e, n, a.list + st);
-        } else {
-            sort_part(s, a.entries + st, (uint32_t)n, part, a.list + st);
+            sort_unit(s, e, (int)m, a.list + st + out);
+            out += m;
+            left -= m;
+            lo = top + 1;
         }
     }
 }
