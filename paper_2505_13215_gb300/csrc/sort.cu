@@ -9,7 +9,7 @@
 // the 8x8-tile super-tiles that its rectangle meets, sorts each super-tile's
 // list by (depth bits, row) on its own (k_cell_count, k_cell_scan,
 // k_cell_scatter, k_unit_sort), and filters it into its tiles' lists in order:
-// the first 512 entries by a saturation head (k_head_count), the rest in
+// the first 512 to 2048 entries by a saturation head (k_head_count), the rest in
 // parallel segments (k_tail_count), the counts turned into ranges by one
 // look-back pass (k_tile_ranges) and the lists written by one pass
 // (k_tile_write).  With culling on, a list holds only the tiles the opacity footprint
@@ -558,7 +558,7 @@ __global__ void __launch_bounds__(256) k_ranges(const uint32_t* keys, const int6
 //                   the sort units: runs of bins of about kUnit / 2 entries
 //   k_cell_scatter  writes each entry (row, key) into its cell, in any order
 //   k_unit_sort     sorts the units in shared memory (sort_unit below): before the
-//                   head count the units that hold the first kHeadEntries of a
+//                   head count the units that hold the head's entries of a
 //                   list, after it the others, of the super-tiles with a list that
 //                   did not end in the head
 //
@@ -581,13 +581,24 @@ constexpr int kSortBuckets = 2048;
 constexpr int kSortBucketBits = 11;
 constexpr uint32_t kCrowded = 48;        // entries in one bucket above which a unit is sorted bitonically
 constexpr uint32_t kWholeUnit = 0xffffffffu;
+constexpr int kRowsPerThread = 2;         // of k_cell_count: 256 kRowsPerThread rows per block
 constexpr int kScatterRounds = 4;         // 32-entry rounds of a warp whose atomics are in flight together
-constexpr int kHeadEntries = 512;        // entries of each list the head pass takes in order
+constexpr int kHeadEntries = 512;        // entries of a list a head CTA takes at a time, in order
+constexpr int kLongList = 4096;          // lists of more entries than this may get kLongHead of them in the head
+constexpr int kLongHead = 2048;
+
+// Entries of a list of n that the head pass may go through before the tail: the
+// certified end of a tile's list can only fall inside them.  What lies past the
+// ends is neither sorted nor counted nor written (figures: k_head_count).
+__host__ __device__ __forceinline__ uint32_t head_reach(uint32_t n, int long_heads)
+{
+    return min(n, (uint32_t)(long_heads && n > (uint32_t)kLongList ? kLongHead : kHeadEntries));
+}
 
 struct CellArgs {
     splat_proj proj;
     int V, bin_bits, nbins;        // nbins = 2^bin_bits depth bins
-    int copies;                    // of the cells (a power of two); block b of a view's rows uses copy b % copies
+    int copies;                    // of the cells (a power of two); a view's b-th run of 512 rows uses copy b % copies
     int64_t n;                     // rows per view
     uint2* range;                  // [V] first depth bits and shift of the views' bins, from k_cell_count
     int super_base[SPLAT_MAX_VIEWS + 1];
@@ -606,6 +617,7 @@ struct CellArgs {
     uint32_t* n_queue;             // [2] their counts (zeroed)
     int64_t queue_cap;
     int total_super;
+    int long_heads;                // head_reach
     int32_t* status;
     int64_t spin_limit;
     // zeroed by k_cell_count (the results of a call that stops early)
@@ -652,16 +664,16 @@ __device__ __forceinline__ uint2 sample_range(const CellArgs& a, int v, uint32_t
     return make_uint2(lo, (uint32_t)min(31, max(0, 32 - __clz(hi - lo) - a.bin_bits)));
 }
 
-// The cells of this block's rows (the same in k_cell_count and k_cell_scatter).
+// The cells of the rows of count block `block` (the same in k_cell_count and k_cell_scatter).
 // Atomics on one cell, and on cells that share a sector, go one after the
 // other; where a batch has few super-tiles, or most rows lie in a few of them,
 // several copies of the cells spread them.
-__device__ __forceinline__ uint32_t* cell_copy(const CellArgs& a)
+__device__ __forceinline__ uint32_t* cell_copy(const CellArgs& a, unsigned block)
 {
-    return a.cell + ((size_t)(blockIdx.x & (a.copies - 1)) * a.total_super << a.bin_bits);
+    return a.cell + ((size_t)(block & (a.copies - 1)) * a.total_super << a.bin_bits);
 }
 
-// One thread per row, blockIdx.y the view.  Each lane walks its own
+// Two rows per thread, blockIdx.y the view.  Each lane walks its own
 // super-rectangle: the reductions return nothing, so a warp only pays issue
 // slots for its widest row (sharing the entries out over the lanes, as the
 // scatter does, costs the same on wide splats and more on small ones).
@@ -670,7 +682,6 @@ __global__ void __launch_bounds__(256) k_cell_count(CellArgs a)
     wait_for_previous_kernel();
     __shared__ uint32_t s_mm[2][8];
     const int v = blockIdx.y;
-    const int64_t i = blockIdx.x * 256ll + threadIdx.x;
     const int64_t gt = ((int64_t)v * gridDim.x + blockIdx.x) * 256 + threadIdx.x;
     for (int64_t t = gt; t < a.total_tiles; t += (int64_t)gridDim.x * gridDim.y * 256) a.ranges[t] = make_uint2(0u, 0u);
     if (gt == 0) {
@@ -678,29 +689,42 @@ __global__ void __launch_bounds__(256) k_cell_count(CellArgs a)
         if (a.n_needed) *a.n_needed = 0;
     }
     if (status_failed(a.status)) return;
-    const uint2 range = sample_range(a, v, s_mm);
-    uint32_t* cells = cell_copy(a);
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.range[v] = range;
-    if (i >= a.n) return;
-    const int64_t r = (int64_t)v * a.n + i;
-    uint32_t pack = 0u, key = 0u;
-    // (all three at once: most rows are visible, and the loads' latency bounds the kernel)
-    const uint32_t nt = a.proj.n_tiles[r];
-    const int4 rc = ((const int4*)a.proj.rect)[r];
-    const float depth = ((const float4*)a.proj.rgb_depth)[r].w;
-    if (nt > 0) {
-        key = __float_as_uint(depth);
-        const int x0 = rc.x >> 3, y0 = rc.y >> 3, x1 = (rc.z + 7) >> 3, y1 = (rc.w + 7) >> 3;
-        if (x1 > x0 && y1 > y0) {
-            pack = (uint32_t)x0 | (uint32_t)y0 << 8 | (uint32_t)x1 << 16 | (uint32_t)y1 << 24;
-            const uint32_t bin = depth_bin(range, a.nbins, key);
-            for (int y = y0; y < y1; ++y) {
-                uint32_t* c = cells + (size_t)(a.super_base[v] + y * a.STX[v]) * a.nbins + bin;
-                for (int x = x0; x < x1; ++x) atomicAdd(c + (size_t)x * a.nbins, 1u);
-            }
+    // (all at once: most rows are visible, and the loads' latency bounds the kernel)
+    uint32_t nt[kRowsPerThread];
+    int4 rc[kRowsPerThread];
+    float depth[kRowsPerThread];
+#pragma unroll
+    for (int q = 0; q < kRowsPerThread; ++q) {
+        const int64_t i = (blockIdx.x * kRowsPerThread + q) * 256ll + threadIdx.x, r = (int64_t)v * a.n + i;
+        nt[q] = 0u;
+        if (i < a.n) {
+            nt[q] = a.proj.n_tiles[r];
+            rc[q] = ((const int4*)a.proj.rect)[r];
+            depth[q] = ((const float4*)a.proj.rgb_depth)[r].w;
         }
     }
-    a.rec[r] = make_uint2(pack, key);
+    const uint2 range = sample_range(a, v, s_mm);
+    uint32_t* cells = cell_copy(a, blockIdx.x);
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.range[v] = range;
+#pragma unroll
+    for (int q = 0; q < kRowsPerThread; ++q) {
+        const int64_t i = (blockIdx.x * kRowsPerThread + q) * 256ll + threadIdx.x;
+        if (i >= a.n) continue;
+        uint32_t pack = 0u, key = 0u;
+        if (nt[q] > 0) {
+            key = __float_as_uint(depth[q]);
+            const int x0 = rc[q].x >> 3, y0 = rc[q].y >> 3, x1 = (rc[q].z + 7) >> 3, y1 = (rc[q].w + 7) >> 3;
+            if (x1 > x0 && y1 > y0) {
+                pack = (uint32_t)x0 | (uint32_t)y0 << 8 | (uint32_t)x1 << 16 | (uint32_t)y1 << 24;
+                const uint32_t bin = depth_bin(range, a.nbins, key);
+                for (int y = y0; y < y1; ++y) {
+                    uint32_t* c = cells + (size_t)(a.super_base[v] + y * a.STX[v]) * a.nbins + bin;
+                    for (int x = x0; x < x1; ++x) atomicAdd(c + (size_t)x * a.nbins, 1u);
+                }
+            }
+        }
+        a.rec[(int64_t)v * a.n + i] = make_uint2(pack, key);
+    }
 }
 
 // First index of the ascending p[0 .. n) with p[index] >= x (n when none).
@@ -820,7 +844,7 @@ __global__ void __launch_bounds__(256) k_cell_scan(CellArgs a)
         const uint32_t u0 = s_p[lower_bound(s_p, a.nbins, k * kUnitStep)];
         const uint32_t u1 = s_p[lower_bound(s_p, a.nbins, (k + 1) * kUnitStep)];
         if (u0 >= u1) continue;  // inside a bin of more than kUnitStep entries
-        const int q = u0 < (uint32_t)kHeadEntries ? 0 : 1;
+        const int q = u0 < head_reach(n, a.long_heads) ? 0 : 1;
         const uint32_t parts = u1 - u0 <= (uint32_t)kUnit ? 1u : (u1 - u0 + kUnitStep - 1) / kUnitStep;
         const uint32_t at = atomicAdd(&a.n_queue[q], parts);
         for (uint32_t g = 0; g < parts; ++g) {
@@ -847,7 +871,7 @@ __global__ void __launch_bounds__(256) k_cell_scatter(CellArgs a)
     // first cell of the row, and of its entries' order in the warp: lane l owns [e, e + c)
     const uint32_t cell0 = (uint32_t)(a.super_base[v] + (int)y0 * a.STX[v] + (int)x0);
     const uint32_t bin = depth_bin(a.range[v], a.nbins, rec.y);
-    uint32_t* cells = cell_copy(a);
+    uint32_t* cells = cell_copy(a, blockIdx.x / kRowsPerThread);
     uint32_t e = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1379,6 +1403,8 @@ struct TileArgs {
     int cull;                         // drop tiles the opacity footprint cannot reach
     int W[SPLAT_MAX_VIEWS], H[SPLAT_MAX_VIEWS];
     uint2* sat_head;                  // [total_super] tiles (bit 8 r + c) whose lists ended in the head
+    uint2* n_head;                    // [total_super] entries the head's two halves (tile rows 0-3, 4-7) went through
+    int long_heads;                   // head_reach
     uint32_t* seg_base;               // [total_super + 1] first tail segment of each super-tile
     uint32_t* seg_super;              // [segments] super-tile of each tail segment
     uint32_t* seg_cnt;                // [segments][64] per-segment tile counts, then offsets
@@ -1459,7 +1485,12 @@ __device__ __forceinline__ uint32_t sat_weight(const SatRow& r, float xlo, float
 
 constexpr int kFilterSeg = 1024;  // list entries per tail segment (one CTA): 32 groups of 32
 
-__device__ __forceinline__ uint32_t head_entries(uint2 rg) { return min(rg.y - rg.x, (uint32_t)kHeadEntries); }
+// First entry (relative to the list) of the tail of a super-tile with open tiles:
+// where the head left its open halves (sat: ended tiles, nh: n_head).
+__device__ __forceinline__ uint32_t tail_start(uint2 sat, uint2 nh)
+{
+    return min(sat.x != 0xffffffffu ? nh.x : 0xffffffffu, sat.y != 0xffffffffu ? nh.y : 0xffffffffu);
+}
 
 // one block of 512 threads (the last of the head count): tail segments per
 // list, exclusive scan -> seg_base
@@ -1471,7 +1502,7 @@ __device__ __forceinline__ void seg_plan(const TileArgs& a, uint32_t* s_tmp)
         uint32_t c = 0;
         if (gs < a.total_super) {  // the tail: what the head pass left, unless every list ended in it
             const uint2 rg = a.sranges[gs], sat = a.sat_head[gs];
-            const uint32_t rest = (sat.x & sat.y) == 0xffffffffu ? 0u : rg.y - rg.x - head_entries(rg);
+            const uint32_t rest = (sat.x & sat.y) == 0xffffffffu ? 0u : rg.y - rg.x - tail_start(sat, a.n_head[gs]);
             c = (rest + kFilterSeg - 1) / kFilterSeg;
         }
         uint32_t tot;
@@ -1677,30 +1708,61 @@ __device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane)
     return x;
 }
 
-// Head pass, counting: the first kHeadEntries entries of each super-tile's list,
-// one CTA per half of the super-tile (four tile rows, 32 tiles), one thread per
-// entry and one warp per group of 32 of them.  A thread finds the tiles of its
-// half that its entry is listed in (a 32-bit mask) and, with culling on, adds
-// the entry's saturation weight in each to the sum of (group, tile) in shared
-// memory.  The warp then transposes its 32 masks, which leaves lane t with
-// tile t's entries: counts are population counts, with no ballot per column.
-// One warp (lane t: tile t) goes through the groups in order, ends tile t's list
-// after the group that takes its sum past the threshold and counts the entries
-// up to there; the groups' words are written with the entries past an end taken
-// out, so that the write pass runs on the words alone.  The last CTA to finish
-// plans the tail segments (seg_plan).
-// Bound by issue and by the entries' gathers.  One CTA per tile row with its
-// entries queued per row and a warp per tile column re-read every entry eight
-// times and evaluated the weights on the few lanes listed in the column: 173 us
-// on 1M Gaussians at 4 x 2704x2028, 50 us on 300k at 4 x 1352x1014.
+// Tile columns (of [tx0, tx0 + 8), as bits) of a tile row that lie wholly inside
+// the footprint: those between its chords at the row's first and last pixel row
+// (the footprint is convex).  Only these can have a saturation weight, which
+// needs every pixel of the tile to pass the alpha skip.
+__device__ __forceinline__ uint32_t inner_columns(const float4& g0, const float4& g1, float ylo, float yhi, int tx0,
+                                                  float xmax_img)
+{
+    const float d0 = g0.y - ylo, d1 = g0.y - yhi;
+    const float q0 = g0.z - g1.w * d0 * d0, q1 = g0.z - g1.w * d1 * d1;
+    if (!(q0 > 0.f && q1 > 0.f)) return 0u;
+    const float s0 = sqrt_approx(q0), s1 = sqrt_approx(q1);
+    const float c0 = g0.x + g1.z * d0, c1 = g0.x + g1.z * d1;  // chord centres
+    const float l = fmaxf(c0 - s0, c1 - s1), r = fminf(c0 + s0, c1 + s1);
+    const float fl = ceilf(l * (1.f / kTile));
+    // the image's last column of tiles ends at its last pixel
+    const float fr = r >= xmax_img ? 1.0e6f : floorf((r - (float)(kTile - 1)) * (1.f / kTile));
+    const int lo = max((int)fminf(fmaxf(fl, -1.f), 1.0e6f) - tx0, 0);
+    const int hi = min((int)fminf(fmaxf(fr, -2.f), 1.0e6f) + 1 - tx0, 8);
+    return hi > lo ? (1u << hi) - (1u << lo) : 0u;
+}
+
+// Head pass, counting: the first entries of each super-tile's list (head_reach),
+// kHeadEntries at a time while one of its tiles is open, one CTA per half of the
+// super-tile (four tile rows, 32 tiles), one thread per entry and one warp per
+// group of 32 of them.  A thread finds the tiles of its half that its entry is
+// listed in (a 32-bit mask) and, with culling on, adds the entry's saturation
+// weight in each to the sum of (group, tile) in shared memory.  The warp then
+// transposes its 32 masks, which leaves lane t with tile t's entries: counts are
+// population counts, with no ballot per column.  One warp (lane t: tile t) goes
+// through the groups in order, ends tile t's list after the group that takes its
+// sum past the threshold and counts the entries up to there; the groups' words
+// are written with the entries past an end taken out, so that the write pass
+// runs on the words alone.  The last CTA to finish plans the tail segments
+// (seg_plan).
+// With long heads a half goes on past its first window while every open tile of
+// it is on its way to close within the reach (one that stays open keeps the tail
+// alive, and a window costs about what three windows of the tail cost); its tail
+// starts where it stopped.  On 1M Gaussians at 4 x 2704x2028 the lists shrink
+// from 87M to 26M instances: head 139 -> 305 us, but the rest of the lists' sort
+// 78 -> 33, tail 259 -> 54, writes 237 -> 85.  Batches of fewer super-tiles than
+// two per SM keep short heads: there the tail's parallel segments are faster.
+// Bound by the entries' gathers (three sectors each) and by issue.  One CTA per
+// tile row with its entries queued per row and a warp per tile column re-read
+// every entry eight times and evaluated the weights on the few lanes listed in
+// the column: 173 us on 1M Gaussians at 4 x 2704x2028, 50 us on 300k at
+// 4 x 1352x1014.
 __global__ void __launch_bounds__(kHeadEntries, 2) k_head_count(TileArgs a)
 {
     wait_for_previous_kernel();
     constexpr int kGroups = kHeadEntries / 32;
     __shared__ uint32_t s_sum[kGroups][32];  // saturation weights of each (group, tile)
     __shared__ uint32_t s_word[kGroups][32];
-    __shared__ int s_cut[32];                // last group of each tile's list
+    __shared__ int s_cut[32];                // last group of each tile's list in this window (-1: ended before it)
     __shared__ uint32_t s_tmp[16];
+    __shared__ bool s_on;                    // the half goes on to another window
     __shared__ bool s_last;
     if (status_failed(a.status)) return;
     const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
@@ -1713,72 +1775,95 @@ __global__ void __launch_bounds__(kHeadEntries, 2) k_head_count(TileArgs a)
     const int TX = a.TX[v], TY = a.TY[v];
     const int ty0 = sy * 8 + 4 * half, tx0 = sx * 8;
     const uint2 rgs = a.sranges[gs];
-    const int n = (int)head_entries(rgs);
+    const int reach = (int)head_reach(rgs.y - rgs.x, a.long_heads);
+    const float xmax_img = (float)(a.W[v] - 1), ymax_img = (float)(a.H[v] - 1);
+    // warp 0, lane t: the state of tile t of the half
+    const int ty = ty0 + (lane >> 3), tx = tx0 + (lane & 7);
+    const bool in = ty < TY && tx < TX;
+    uint32_t cnt = 0u, sum = 0u;
+    bool ended = !in;  // tiles outside the grid count as ended
     s_sum[g][lane] = 0u;
     __syncthreads();
-    uint32_t m = 0u;
-    if (tid < n) {
-        const uint32_t row = a.list[rgs.x + tid];
-        const int4 rc = ((const int4*)a.proj.rect)[row];
-        const float2 xy = ((const float2*)a.proj.xy)[row];
-        const float4 co = ((const float4*)a.proj.conic_opacity)[row];
-        const int x0 = max(rc.x - tx0, 0), x1 = min(rc.z - tx0, 8);
-        const int y0 = max(rc.y - ty0, 0), y1 = min(rc.w - ty0, 4);
-        if (x0 < x1 && y0 < y1) {
-            float4 g0, g1;
-            if (a.cull) footprint(xy, co, g0, g1);
-            // the saturation bound needs a*c - b^2 >= 1e-3 a c: the relative
-            // rounding of the power stays far below its size
-            const bool sat_ok = a.cull && co.x > 0.f && co.z > 0.f &&
-                                co.x * co.z - co.y * co.y >= 1e-3f * co.x * co.z && co.w <= 1.f && co.w > 0.f;
-            const float xmax_img = (float)(a.W[v] - 1), ymax_img = (float)(a.H[v] - 1);
-            for (int r = y0; r < y1; ++r) {
-                const float vlo = (float)((ty0 + r) * kTile);
-                const uint32_t cols = row_columns(x0, x1, tx0, vlo, g0, g1, a.cull);
-                m |= cols << (8 * r);
-                if (sat_ok && cols) {
-                    const SatRow sr = sat_row(co, xy.x, xy.y, vlo, fminf(vlo + (float)(kTile - 1), ymax_img));
-                    for (uint32_t left = cols; left; left &= left - 1) {
-                        const int c = __ffs(left) - 1;
-                        const float xlo = (float)((tx0 + c) * kTile);
-                        const uint32_t wt = sat_weight(sr, xlo, fminf(xlo + (float)(kTile - 1), xmax_img));
-                        if (wt) atomicAdd(&s_sum[g][8 * r + c], wt);
+    int w0 = 0;
+    while (w0 < reach) {
+        const int n = min(reach - w0, kHeadEntries);
+        uint32_t m = 0u;
+        if (tid < n) {
+            const uint32_t row = a.list[rgs.x + w0 + tid];
+            const int4 rc = ((const int4*)a.proj.rect)[row];
+            const float2 xy = ((const float2*)a.proj.xy)[row];
+            const float4 co = ((const float4*)a.proj.conic_opacity)[row];
+            const int x0 = max(rc.x - tx0, 0), x1 = min(rc.z - tx0, 8);
+            const int y0 = max(rc.y - ty0, 0), y1 = min(rc.w - ty0, 4);
+            if (x0 < x1 && y0 < y1) {
+                float4 g0, g1;
+                if (a.cull) footprint(xy, co, g0, g1);
+                // the saturation bound needs a*c - b^2 >= 1e-3 a c: the relative
+                // rounding of the power stays far below its size
+                const bool sat_ok = a.cull && co.x > 0.f && co.z > 0.f &&
+                                    co.x * co.z - co.y * co.y >= 1e-3f * co.x * co.z && co.w <= 1.f && co.w > 0.f;
+                for (int r = y0; r < y1; ++r) {
+                    const float vlo = (float)((ty0 + r) * kTile), vhi = fminf(vlo + (float)(kTile - 1), ymax_img);
+                    const uint32_t cols = row_columns(x0, x1, tx0, vlo, g0, g1, a.cull);
+                    m |= cols << (8 * r);
+                    uint32_t left = sat_ok ? cols & inner_columns(g0, g1, vlo, vhi, tx0, xmax_img) : 0u;
+                    if (left) {
+                        const SatRow sr = sat_row(co, xy.x, xy.y, vlo, vhi);
+                        for (; left; left &= left - 1) {
+                            const int c = __ffs(left) - 1;
+                            const float xlo = (float)((tx0 + c) * kTile);
+                            const uint32_t wt = sat_weight(sr, xlo, fminf(xlo + (float)(kTile - 1), xmax_img));
+                            if (wt) atomicAdd(&s_sum[g][8 * r + c], wt);
+                        }
                     }
                 }
             }
         }
-    }
-    __syncwarp();
-    const uint32_t word = warp_transpose(m, lane);
-    s_word[g][lane] = word;
-    __syncthreads();
-    if (g == 0) {
-        const int ty = ty0 + (lane >> 3), tx = tx0 + (lane & 7);
-        const bool in = ty < TY && tx < TX;
-        uint32_t cnt = 0u, sum = 0u;
-        int cut = kGroups;
+        __syncwarp();
+        const uint32_t word = warp_transpose(m, lane);
+        s_word[g][lane] = word;
+        __syncthreads();
+        if (g == 0) {
+            int cut = ended ? -1 : kGroups;
 #pragma unroll
-        for (int q = 0; q < kGroups; ++q) {
-            if (q <= cut) {
-                cnt += __popc(s_word[q][lane]);
-                sum += s_sum[q][lane];
-                if (sum >= kSatThreshold) cut = min(cut, q);  // the list ends after this group
+            for (int q = 0; q < kGroups; ++q) {
+                if (q <= cut) {
+                    cnt += __popc(s_word[q][lane]);
+                    sum += s_sum[q][lane];
+                    if (sum >= kSatThreshold) cut = min(cut, q);  // the list ends after this group
+                }
+                s_sum[q][lane] = 0u;
             }
+            s_cut[lane] = cut;
+            ended = cut < kGroups;
+            // on its way: a quarter above the threshold by the end of the reach, at the mean rate so far (weights
+            // fall with the depth)
+            const bool good = ended || 4ull * sum * (unsigned)reach >= 5ull * kSatThreshold * (unsigned)(w0 + n);
+            const bool open = __any_sync(0xffffffffu, !ended), all_good = __all_sync(0xffffffffu, good);
+            if (lane == 0) s_on = open && all_good;
         }
-        s_cut[lane] = cut;
+        __syncthreads();
+        if (32 * g < n) {  // warp-uniform
+            const bool open = g <= s_cut[lane];
+            const uint32_t allowed = __ballot_sync(0xffffffffu, open);
+            uint32_t* out = reinterpret_cast<uint32_t*>(a.mask + rgs.x + w0 + 32 * g);
+            if (32 * g + 32 <= n) out[32 * half + lane] = open ? word : 0u;
+            else if (tid < n) out[2 * lane + half] = m & allowed;
+        }
+        w0 += n;
+        if (w0 >= reach || !s_on) break;  // block-uniform
+        __syncthreads();  // s_on, s_cut and s_word are rewritten by the next window
+    }
+    if (g == 0) {
         if (in) a.tile_total[a.tile_base[v] + ty * TX + tx] = cnt;
-        // columns outside the grid count as ended
-        const uint32_t sat = __ballot_sync(0xffffffffu, !in || cut < kGroups);
-        if (lane == 0) reinterpret_cast<uint32_t*>(a.sat_head + gs)[half] = sat;
+        const uint32_t sat = __ballot_sync(0xffffffffu, ended);
+        if (lane == 0) {
+            reinterpret_cast<uint32_t*>(a.sat_head + gs)[half] = sat;
+            reinterpret_cast<uint32_t*>(a.n_head + gs)[half] = (uint32_t)w0;
+        }
+        __syncwarp();
     }
     __syncthreads();
-    if (32 * g < n) {  // warp-uniform
-        const bool open = g <= s_cut[lane];
-        const uint32_t allowed = __ballot_sync(0xffffffffu, open);
-        uint32_t* out = reinterpret_cast<uint32_t*>(a.mask + rgs.x + 32 * g);
-        if (32 * g + 32 <= n) out[32 * half + lane] = open ? word : 0u;
-        else if (tid < n) out[2 * lane + half] = m & allowed;
-    }
     if (tid == 0) {  // the last CTA to finish plans the tail from every CTA's results
         __threadfence();
         s_last = atomicAdd(a.ticket + 2, 1u) == gridDim.x - 1;
@@ -1821,12 +1906,14 @@ __global__ void __launch_bounds__(256) k_tail_count(TileArgs a)
         const int ls = gs - a.super_base[v];
         const int sy = ls / a.STX[v], sx = ls - sy * a.STX[v];
         const int ty0 = sy * 8, tx0 = sx * 8;
-        const uint2 rgs = a.sranges[gs], sat = a.sat_head[gs];
-        const uint32_t b0 = rgs.x + head_entries(rgs) + (g - a.seg_base[gs]) * kFilterSeg;
+        const uint2 rgs = a.sranges[gs], sat = a.sat_head[gs], nh = a.n_head[gs];
+        const uint32_t r0 = tail_start(sat, nh) + (g - a.seg_base[gs]) * kFilterSeg, b0 = rgs.x + r0;
         const int n = (int)min((uint32_t)kFilterSeg, rgs.y - b0);
         uint32_t c0 = 0u, c1 = 0u;  // entries listed in tiles lane and lane + 32
         for (int q = 32 * warp; q < n; q += 256) {  // warp-uniform
             const int e = q + lane;
+            // (warp-uniform) whether each half is open and past its head: the words of a half's head stay as they are
+            const bool h0 = sat.x != 0xffffffffu && r0 + q >= nh.x, h1 = sat.y != 0xffffffffu && r0 + q >= nh.y;
             uint32_t m0 = 0u, m1 = 0u;
             if (e < n) {
                 const uint32_t row = a.list[b0 + e];
@@ -1834,7 +1921,7 @@ __global__ void __launch_bounds__(256) k_tail_count(TileArgs a)
                 const float2 xy = ((const float2*)a.proj.xy)[row];
                 const float4 co = ((const float4*)a.proj.conic_opacity)[row];
                 const int x0 = max(rc.x - tx0, 0), x1 = min(rc.z - tx0, 8);
-                const int y0 = max(rc.y - ty0, 0), y1 = min(rc.w - ty0, 8);
+                const int y0 = max(rc.y - ty0, h0 ? 0 : 4), y1 = min(rc.w - ty0, h1 ? 8 : 4);
                 if (x0 < x1 && y0 < y1) {
                     float4 g0, g1;
                     if (a.cull) footprint(xy, co, g0, g1);
@@ -1853,10 +1940,11 @@ __global__ void __launch_bounds__(256) k_tail_count(TileArgs a)
             c1 += __popc(t1);
             if (q + 32 <= n) {
                 uint32_t* out = reinterpret_cast<uint32_t*>(a.mask + b0 + q);
-                out[lane] = t0;
-                out[32 + lane] = t1;
+                if (h0) out[lane] = t0;
+                if (h1) out[32 + lane] = t1;
             } else if (e < n) {
-                a.mask[b0 + e] = make_uint2(m0, m1);
+                if (h0) a.mask[b0 + e].x = m0;
+                if (h1) a.mask[b0 + e].y = m1;
             }
         }
         s_cnt[warp][lane] = c0;
@@ -1914,86 +2002,100 @@ __global__ void __launch_bounds__(256) k_tile_write(TileArgs a)
         const int sy = ls / a.STX[v], sx = ls - sy * a.STX[v];
         const int TX = a.TX[v], TY = a.TY[v];
         const int ty = sy * 8 + warp, tx0 = sx * 8;
-        const uint2 rgs = a.sranges[gs];
-        uint32_t b0 = rgs.x;
-        int n = (int)head_entries(rgs);
-        if (!head) {
-            b0 += n + (tk - nhead - a.seg_base[gs]) * kFilterSeg;
-            n = (int)min((uint32_t)kFilterSeg, rgs.y - b0);
+        const uint2 rgs = a.sranges[gs], sat = a.sat_head[gs], nh = a.n_head[gs];
+        const bool open = (warp < 4 ? sat.x : sat.y) != 0xffffffffu;  // this warp's half has a tail
+        const uint32_t my_head = warp < 4 ? nh.x : nh.y;
+        uint32_t b0 = rgs.x, b1, from, to;  // the item's entries [b0, b1), of which this warp's are [from, to)
+        if (head) {  // each half of the super-tile up to where its head stopped
+            b1 = b0 + max(nh.x, nh.y);
+            from = b0;
+            to = b0 + my_head;
+        } else {
+            b0 += tail_start(sat, nh) + (tk - nhead - a.seg_base[gs]) * kFilterSeg;
+            b1 = min(b0 + (uint32_t)kFilterSeg, rgs.y);
+            from = max(b0, rgs.x + my_head);  // (whole groups: heads stop at multiples of kHeadEntries)
+            to = open ? b1 : b0;
         }
-        for (int i = tid; i < n; i += 256) s_row[i] = a.list[b0 + i];
-        __syncthreads();
-        if (ty < TY && n > 0) {  // warp-uniform
-            const int full = n >> 5, part = n & 31, groups = full + (part ? 1 : 0);
-            uint32_t word[8], first[8];
+        uint32_t first[8];  // next slot of each tile's list
 #pragma unroll
-            for (int k = 0; k < 8; ++k) word[k] = 0u;
-            if (lane < full) {
-                const uint2* p = a.mask + b0 + 32 * lane + 4 * warp;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint2 t = p[k];
-                    word[2 * k] = t.x;
-                    word[2 * k + 1] = t.y;
-                }
+        for (int k = 0; k < 8; ++k) {
+            first[k] = 0u;
+            if (ty < TY && tx0 + k < TX) {
+                const int tile = a.tile_base[v] + ty * TX + tx0 + k;
+                first[k] = head ? a.ranges[tile].x
+                                : a.tile_total[tile] + a.seg_cnt[(size_t)(tk - nhead) * 64 + 8 * warp + k];
             }
-            if (part) {  // the last group keeps a word pair per entry
-                uint32_t byte = 0u;
-                if (lane < part) {
-                    const uint2 t = a.mask[b0 + 32 * full + lane];
-                    byte = (warp < 4 ? t.x >> (8 * warp) : t.y >> (8 * (warp - 4))) & 0xffu;
+        }
+        for (; b0 < b1; b0 += kFilterSeg) {
+            const int rows = (int)min((uint32_t)kFilterSeg, b1 - b0);
+            for (int i = tid; i < rows; i += 256) s_row[i] = a.list[b0 + i];
+            __syncthreads();
+            const int n = to > max(b0, from) ? (int)min((uint32_t)kFilterSeg, to - b0) : 0;
+            const int skip = from > b0 ? (int)(from - b0) >> 5 : 0;  // groups of the half's head
+            if (ty < TY && n > 0) {  // warp-uniform
+                const int full = n >> 5, part = n & 31, groups = full + (part ? 1 : 0);
+                uint32_t word[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) word[k] = 0u;
+                if (lane >= skip && lane < full) {
+                    const uint2* p = a.mask + b0 + 32 * lane + 4 * warp;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint2 t = p[k];
+                        word[2 * k] = t.x;
+                        word[2 * k + 1] = t.y;
+                    }
+                }
+                if (part && full >= skip) {  // the last group keeps a word pair per entry
+                    uint32_t byte = 0u;
+                    if (lane < part) {
+                        const uint2 t = a.mask[b0 + 32 * full + lane];
+                        byte = (warp < 4 ? t.x >> (8 * warp) : t.y >> (8 * (warp - 4))) & 0xffu;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const uint32_t bal = __ballot_sync(0xffffffffu, (byte >> k) & 1u);
+                        if (lane == full) word[k] = bal;
+                    }
                 }
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const uint32_t bal = __ballot_sync(0xffffffffu, (byte >> k) & 1u);
-                    if (lane == full) word[k] = bal;
-                }
-            }
+                    uint32_t w = word[k];
+                    const uint32_t c = __popc(w);
+                    uint32_t at = c;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                first[k] = 0u;
-                if (tx0 + k < TX) {
-                    const int tile = a.tile_base[v] + ty * TX + tx0 + k;
-                    first[k] = head ? a.ranges[tile].x
-                                    : a.tile_total[tile] + a.seg_cnt[(size_t)(tk - nhead) * 64 + 8 * warp + k];
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                uint32_t w = word[k];
-                const uint32_t c = __popc(w);
-                uint32_t at = c;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t y = __shfl_up_sync(0xffffffffu, at, o);
-                    if (lane >= o) at += y;
-                }
-                const uint32_t total = __shfl_sync(0xffffffffu, at, 31);
-                at -= c;
-                if (total == 0u) continue;  // warp-uniform
-                uint32_t* out = a.vals_out + first[k];
-                if (total <= (uint32_t)(kSparse * groups)) {
-                    while (w) {
-                        const int e = __ffs(w) - 1;
-                        w &= w - 1;
-                        s_buf[warp][at++] = s_row[32 * lane + e];
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t y = __shfl_up_sync(0xffffffffu, at, o);
+                        if (lane >= o) at += y;
                     }
-                    __syncwarp();
-                    for (uint32_t i = lane; i < total; i += 32) out[i] = s_buf[warp][i];
-                    __syncwarp();
-                } else {
-                    for (int q = 0; q < groups; ++q) {
-                        const uint32_t gw = __shfl_sync(0xffffffffu, w, q), ga = __shfl_sync(0xffffffffu, at, q);
-                        if ((gw >> lane) & 1u) out[ga + __popc(gw & lt)] = s_row[32 * q + lane];
+                    const uint32_t total = __shfl_sync(0xffffffffu, at, 31);
+                    at -= c;
+                    if (total == 0u) continue;  // warp-uniform
+                    uint32_t* out = a.vals_out + first[k];
+                    if (total <= (uint32_t)(kSparse * groups)) {
+                        while (w) {
+                            const int e = __ffs(w) - 1;
+                            w &= w - 1;
+                            s_buf[warp][at++] = s_row[32 * lane + e];
+                        }
+                        __syncwarp();
+                        for (uint32_t i = lane; i < total; i += 32) out[i] = s_buf[warp][i];
+                        __syncwarp();
+                    } else {
+                        for (int q = 0; q < groups; ++q) {
+                            const uint32_t gw = __shfl_sync(0xffffffffu, w, q), ga = __shfl_sync(0xffffffffu, at, q);
+                            if ((gw >> lane) & 1u) out[ga + __popc(gw & lt)] = s_row[32 * q + lane];
+                        }
                     }
-                }
-                if (a.keys_out) {
-                    const uint32_t tile = (uint32_t)(a.tile_base[v] + ty * TX + tx0 + k);
-                    for (uint32_t i = lane; i < total; i += 32) a.keys_out[first[k] + i] = tile;
+                    if (a.keys_out) {
+                        const uint32_t tile = (uint32_t)(a.tile_base[v] + ty * TX + tx0 + k);
+                        for (uint32_t i = lane; i < total; i += 32) a.keys_out[first[k] + i] = tile;
+                    }
+                    first[k] += total;
                 }
             }
+            __syncthreads();
         }
-        __syncthreads();
     }
 }
 
@@ -2015,7 +2117,7 @@ struct SortLayout {
     int bin_bits, copies;
     int64_t queue_cap;
     size_t off_rec, off_range, off_cell, off_cell_lb, off_queue, off_nqueue, off_rlb, off_total, off_vals1, off_sranges,
-        off_ninst1, off_segbase, off_segcnt, off_segsuper, off_sathead, off_mask;
+        off_ninst1, off_segbase, off_segcnt, off_segsuper, off_sathead, off_nhead, off_mask;
     // both
     size_t off_tord, off_tickets, zero_begin, zero_end;
     size_t bytes;
@@ -2115,6 +2217,7 @@ SortLayout sort_layout(int64_t n_rows, int64_t capacity, int V, const int* TX, c
         L.off_segcnt = take(4 * 64 * (size_t)L.max_segs);
         L.off_segsuper = take(4 * (size_t)L.max_segs);
         L.off_sathead = take(8 * (size_t)std::max<int64_t>(L.total_super, 1));
+        L.off_nhead = take(8 * (size_t)std::max<int64_t>(L.total_super, 1));
         L.off_mask = take(8 * (size_t)capacity);  // the unsorted entries, then the coverage words
         L.off_rec = take(8 * (size_t)n_rows);
         L.off_range = take(8 * (size_t)std::max(V, 1));
@@ -2216,6 +2319,7 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         // 1. the super-tile lists, unsorted inside their cells.  The lists (K1 entries) live in a
         // capacity-sized buffer, so K1 is checked by the scan, before anything is written (K itself is
         // checked by the tile ranges once the tile lists are counted)
+        const int long_heads = sb >= 2 * ctx.num_sms;  // (see k_head_count)
         CellArgs c{};
         c.proj = proj;
         c.V = vb.V;
@@ -2238,17 +2342,18 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         c.n_queue = U(L.off_nqueue);
         c.queue_cap = L.queue_cap;
         c.total_super = sb;
+        c.long_heads = long_heads;
         c.status = status;
         c.spin_limit = ctx.spin_limit;
         c.ranges = (uint2*)bins.ranges;
         c.total_tiles = vb.total_tiles;
         c.n_instances = bins.n_instances;
         c.n_needed = bins.n_needed;
-        const dim3 row_grid((unsigned)((proj.n + 255) / 256), (unsigned)vb.V);
+        auto row_grid = [&](int rows) { return dim3((unsigned)((proj.n + rows - 1) / rows), (unsigned)vb.V); };
         count_launch(3);
-        launch_kernel(k_cell_count, row_grid, 256, 0, s, c);
+        launch_kernel(k_cell_count, row_grid(256 * kRowsPerThread), 256, 0, s, c);
         launch_kernel(k_cell_scan, sb, 256, 0, s, c);
-        launch_kernel(k_cell_scatter, row_grid, 256, 0, s, c);
+        launch_kernel(k_cell_scatter, row_grid(256), 256, 0, s, c);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         // 2. the units of each list that the head pass takes, in order
         SortArgs u{};
@@ -2297,6 +2402,8 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         t.seg_cnt = U(L.off_segcnt);
         t.seg_super = U(L.off_segsuper);
         t.sat_head = (uint2*)(w + L.off_sathead);
+        t.n_head = (uint2*)(w + L.off_nhead);
+        t.long_heads = long_heads;
         t.mask = (uint2*)(w + L.off_mask);
         t.ticket = tickets + 1;
         TileRangeArgs tr{};
