@@ -111,16 +111,58 @@ __device__ __forceinline__ void sh_accumulate(const float c[48], float w, const 
     }
 }
 
+// A warp's SH rows in shared memory: 32 rows of 48 FP32 values at a stride of 13
+// 16-byte units (no bank conflicts).  A lane that reads or writes its own row in
+// global memory touches 32 lines with every 16 bytes.
+// The projection reads the rows (block 0) again for every view: L1 at 85% bound it
+// (V = 8, 500k Gaussians: 108 us).  The warp copies its 32 rows together instead: 82
+// us; V = 2, 1M: 80 -> 67.  V = 1 reads a row once and wants L1 for it (300k: 16.5 us
+// direct, 18 staged) and 16-bit rows are half as long (staged: V = 1 33 -> 42 us, V = 4
+// 81 -> 89 at 1M): these stay with direct loads.
+constexpr int kShStride = 208;
+constexpr int kProjectThreads = 128;
+
+__host__ __device__ constexpr int slice_project_smem(int dtype, int V)
+{
+    return dtype == SPLAT_F32 && V > 1 ? kProjectThreads * kShStride : 0;
+}
+
+// Starts the copy of block 0 of Gaussians i0 .. i0 + 31 to buf.
+__device__ __forceinline__ void stage_sh_rows(unsigned char* buf, const splat_g3& g3, const splat_g4& g4, int64_t i0,
+                                              int64_t N, int lane)
+{
+    for (int c = lane; c < 32 * 12; c += 32) {
+        const int r = c / 12, part = c - 12 * r;
+        const int64_t i = i0 + r;
+        if (i < N) {
+            const char* row = i < g4.n ? (const char*)g4.sh + i * 192 * (g4.sh_time + 1)
+                                       : (const char*)g3.sh + (i - g4.n) * 192;
+            cp_async16(buf + r * kShStride + 16 * part, row + 16 * part);
+        }
+    }
+    cp_async_commit();
+}
+
 // rgb = 0.5 + sum_{n=0..T} cos(2 pi n t) sum_k c_nk Y_k(d) (unclamped); T = 0: plain SH.
-// Y receives the SH basis at d, c0 the coefficients of block 0.
+// sh0: block 0 of the coefficients in shared memory, if it was staged.
 template <int DT>
-__device__ __forceinline__ void sh_rgb(const void* sh_base, int64_t row, int T, float t, const float dir[3],
-                                       float rgb[3], float Y[16], float c0[48])
+__device__ __forceinline__ void sh_rgb(const unsigned char* sh0, const void* sh_base, int64_t row, int T, float t,
+                                       const float dir[3], float rgb[3])
 {
     using S = Storage<DT>;
+    float Y[16], c0[48];
     sh_basis(dir[0], dir[1], dir[2], Y);
     const typename S::T* p = (const typename S::T*)sh_base + row * 48 * (T + 1);
-    load_sh48<DT>(p, c0);
+    if constexpr (DT == SPLAT_F32) {
+        const float4* c4 = sh0 ? (const float4*)sh0 : (const float4*)p;  // plain loads: either space
+#pragma unroll
+        for (int q = 0; q < 12; ++q) {
+            const float4 v = c4[q];
+            c0[4 * q + 0] = v.x; c0[4 * q + 1] = v.y; c0[4 * q + 2] = v.z; c0[4 * q + 3] = v.w;
+        }
+    } else {
+        load_sh48<DT>(p, c0);
+    }
     float r = 0.5f, g = 0.5f, b = 0.5f;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {  // block 0 (weight 1): exactly the plain SH sum
@@ -264,16 +306,31 @@ __device__ __forceinline__ void at_time(const Geo& G, bool is4, float t, float m
 }
 
 template <int DT>
-__global__ void __launch_bounds__(128, 7) k_slice_project(splat_g3 g3, splat_g4 g4, ViewBatch vb, splat_proj out,
+__global__ void __launch_bounds__(kProjectThreads, 7) k_slice_project(splat_g3 g3, splat_g4 g4, ViewBatch vb, splat_proj out,
                                                        int32_t* status)
 {
+    // rows are staged if the launch brought room for them (slice_project_smem)
+    extern __shared__ __align__(16) unsigned char s_rows[];
+    const bool staged = DT == SPLAT_F32 && slice_project_smem(DT, vb.V) > 0;
     wait_for_previous_kernel();
     const int64_t N = out.n;
     const int64_t n4 = g4.n;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned char* sh0 = s_rows + warp * 32 * kShStride;
+    for (int64_t wb = blockIdx.x * (int64_t)blockDim.x + 32 * warp; wb < N; wb += (int64_t)gridDim.x * blockDim.x) {
+        if (staged) {
+            __syncwarp();  // the last trip's rows have been read
+            stage_sh_rows(sh0, g3, g4, wb, N, lane);
+        }
+        const int64_t i = wb + lane;
         const bool is4 = i < n4;
         Geo G;
-        load_geo<DT>(g3, g4, i, is4, G);
+        if (i < N) load_geo<DT>(g3, g4, i, is4, G);
+        if (staged) {
+            cp_async_wait_all();
+            __syncwarp();
+        }
+        if (i >= N) continue;
         const void* sh_base = is4 ? g4.sh : g3.sh;
         const int64_t sh_row = is4 ? i : i - n4;
         // non-finite parameters: reported (row of the first view) and the Gaussian culled
@@ -333,8 +390,9 @@ __global__ void __launch_bounds__(128, 7) k_slice_project(splat_g3 g3, splat_g4 
                         float d[3] = {mu[0] - vp.cam[0], mu[1] - vp.cam[1], mu[2] - vp.cam[2]};
                         const float id = rsqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
                         d[0] *= id; d[1] *= id; d[2] *= id;
-                        float rgb[3], Y[16], c0[48];
-                        sh_rgb<DT>(sh_base, sh_row, is4 ? g4.sh_time : 0, vp.t, d, rgb, Y, c0);
+                        float rgb[3];
+                        sh_rgb<DT>(staged ? sh0 + lane * kShStride : nullptr, sh_base, sh_row,
+                                   is4 ? g4.sh_time : 0, vp.t, d, rgb);
                         rd = make_float4(fmaxf(rgb[0], 0.f), fmaxf(rgb[1], 0.f), fmaxf(rgb[2], 0.f), e.z);
                         if (!isfinite(rgb[0] + rgb[1] + rgb[2])) {  // non-finite colour coefficients
                             set_status(status, SPLAT_ERR_NONFINITE, SPLAT_STAGE_SLICE_PROJECT, row);
@@ -445,6 +503,13 @@ __device__ __forceinline__ void normalise_backward(const float q[4], const float
     for (int k = 0; k < 4; ++k) out[k] = (g[k] - qn[k] * dot) * in;
 }
 
+// Blocks per SM.  Six leave 80 registers a thread and spill 72 to 116 bytes, five 96
+// and none.  L = 1 (V = 1): six 36 and 144 us, five 34 and 130 us (300k BF16, 1M FP16).
+// FP32, L > 1: six 208 and 139 us, five 197 and 131 us (V = 8, 500k; V = 2, 1M).  16-bit
+// storage with L > 1 spills less and waits more: six 53, 165 and 160 us, five 60, 193
+// and 171 us (V = 4, 300k; V = 16, 200k; V = 4, 1M).
+__host__ __device__ constexpr int adjoint_blocks(int DT, int L) { return L == 1 || DT == SPLAT_F32 ? 5 : 6; }
+
 constexpr int kAdjThreads = 128;  // threads per block of the adjoint
 
 // One lane's share of the colour gradient, staged for its group: the view's
@@ -469,7 +534,7 @@ struct ShPart {
 // gradients.  No atomics; the views' memory requests are independent of one
 // another, and the heavy view-independent chain runs on full warps.
 template <int DT, int L>
-__global__ void __launch_bounds__(kAdjThreads, 6) k_adjoint(splat_g3 g3, splat_g4 g4, ViewBatch vb, splat_proj proj,
+__global__ void __launch_bounds__(kAdjThreads, adjoint_blocks(DT, L)) k_adjoint(splat_g3 g3, splat_g4 g4, ViewBatch vb, splat_proj proj,
                                                  const float* __restrict__ dproj, splat_grads3 dg3,
                                                  splat_grads4 dg4, int32_t* status)
 {
@@ -477,7 +542,12 @@ __global__ void __launch_bounds__(kAdjThreads, 6) k_adjoint(splat_g3 g3, splat_g
     static_assert(L == 1 || L == 2 || L == 4 || L == 8 || L == 16, "lanes per Gaussian");
     constexpr int KPL = 16 / L;  // SH functions whose gradient a lane writes
     constexpr int GPS = 32 / L;  // Gaussians per sub-batch of a warp
-    __shared__ ShPart s_part[kAdjThreads];
+    __shared__ ShPart s_part[L > 1 ? kAdjThreads : 1];
+    // L = 1: every lane has a gradient row of its own, and the warp writes them together
+    // through shared memory (kShStride; 1M: 97 -> 91 us BF16, 130 -> 108 us FP16 with
+    // time blocks; 300k FP32 43 -> 44).  With L > 1 the lanes of a group share a row,
+    // and staging it measured slower (V = 8 212 -> 227 us, V = 4 164 -> 183).
+    __shared__ __align__(16) unsigned char s_sh[kAdjThreads / 32][L == 1 ? 32 * kShStride : 16];
     __shared__ float s_sum[kAdjThreads / 32][15][32];  // per warp: the 15 view sums of its 32 Gaussians
     __shared__ float s_geo[kAdjThreads / 32][15][32];  // per warp: the view-independent geometry (Geo)
     __shared__ ViewParams s_view[SPLAT_MAX_VIEWS];  // lanes of one warp read different views
@@ -588,19 +658,19 @@ __global__ void __launch_bounds__(kAdjThreads, 6) k_adjoint(splat_g3 g3, splat_g
                 add(gal); add(gp_dt); add(gp_dt2);
             }
         }
-        s_part[threadIdx.x] = part;
+        if (L > 1) s_part[threadIdx.x] = part;
         __syncwarp();
-        if (valid) {
-            // SH gradient of functions k0 .. k0 + KPL - 1, every time block
-            const int k0 = q * KPL;
-            float* shrow = (is4 ? dg4.sh + i * (Tn + 1) * 48 : dg3.sh + (i - n4) * 48) + 3 * k0;
-            for (int n = 0; n <= Tn; ++n) {
-                float acc[3 * KPL];
+        // SH gradient of functions k0 .. k0 + KPL - 1, every time block
+        const int k0 = q * KPL;
+        const int blocks = L > 1 ? (valid ? Tn + 1 : 0) : (c0 < n4 ? g4.sh_time + 1 : 1);  // L = 1: warp-uniform
+        for (int n = 0; n < blocks; ++n) {
+            float acc[3 * KPL];
 #pragma unroll
-                for (int e = 0; e < 3 * KPL; ++e) acc[e] = 0.f;
+            for (int e = 0; e < 3 * KPL; ++e) acc[e] = 0.f;
+            if (L > 1 || (valid && n <= Tn)) {
 #pragma unroll
                 for (int j = 0; j < L; ++j) {
-                    const ShPart& pj = s_part[gbase + j];
+                    const ShPart& pj = L > 1 ? s_part[L > 1 ? gbase + j : 0] : part;
                     const float4 g = pj.gct;
                     const float tw = n == 0 ? 1.f : time_weight(n, g.w);
                     const float gr = tw * g.x, gg = tw * g.y, gb = tw * g.z;
@@ -614,7 +684,25 @@ __global__ void __launch_bounds__(kAdjThreads, 6) k_adjoint(splat_g3 g3, splat_g
                         acc[3 * kk + 2] += gb * y;
                     }
                 }
-                float* out = shrow + n * 48;
+            }
+            if constexpr (L == 1) {  // the warp's rows together
+                unsigned char* shbuf = s_sh[warp];
+                float4* mine = (float4*)(shbuf + lane * kShStride);
+#pragma unroll
+                for (int e = 0; e < 12; ++e)
+                    mine[e] = make_float4(acc[4 * e], acc[4 * e + 1], acc[4 * e + 2], acc[4 * e + 3]);
+                __syncwarp();
+                for (int c = lane; c < 32 * 12; c += 32) {
+                    const int r = c / 12, w = c - 12 * r;
+                    const int64_t gi = c0 + r;
+                    if (gi < N && (n == 0 || gi < n4)) {
+                        float* row = gi < n4 ? dg4.sh + (gi * (g4.sh_time + 1) + n) * 48 : dg3.sh + (gi - n4) * 48;
+                        ((float4*)row)[w] = *(const float4*)(shbuf + r * kShStride + 16 * w);
+                    }
+                }
+                __syncwarp();
+            } else {
+                float* out = (is4 ? dg4.sh + i * (Tn + 1) * 48 : dg3.sh + (i - n4) * 48) + 3 * k0 + n * 48;
                 if constexpr ((3 * KPL) % 4 == 0) {
 #pragma unroll
                     for (int e = 0; e < 3 * KPL; e += 4)
@@ -812,14 +900,20 @@ cudaError_t launch_slice_project(const splat_g3& g3, const splat_g4& g4, const V
 {
     const int64_t N = out.n;
     if (N == 0) return cudaSuccess;
-    const int threads = 128;
+    const int threads = kProjectThreads, smem = slice_project_smem(dtype, vb.V);
     const int64_t want = (N + threads - 1) / threads;
     const int blocks = (int)(want < (int64_t)ctx.num_sms * 64 ? want : (int64_t)ctx.num_sms * 64);
     count_launch();
     switch (dtype) {
-    case SPLAT_F32: launch_kernel(k_slice_project<SPLAT_F32>, blocks, threads, 0, ctx.stream, g3, g4, vb, out, status); break;
-    case SPLAT_BF16: launch_kernel(k_slice_project<SPLAT_BF16>, blocks, threads, 0, ctx.stream, g3, g4, vb, out, status); break;
-    default: launch_kernel(k_slice_project<SPLAT_F16>, blocks, threads, 0, ctx.stream, g3, g4, vb, out, status); break;
+    case SPLAT_F32:
+        launch_kernel(k_slice_project<SPLAT_F32>, blocks, threads, smem, ctx.stream, g3, g4, vb, out, status);
+        break;
+    case SPLAT_BF16:
+        launch_kernel(k_slice_project<SPLAT_BF16>, blocks, threads, smem, ctx.stream, g3, g4, vb, out, status);
+        break;
+    default:
+        launch_kernel(k_slice_project<SPLAT_F16>, blocks, threads, smem, ctx.stream, g3, g4, vb, out, status);
+        break;
     }
     return cudaGetLastError();
 }
