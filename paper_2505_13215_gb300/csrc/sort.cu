@@ -8,7 +8,8 @@
 // The binned path (the default up to 40960 tiles per view) lists every row in
 // the 8x8-tile super-tiles that its rectangle meets, sorts each super-tile's
 // list by (depth bits, row) on its own (k_cell_count, k_cell_scan,
-// k_cell_scatter, k_unit_sort), and filters it into its tiles' lists in order:
+// k_cell_scatter, k_unit_sort; with few rows k_small_lists), and filters it into
+// its tiles' lists in order:
 // the first 512 to 2048 entries by a saturation head (k_head_count), the rest in
 // parallel segments (k_tail_count), the counts turned into ranges by one
 // look-back pass (k_tile_ranges) and the lists written by one pass
@@ -915,6 +916,8 @@ __global__ void __launch_bounds__(256) k_cell_scatter(CellArgs a)
     }
 }
 
+constexpr int log2_of(int x) { return x > 1 ? 1 + log2_of(x / 2) : 0; }
+
 struct SortArgs {
     const uint2* sranges;
     int total_super;
@@ -927,25 +930,29 @@ struct SortArgs {
     int32_t* status;
 };
 
+// Of a block of THREADS that sorts kPer entries per thread, into as many buckets.
+template <int THREADS>
 struct SortSmem {
-    unsigned long long e[kUnit];
-    uint32_t h[kSortBuckets + 4];  // bucket counts, then first positions; [kSortBuckets]: the total
-    uint32_t h2[kSortBuckets + 4];  // the same of the second level
-    uint16_t at[kUnit];            // arrival in a second-level bucket
-    uint32_t red[4][kUnitThreads / 32], tmp[kUnitThreads / 32];
+    static constexpr int kEntries = kPer * THREADS;
+    unsigned long long e[kEntries];
+    uint32_t h[kEntries + 4];   // bucket counts, then first positions; [kEntries]: the total
+    uint32_t h2[kEntries + 4];  // the same of the second level
+    uint16_t at[kEntries];      // arrival in a second-level bucket
+    uint32_t red[4][THREADS / 32], tmp[THREADS / 32];
     uint32_t n;
 };
+using UnitSmem = SortSmem<kUnitThreads>;
 
 // Bounds of a key range and the right shift that maps its differences to
-// kSortBuckets buckets (at least half of them used), order preserved.
+// 2^bits buckets (at least half of them used), order preserved.
 struct KeyRange {
     unsigned long long lo;
     int shift;
 };
 
-__device__ __forceinline__ KeyRange key_range(unsigned long long lo, unsigned long long hi)
+__device__ __forceinline__ KeyRange key_range(unsigned long long lo, unsigned long long hi, int bits)
 {
-    return {lo, max(0, 64 - kSortBucketBits - __clzll((long long)(hi - lo)))};
+    return {lo, max(0, 64 - bits - __clzll((long long)(hi - lo)))};
 }
 
 __device__ __forceinline__ uint32_t key_bucket(const KeyRange& r, unsigned long long e)
@@ -955,7 +962,8 @@ __device__ __forceinline__ uint32_t key_bucket(const KeyRange& r, unsigned long 
 
 // Block-wide key range from the threads' own extremes of the depth bits and,
 // should all depths be equal, of the rows.
-__device__ __forceinline__ void block_bounds(SortSmem& s, uint32_t dmin, uint32_t dmax, uint32_t rmin, uint32_t rmax,
+template <int THREADS>
+__device__ __forceinline__ void block_bounds(SortSmem<THREADS>& s, uint32_t dmin, uint32_t dmax, uint32_t rmin, uint32_t rmax,
                                              unsigned long long& lo, unsigned long long& hi)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -971,7 +979,7 @@ __device__ __forceinline__ void block_bounds(SortSmem& s, uint32_t dmin, uint32_
     }
     __syncthreads();
 #pragma unroll
-    for (int w = 0; w < kUnitThreads / 32; ++w) {
+    for (int w = 0; w < THREADS / 32; ++w) {
         dmin = min(dmin, s.red[0][w]);
         dmax = max(dmax, s.red[1][w]);
         rmin = min(rmin, s.red[2][w]);
@@ -981,32 +989,34 @@ __device__ __forceinline__ void block_bounds(SortSmem& s, uint32_t dmin, uint32_
     hi = (unsigned long long)dmax << 32 | (dmin == dmax ? rmax : 0xffffffffu);
 }
 
-// h: bucket counts -> first positions, h[kSortBuckets] the total; returns
+// h: bucket counts -> first positions, the last the total; returns
 // (block-uniform) whether a bucket is crowded.
-__device__ __forceinline__ bool scan_buckets(SortSmem& s, uint32_t* h)
+template <int THREADS>
+__device__ __forceinline__ bool scan_buckets(SortSmem<THREADS>& s, uint32_t* h)
 {
-    static_assert(kSortBuckets == 8 * kUnitThreads, "eight buckets per thread");
+    static_assert(kPer == 8, "eight buckets per thread");
     uint4* h4 = (uint4*)h + 2 * threadIdx.x;
     const uint4 c = h4[0], d = h4[1];
     const uint32_t mx = max(max(max(c.x, c.y), max(c.z, c.w)), max(max(d.x, d.y), max(d.z, d.w)));
     const uint32_t sc = c.x + c.y + c.z + c.w;
     uint32_t total;
-    const uint32_t x = block_excl_scan<kUnitThreads / 32>(sc + d.x + d.y + d.z + d.w, s.tmp, &total), y = x + sc;
+    const uint32_t x = block_excl_scan<THREADS / 32>(sc + d.x + d.y + d.z + d.w, s.tmp, &total), y = x + sc;
     h4[0] = make_uint4(x, x + c.x, x + c.x + c.y, x + c.x + c.y + c.z);
     h4[1] = make_uint4(y, y + d.x, y + d.x + d.y, y + d.x + d.y + d.z);
-    if (threadIdx.x == 0) h[kSortBuckets] = total;
+    if (threadIdx.x == 0) h[kPer * THREADS] = total;
     return __syncthreads_or(mx > kCrowded);
 }
 
 // The second-level position of entry e, whose bucket is b: the bucket's first
 // position, in a crowded bucket plus a share of its length linear in the row.
-__device__ __forceinline__ uint32_t second_level(const SortSmem& s, uint32_t b, uint32_t row, uint32_t rmin, int up)
+template <int THREADS>
+__device__ __forceinline__ uint32_t second_level(const SortSmem<THREADS>& s, uint32_t b, uint32_t row, uint32_t rmin, int up)
 {
     const uint32_t p = s.h[b], c = s.h[b + 1] - p;
     return c > kCrowded ? p + __umulhi((row - rmin) << up, c) : p;
 }
 
-// Sorts a unit of n <= kUnit entries, entry t + kUnitThreads k in e[k] of thread
+// Sorts a unit of n <= kPer THREADS entries, entry t + THREADS k in e[k] of thread
 // t, and writes their rows to dst: one counting-sort pass over buckets linear in
 // the key (about one entry each), then every entry counts the smaller ones of its
 // bucket.  Where a bucket is crowded (many equal depths: means stored in 16 bits
@@ -1016,14 +1026,15 @@ __device__ __forceinline__ uint32_t second_level(const SortSmem& s, uint32_t b, 
 // bitonically.  (The second pass keeps its arrivals in shared memory: in
 // registers they made the common path spill, 78 -> 118 us for the rest of the
 // lists of 1M Gaussians at 4 x 2704x2028.)
-__device__ __forceinline__ void sort_unit(SortSmem& s, const unsigned long long (&e)[kPer], int n,
+template <int THREADS>
+__device__ __forceinline__ void sort_unit(SortSmem<THREADS>& s, const unsigned long long (&e)[kPer], int n,
                                           uint32_t* __restrict__ dst)
 {
     const int tid = threadIdx.x;
     uint32_t dmin = 0xffffffffu, dmax = 0u, rmin = 0xffffffffu, rmax = 0u;
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-        if (tid + kUnitThreads * k < n) {
+        if (tid + THREADS * k < n) {
             const uint32_t d = (uint32_t)(e[k] >> 32), r = (uint32_t)e[k];
             dmin = min(dmin, d);
             dmax = max(dmax, d);
@@ -1032,19 +1043,19 @@ __device__ __forceinline__ void sort_unit(SortSmem& s, const unsigned long long 
         }
     }
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) s.h[tid + kUnitThreads * k] = 0u;
+    for (int k = 0; k < kPer; ++k) s.h[tid + THREADS * k] = 0u;
     unsigned long long lo, hi;
     block_bounds(s, dmin, dmax, rmin, rmax, lo, hi);
-    const KeyRange kr = key_range(lo, hi);
+    const KeyRange kr = key_range(lo, hi, log2_of(kPer * THREADS));
     uint32_t at[kPer];
 #pragma unroll
     for (int k = 0; k < kPer; ++k)
-        if (tid + kUnitThreads * k < n) at[k] = atomicAdd(&s.h[key_bucket(kr, e[k])], 1u);
+        if (tid + THREADS * k < n) at[k] = atomicAdd(&s.h[key_bucket(kr, e[k])], 1u);
     __syncthreads();
     const bool crowded = scan_buckets(s, s.h);
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-        if (tid + kUnitThreads * k < n) {
+        if (tid + THREADS * k < n) {
             const uint32_t b = key_bucket(kr, e[k]);
             s.e[s.h[b] + at[k]] = e[k];
         }
@@ -1053,7 +1064,7 @@ __device__ __forceinline__ void sort_unit(SortSmem& s, const unsigned long long 
     if (!crowded) {
 #pragma unroll
         for (int k = 0; k < kPer; ++k) {
-            if (tid + kUnitThreads * k < n) {
+            if (tid + THREADS * k < n) {
                 const uint32_t b = key_bucket(kr, e[k]), j1 = s.h[b + 1];
                 uint32_t j = s.h[b], r = j;
                 for (; j < j1; ++j) r += s.e[j] < e[k];
@@ -1064,27 +1075,27 @@ __device__ __forceinline__ void sort_unit(SortSmem& s, const unsigned long long 
         uint32_t* rows = (uint32_t*)s.e;
 #pragma unroll
         for (int k = 0; k < kPer; ++k)
-            if (tid + kUnitThreads * k < n) rows[at[k]] = (uint32_t)e[k];
+            if (tid + THREADS * k < n) rows[at[k]] = (uint32_t)e[k];
         __syncthreads();
-        for (int i = tid; i < n; i += kUnitThreads) dst[i] = rows[i];
+        for (int i = tid; i < n; i += THREADS) dst[i] = rows[i];
     } else {
         rmin = 0xffffffffu;
         rmax = 0u;
-        for (int w = 0; w < kUnitThreads / 32; ++w) {  // the block's bounds of the rows, as block_bounds left the warps'
+        for (int w = 0; w < THREADS / 32; ++w) {  // the block's bounds of the rows, as block_bounds left the warps'
             rmin = min(rmin, s.red[2][w]);
             rmax = max(rmax, s.red[3][w]);
         }
         const int up = __clz(max(1u, rmax - rmin));
-        for (int i = tid; i < kSortBuckets; i += kUnitThreads) s.h2[i] = 0u;
+        for (int i = tid; i < kPer * THREADS; i += THREADS) s.h2[i] = 0u;
         __syncthreads();
         bool mixed = false;
 #pragma unroll
         for (int k = 0; k < kPer; ++k) {
-            if (tid + kUnitThreads * k < n) {
+            if (tid + THREADS * k < n) {
                 const uint32_t b = key_bucket(kr, e[k]);
                 const uint32_t p = second_level(s, b, (uint32_t)e[k], rmin, up);
                 mixed |= s.h[b + 1] - s.h[b] > kCrowded && (s.e[s.h[b]] >> 32) != (e[k] >> 32);
-                s.at[tid + kUnitThreads * k] = (uint16_t)atomicAdd(&s.h2[p], 1u);
+                s.at[tid + THREADS * k] = (uint16_t)atomicAdd(&s.h2[p], 1u);
             }
         }
         mixed = __syncthreads_or(mixed);
@@ -1092,15 +1103,15 @@ __device__ __forceinline__ void sort_unit(SortSmem& s, const unsigned long long 
         if (!mixed) {
 #pragma unroll
             for (int k = 0; k < kPer; ++k) {
-                if (tid + kUnitThreads * k < n) {
+                if (tid + THREADS * k < n) {
                     const uint32_t p = second_level(s, key_bucket(kr, e[k]), (uint32_t)e[k], rmin, up);
-                    s.e[s.h2[p] + s.at[tid + kUnitThreads * k]] = e[k];
+                    s.e[s.h2[p] + s.at[tid + THREADS * k]] = e[k];
                 }
             }
             __syncthreads();
 #pragma unroll
             for (int k = 0; k < kPer; ++k) {
-                if (tid + kUnitThreads * k < n) {
+                if (tid + THREADS * k < n) {
                     const uint32_t p = second_level(s, key_bucket(kr, e[k]), (uint32_t)e[k], rmin, up);
                     const uint32_t j1 = s.h2[p + 1];
                     uint32_t j = s.h2[p], r = j;
@@ -1112,11 +1123,11 @@ __device__ __forceinline__ void sort_unit(SortSmem& s, const unsigned long long 
         } else {
             int P = 2;
             while (P < n) P <<= 1;
-            for (int i = n + tid; i < P; i += kUnitThreads) s.e[i] = ~0ull;
+            for (int i = n + tid; i < P; i += THREADS) s.e[i] = ~0ull;
             __syncthreads();
             for (int size = 2; size <= P; size <<= 1) {
                 for (int step = size >> 1; step > 0; step >>= 1) {
-                    for (int t = tid; t < P / 2; t += kUnitThreads) {
+                    for (int t = tid; t < P / 2; t += THREADS) {
                         const int i = 2 * t - (t & (step - 1)), j = i + step;
                         const unsigned long long x = s.e[i], y = s.e[j];
                         if ((x > y) == ((i & size) == 0)) {
@@ -1127,7 +1138,7 @@ __device__ __forceinline__ void sort_unit(SortSmem& s, const unsigned long long 
                     __syncthreads();
                 }
             }
-            for (int i = tid; i < n; i += kUnitThreads) dst[i] = (uint32_t)s.e[i];
+            for (int i = tid; i < n; i += THREADS) dst[i] = (uint32_t)s.e[i];
         }
     }
     __syncthreads();
@@ -1151,10 +1162,10 @@ __device__ __forceinline__ void each_entry(const unsigned long long* __restrict_
 
 // Bucket counts (scanned, in s.h) of those of src[0 .. n) within [lo, hi]; with
 // `all` of every entry, the first and the last bucket open-ended.
-__device__ __forceinline__ KeyRange count_range(SortSmem& s, const unsigned long long* src, uint32_t n,
+__device__ __forceinline__ KeyRange count_range(UnitSmem& s, const unsigned long long* src, uint32_t n,
                                                 unsigned long long lo, unsigned long long hi, bool all = false)
 {
-    const KeyRange kr = key_range(lo, hi);
+    const KeyRange kr = key_range(lo, hi, kSortBucketBits);
     for (int k = threadIdx.x; k < kSortBuckets; k += kUnitThreads) s.h[k] = 0u;
     __syncthreads();
     each_entry(src, n, [&](unsigned long long e) {
@@ -1172,7 +1183,7 @@ __device__ __forceinline__ KeyRange count_range(SortSmem& s, const unsigned long
 // number of blocks share a long unit without waiting for one another.
 // Sets the value range [lo, hi] of the part, the number of its entries and their
 // first position in the unit.
-__device__ __noinline__ void part_range(SortSmem& s, const unsigned long long* src, uint32_t n, uint32_t g,
+__device__ __noinline__ void part_range(UnitSmem& s, const unsigned long long* src, uint32_t n, uint32_t g,
                                         unsigned long long& lo, unsigned long long& hi, uint32_t& left, uint32_t& out)
 {
     const int tid = threadIdx.x;
@@ -1202,7 +1213,7 @@ __device__ __noinline__ void part_range(SortSmem& s, const unsigned long long* s
 // part that holds more than kUnit (one crowded bucket) goes through several of
 // these, each found by counting again over ever finer buckets (entries are unique,
 // so this ends).
-__device__ __noinline__ uint32_t take_range(SortSmem& s, const unsigned long long* src, uint32_t n, uint32_t left,
+__device__ __noinline__ uint32_t take_range(UnitSmem& s, const unsigned long long* src, uint32_t n, uint32_t left,
                                             unsigned long long& lo, unsigned long long hi, unsigned long long& top)
 {
     const int tid = threadIdx.x;
@@ -1243,7 +1254,7 @@ template <bool REST>
 __global__ void __launch_bounds__(kUnitThreads, 4) k_unit_sort(SortArgs a)
 {
     wait_for_previous_kernel();
-    __shared__ SortSmem s;
+    __shared__ UnitSmem s;
     if (status_failed(a.status)) return;
     const uint32_t direct = REST ? 0u : (uint32_t)a.total_super;
     const uint32_t items = direct + a.n_queue[REST ? 1 : 0];
@@ -1295,6 +1306,113 @@ __global__ void __launch_bounds__(kUnitThreads, 4) k_unit_sort(SortArgs a)
             lo = top + 1;
         }
     }
+}
+
+// The sorted super-tile lists of a call with few rows, in one kernel: a block per
+// super-tile reads every row of its view, keeps the entries of its own list in
+// shared memory and sorts them there (sort_unit).  The list starts behind the
+// entries of the super-tiles before it, which the block counts from the same
+// rectangles (and those of the earlier views), so blocks do not wait for one
+// another.  A block also clears what the later passes count in.  Where a call is as
+// small as this, the kernels above are bound by their launches and first loads:
+// 4096 rows in 128x128 sort in 40 us instead of 50, 8192 rows in 1600x1400 (143
+// super-tiles) in 48 instead of 60.
+constexpr int kSmallThreads = 1024;
+constexpr int64_t kSmallRows = kPer * kSmallThreads;  // a list holds at most every row
+
+struct SmallArgs {
+    CellArgs c;
+    uint32_t* list;  // out: the lists' rows in order
+    uint32_t* zero;  // cleared
+    int n_zero;
+};
+
+__global__ void __launch_bounds__(kSmallThreads) k_small_lists(SmallArgs s)
+{
+    wait_for_previous_kernel();
+    extern __shared__ __align__(16) unsigned char smem[];
+    SortSmem<kSmallThreads>& m = *(SortSmem<kSmallThreads>*)smem;
+    const CellArgs& a = s.c;
+    const int tid = threadIdx.x, lane = tid & 31, gs = blockIdx.x;
+    for (int64_t t = gs * (int64_t)kSmallThreads + tid; t < a.total_tiles; t += (int64_t)gridDim.x * kSmallThreads)
+        a.ranges[t] = make_uint2(0u, 0u);
+    if (gs == 0) {
+        for (int i = tid; i < s.n_zero; i += kSmallThreads) s.zero[i] = 0u;
+        if (tid == 0) {
+            *a.n_instances = 0;
+            if (a.n_needed) *a.n_needed = 0;
+        }
+    }
+    if (status_failed(a.status)) return;
+    if (tid == 0) m.n = 0u;
+    int v = 0;
+    for (int q = 1; q < a.V; ++q)
+        if (gs >= a.super_base[q]) v = q;
+    const int ls = gs - a.super_base[v], sy = ls / a.STX[v], sx = ls - sy * a.STX[v];
+    __syncthreads();
+    // rows of this view and the views before it, at most kPer per thread (all loads in flight together)
+    const int first = (int)(v * a.n), end = first + (int)a.n;
+    uint32_t nt[kPer];
+    int4 rc[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int r = tid + kSmallThreads * k;
+        nt[k] = 0u;
+        if (r < end) {
+            nt[k] = a.proj.n_tiles[r];
+            rc[k] = ((const int4*)a.proj.rect)[r];
+        }
+    }
+    uint32_t before = 0u;  // entries of the lists before this one
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int r = tid + kSmallThreads * k;
+        bool in = false;
+        if (nt[k] > 0) {
+            const int x0 = rc[k].x >> 3, y0 = rc[k].y >> 3, x1 = (rc[k].z + 7) >> 3, y1 = (rc[k].w + 7) >> 3;
+            if (x1 > x0 && y1 > y0) {
+                const int w = x1 - x0;
+                if (r < first) {
+                    before += (uint32_t)(w * (y1 - y0));
+                } else {
+                    const bool row_in = sy >= y0 && sy < y1;
+                    before += (uint32_t)(w * min(max(sy - y0, 0), y1 - y0) + (row_in ? min(max(sx - x0, 0), w) : 0));
+                    in = row_in && sx >= x0 && sx < x1;
+                }
+            }
+        }
+        const unsigned hits = __ballot_sync(0xffffffffu, in);
+        if (!hits) continue;
+        uint32_t at = 0u;
+        if (lane == 0) at = atomicAdd(&m.n, (uint32_t)__popc(hits));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(hits & lanemask_lt());
+        if (in) {
+            const float depth = ((const float4*)a.proj.rgb_depth)[r].w;
+            m.e[at] = (unsigned long long)__float_as_uint(depth) << 32 | (uint32_t)r;
+        }
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0) m.tmp[tid >> 5] = before;
+    __syncthreads();
+    const uint32_t n = m.n;
+    uint32_t start = __reduce_add_sync(0xffffffffu, m.tmp[lane]);
+    if (tid == 0) {
+        a.sranges[gs] = n ? make_uint2(start, start + n) : make_uint2(0u, 0u);
+        if (gs == a.total_super - 1) {
+            const int64_t K1 = (int64_t)start + n;
+            *a.K1 = K1;
+            if (K1 > a.capacity) set_status(a.status, SPLAT_ERR_CAPACITY, SPLAT_STAGE_SCAN, K1);
+        }
+    }
+    if (!n || (int64_t)start + n > a.capacity) return;  // (block-uniform)
+    unsigned long long e[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const uint32_t i = tid + kSmallThreads * k;
+        e[k] = i < n ? m.e[i] : 0ull;
+    }
+    __syncthreads();
+    sort_unit<kSmallThreads>(m, e, (int)n, s.list + start);
 }
 
 // Tiles in decreasing order of list length for the compositing kernels'
@@ -1554,7 +1672,8 @@ struct TileRangeArgs {
     int64_t capacity;
     const int64_t* K_super;  // entries of the super-tile lists, which share the capacity
     int64_t* needed;         // may be null
-    uint32_t* cls;           // [33] tiles per list-length class for the tile order (zeroed), or null
+    uint32_t* cls;           // [kOrderClasses] tiles per list-length class for the tile order (zeroed), or null
+    uint32_t* order;         // the tile order, where one block holds every tile (else null)
     int64_t spin_limit;
 };
 
@@ -1649,9 +1768,21 @@ __global__ void __launch_bounds__(256) k_tile_ranges(TileArgs a, TileRangeArgs r
         }
     }
     __syncthreads();
-    if (r.cls)
+    if (r.order) {  // (block-uniform) k_tile_order's slots: the classes' starts, the longest first, then cursors
+        __shared__ uint32_t s_tmp[8];
+        const uint32_t cb = kOrderClasses - 1u - tid;
+        uint32_t total;
+        const uint32_t ex = block_excl_scan256(s_cls[cb], s_tmp, &total);
+        s_cls[cb] = ex;
+        if (tid == 0) s_cls[0] = total;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kRangeTileItems; ++q)
+            if (t0 + q < a.total_tiles) r.order[atomicAdd(&s_cls[length_class(cnt[q])], 1u)] = (uint32_t)(t0 + q);
+    } else if (r.cls) {
         for (int c = tid; c < (int)kOrderClasses; c += blockDim.x)
             if (s_cls[c]) atomicAdd(&r.cls[c], s_cls[c]);
+    }
     // slots past 2^32 only arise with K beyond any capacity: the check above reports them
     uint32_t st = (uint32_t)(s_excl + texcl);
 #pragma unroll
@@ -2271,6 +2402,13 @@ static int sort_ctas_per_sm()
 }
 
 
+// Whether a call takes k_small_lists: a list may hold every row, and its blocks,
+// which fill an SM, run in one wave.
+static bool small_lists(int64_t n_rows, int64_t total_super, int num_sms)
+{
+    return n_rows <= kSmallRows && total_super <= num_sms;
+}
+
 static cudaError_t run_pass(const PassArgs& a, int64_t parts, int resident, cudaStream_t s)
 {
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(parts, resident));
@@ -2297,7 +2435,9 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
     auto U = [&](size_t off) { return (uint32_t*)(w + off); };
     cudaStream_t s = ctx.stream;
     cudaError_t err;
-    if ((err = cudaMemsetAsync(w + L.zero_begin, 0, L.zero_end - L.zero_begin, s)) != cudaSuccess) return err;
+    // (k_small_lists clears what its call needs)
+    const bool small = L.binned && n_rows > 0 && small_lists(n_rows, L.total_super, ctx.num_sms);
+    if (!small && (err = cudaMemsetAsync(w + L.zero_begin, 0, L.zero_end - L.zero_begin, s)) != cudaSuccess) return err;
     if (n_rows == 0 || !L.binned) {  // (k_cell_count clears them otherwise)
         if ((err = cudaMemsetAsync(bins.ranges, 0, sizeof(uint32_t) * 2 * (size_t)vb.total_tiles, s)) != cudaSuccess)
             return err;
@@ -2350,10 +2490,19 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         c.n_instances = bins.n_instances;
         c.n_needed = bins.n_needed;
         auto row_grid = [&](int rows) { return dim3((unsigned)((proj.n + rows - 1) / rows), (unsigned)vb.V); };
-        count_launch(3);
-        launch_kernel(k_cell_count, row_grid(256 * kRowsPerThread), 256, 0, s, c);
-        launch_kernel(k_cell_scan, sb, 256, 0, s, c);
-        launch_kernel(k_cell_scatter, row_grid(256), 256, 0, s, c);
+        if (small) {
+            SmallArgs sm{c, U(L.off_vals1), (uint32_t*)(w + L.zero_begin), (int)((L.off_cell - L.zero_begin) / 4)};
+            constexpr int smem = (int)sizeof(SortSmem<kSmallThreads>);
+            err = cudaFuncSetAttribute(k_small_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (err != cudaSuccess) return err;  // (set for the current device)
+            count_launch();
+            launch_kernel(k_small_lists, sb, kSmallThreads, smem, s, sm);
+        } else {
+            count_launch(3);
+            launch_kernel(k_cell_count, row_grid(256 * kRowsPerThread), 256, 0, s, c);
+            launch_kernel(k_cell_scan, sb, 256, 0, s, c);
+            launch_kernel(k_cell_scatter, row_grid(256), 256, 0, s, c);
+        }
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         // 2. the units of each list that the head pass takes, in order
         SortArgs u{};
@@ -2415,6 +2564,7 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         tr.K_super = (const int64_t*)(w + L.off_ninst1);
         tr.needed = bins.n_needed;
         tr.cls = bins.tile_order ? U(L.off_tord) : nullptr;
+        tr.order = vb.total_tiles <= kRangeTiles ? bins.tile_order : nullptr;
         tr.spin_limit = ctx.spin_limit;
         // the head of each super-tile list in order (each tile's list up to its
         // saturation), the rest of the units and the tail in parallel segments, the
@@ -2424,14 +2574,14 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         auto blocks_f = [&](int write) {
             return (int)std::min<int64_t>(L.max_segs + (write ? sb : 0), (int64_t)ctx.num_sms * per_sm_f[write]);
         };
-        count_launch(6);
-        launch_kernel(k_unit_sort<false>, blocks_u(0), kUnitThreads, 0, s, u);
+        count_launch(small ? 4 : 6);
+        if (!small) launch_kernel(k_unit_sort<false>, blocks_u(0), kUnitThreads, 0, s, u);
         launch_kernel(k_head_count, 2 * sb, kHeadEntries, 0, s, t);
-        launch_kernel(k_unit_sort<true>, blocks_u(1), kUnitThreads, 0, s, u);
+        if (!small) launch_kernel(k_unit_sort<true>, blocks_u(1), kUnitThreads, 0, s, u);
         launch_kernel(k_tail_count, blocks_f(0), 256, 0, s, t);
         launch_kernel(k_tile_ranges, (int)((vb.total_tiles + kRangeTiles - 1) / kRangeTiles), 256, 0, s, t, tr);
         launch_kernel(k_tile_write, blocks_f(1), 256, 0, s, t);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+        if ((err = cudaGetLastError()) != cudaSuccess || tr.order) return err;
         return launch_tile_order(bins, L.total_tiles, U(L.off_tord), status, ctx, true);
     }
     // radix path: 1. depth keys + digit counts; zero the first depth look-back buffer and the scan's
