@@ -1350,45 +1350,46 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_lists(SmallArgs s)
         if (gs >= a.super_base[q]) v = q;
     const int ls = gs - a.super_base[v], sy = ls / a.STX[v], sx = ls - sy * a.STX[v];
     __syncthreads();
-    // rows of this view and the views before it, at most kPer per thread (all loads in flight together)
+    // rows of this view and the views before it, at most kPer per thread, four with all their loads in flight
     const int first = (int)(v * a.n), end = first + (int)a.n;
-    uint32_t nt[kPer];
-    int4 rc[kPer];
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        const int r = tid + kSmallThreads * k;
-        nt[k] = 0u;
-        if (r < end) {
-            nt[k] = a.proj.n_tiles[r];
-            rc[k] = ((const int4*)a.proj.rect)[r];
-        }
-    }
     uint32_t before = 0u;  // entries of the lists before this one
+    for (int r0 = tid; r0 - tid < end; r0 += 4 * kSmallThreads) {
+        uint32_t nt[4];
+        int4 rc[4];
+        float depth[4];
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        const int r = tid + kSmallThreads * k;
-        bool in = false;
-        if (nt[k] > 0) {
-            const int x0 = rc[k].x >> 3, y0 = rc[k].y >> 3, x1 = (rc[k].z + 7) >> 3, y1 = (rc[k].w + 7) >> 3;
-            if (x1 > x0 && y1 > y0) {
-                const int w = x1 - x0;
-                if (r < first) {
-                    before += (uint32_t)(w * (y1 - y0));
-                } else {
-                    const bool row_in = sy >= y0 && sy < y1;
-                    before += (uint32_t)(w * min(max(sy - y0, 0), y1 - y0) + (row_in ? min(max(sx - x0, 0), w) : 0));
-                    in = row_in && sx >= x0 && sx < x1;
-                }
+        for (int k = 0; k < 4; ++k) {
+            const int r = r0 + kSmallThreads * k;
+            nt[k] = 0u;
+            if (r < end) {
+                nt[k] = a.proj.n_tiles[r];
+                rc[k] = ((const int4*)a.proj.rect)[r];
+                depth[k] = ((const float4*)a.proj.rgb_depth)[r].w;
             }
         }
-        const unsigned hits = __ballot_sync(0xffffffffu, in);
-        if (!hits) continue;
-        uint32_t at = 0u;
-        if (lane == 0) at = atomicAdd(&m.n, (uint32_t)__popc(hits));
-        at = __shfl_sync(0xffffffffu, at, 0) + __popc(hits & lanemask_lt());
-        if (in) {
-            const float depth = ((const float4*)a.proj.rgb_depth)[r].w;
-            m.e[at] = (unsigned long long)__float_as_uint(depth) << 32 | (uint32_t)r;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int r = r0 + kSmallThreads * k;
+            bool in = false;
+            if (nt[k] > 0) {
+                const int x0 = rc[k].x >> 3, y0 = rc[k].y >> 3, x1 = (rc[k].z + 7) >> 3, y1 = (rc[k].w + 7) >> 3;
+                if (x1 > x0 && y1 > y0) {
+                    const int w = x1 - x0;
+                    if (r < first) {
+                        before += (uint32_t)(w * (y1 - y0));
+                    } else {
+                        const bool row_in = sy >= y0 && sy < y1;
+                        before += (uint32_t)(w * min(max(sy - y0, 0), y1 - y0) + (row_in ? min(max(sx - x0, 0), w) : 0));
+                        in = row_in && sx >= x0 && sx < x1;
+                    }
+                }
+            }
+            const unsigned hits = __ballot_sync(0xffffffffu, in);
+            if (!hits) continue;
+            uint32_t at = 0u;
+            if (lane == 0) at = atomicAdd(&m.n, (uint32_t)__popc(hits));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(hits & lanemask_lt());
+            if (in) m.e[at] = (unsigned long long)__float_as_uint(depth[k]) << 32 | (uint32_t)r;
         }
     }
     before = __reduce_add_sync(0xffffffffu, before);
@@ -2013,10 +2014,11 @@ __global__ void __launch_bounds__(kHeadEntries, 2) k_head_count(TileArgs a)
 // the masks of its group and counts by population counts.  A queue of entries
 // per tile row and a warp reduction per pair of columns took 312 us on 1M
 // Gaussians at 4 x 2704x2028.
-__global__ void __launch_bounds__(256) k_tail_count(TileArgs a)
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) k_tail_count(TileArgs a)
 {
     wait_for_previous_kernel();
-    __shared__ uint32_t s_cnt[8][64];
+    __shared__ uint32_t s_cnt[WARPS][64];
     __shared__ uint32_t s_g;
     __shared__ int s_gs;
     if (status_failed(a.status)) return;
@@ -2041,7 +2043,7 @@ __global__ void __launch_bounds__(256) k_tail_count(TileArgs a)
         const uint32_t r0 = tail_start(sat, nh) + (g - a.seg_base[gs]) * kFilterSeg, b0 = rgs.x + r0;
         const int n = (int)min((uint32_t)kFilterSeg, rgs.y - b0);
         uint32_t c0 = 0u, c1 = 0u;  // entries listed in tiles lane and lane + 32
-        for (int q = 32 * warp; q < n; q += 256) {  // warp-uniform
+        for (int q = 32 * warp; q < n; q += 32 * WARPS) {  // warp-uniform
             const int e = q + lane;
             // (warp-uniform) whether each half is open and past its head: the words of a half's head stay as they are
             const bool h0 = sat.x != 0xffffffffu && r0 + q >= nh.x, h1 = sat.y != 0xffffffffu && r0 + q >= nh.y;
@@ -2084,7 +2086,7 @@ __global__ void __launch_bounds__(256) k_tail_count(TileArgs a)
         if (tid < 64) {
             uint32_t c = 0u;
 #pragma unroll
-            for (int w = 0; w < 8; ++w) c += s_cnt[w][tid];
+            for (int w = 0; w < WARPS; ++w) c += s_cnt[w][tid];
             a.seg_cnt[(size_t)g * 64 + tid] = c;
         }
         __syncthreads();
@@ -2092,7 +2094,7 @@ __global__ void __launch_bounds__(256) k_tail_count(TileArgs a)
 }
 
 // Writing pass: the heads (one ticket per super-tile), then the tail segments,
-// one CTA each, warp w serving tile row w; driven by the coverage words alone.
+// one CTA each, 8 / COLS warps per tile row; driven by the coverage words alone.
 // Lane j holds group j's words of the row's eight tiles.  Tile by tile, the
 // prefix over the groups' counts gives every listed entry its slot.  Where the
 // groups list few entries (a mean of at most kSparse), each lane goes through
@@ -2103,15 +2105,19 @@ __global__ void __launch_bounds__(256) k_tail_count(TileArgs a)
 // Gaussians at 4 x 2704x2028.)
 constexpr int kSparse = 6;
 
-__global__ void __launch_bounds__(256) k_tile_write(TileArgs a)
+// COLS columns of the row per warp: 8 / COLS warps share it.
+template <int COLS>
+__global__ void __launch_bounds__(32 * 64 / COLS) k_tile_write(TileArgs a)
 {
     wait_for_previous_kernel();
     __shared__ uint32_t s_row[kFilterSeg];
-    __shared__ uint32_t s_buf[8][32 * kSparse];
+    constexpr int kThreads = 32 * 64 / COLS;
+    __shared__ uint32_t s_buf[64 / COLS][32 * kSparse];
     __shared__ uint32_t s_tk;
     __shared__ int s_gs;
     if (status_failed(a.status)) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tr = warp / (8 / COLS), tc = warp % (8 / COLS) * COLS;  // the warp's tile row and first column
     const unsigned lt = lanemask_lt();
     const uint32_t nseg = a.seg_base[a.total_super], nhead = (uint32_t)a.total_super;
     for (;;) {
@@ -2132,10 +2138,10 @@ __global__ void __launch_bounds__(256) k_tile_write(TileArgs a)
         const int ls = gs - a.super_base[v];
         const int sy = ls / a.STX[v], sx = ls - sy * a.STX[v];
         const int TX = a.TX[v], TY = a.TY[v];
-        const int ty = sy * 8 + warp, tx0 = sx * 8;
+        const int ty = sy * 8 + tr, tx0 = sx * 8 + tc;
         const uint2 rgs = a.sranges[gs], sat = a.sat_head[gs], nh = a.n_head[gs];
-        const bool open = (warp < 4 ? sat.x : sat.y) != 0xffffffffu;  // this warp's half has a tail
-        const uint32_t my_head = warp < 4 ? nh.x : nh.y;
+        const bool open = (tr < 4 ? sat.x : sat.y) != 0xffffffffu;  // this warp's half has a tail
+        const uint32_t my_head = tr < 4 ? nh.x : nh.y;
         uint32_t b0 = rgs.x, b1, from, to;  // the item's entries [b0, b1), of which this warp's are [from, to)
         if (head) {  // each half of the super-tile up to where its head stopped
             b1 = b0 + max(nh.x, nh.y);
@@ -2147,31 +2153,31 @@ __global__ void __launch_bounds__(256) k_tile_write(TileArgs a)
             from = max(b0, rgs.x + my_head);  // (whole groups: heads stop at multiples of kHeadEntries)
             to = open ? b1 : b0;
         }
-        uint32_t first[8];  // next slot of each tile's list
+        uint32_t first[COLS];  // next slot of each tile's list
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
+        for (int k = 0; k < COLS; ++k) {
             first[k] = 0u;
             if (ty < TY && tx0 + k < TX) {
                 const int tile = a.tile_base[v] + ty * TX + tx0 + k;
                 first[k] = head ? a.ranges[tile].x
-                                : a.tile_total[tile] + a.seg_cnt[(size_t)(tk - nhead) * 64 + 8 * warp + k];
+                                : a.tile_total[tile] + a.seg_cnt[(size_t)(tk - nhead) * 64 + 8 * tr + tc + k];
             }
         }
         for (; b0 < b1; b0 += kFilterSeg) {
             const int rows = (int)min((uint32_t)kFilterSeg, b1 - b0);
-            for (int i = tid; i < rows; i += 256) s_row[i] = a.list[b0 + i];
+            for (int i = tid; i < rows; i += kThreads) s_row[i] = a.list[b0 + i];
             __syncthreads();
             const int n = to > max(b0, from) ? (int)min((uint32_t)kFilterSeg, to - b0) : 0;
             const int skip = from > b0 ? (int)(from - b0) >> 5 : 0;  // groups of the half's head
             if (ty < TY && n > 0) {  // warp-uniform
                 const int full = n >> 5, part = n & 31, groups = full + (part ? 1 : 0);
-                uint32_t word[8];
+                uint32_t word[COLS];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) word[k] = 0u;
+                for (int k = 0; k < COLS; ++k) word[k] = 0u;
                 if (lane >= skip && lane < full) {
-                    const uint2* p = a.mask + b0 + 32 * lane + 4 * warp;
+                    const uint2* p = a.mask + b0 + 32 * lane + 4 * tr + tc / 2;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
+                    for (int k = 0; k < COLS / 2; ++k) {
                         const uint2 t = p[k];
                         word[2 * k] = t.x;
                         word[2 * k + 1] = t.y;
@@ -2181,16 +2187,16 @@ __global__ void __launch_bounds__(256) k_tile_write(TileArgs a)
                     uint32_t byte = 0u;
                     if (lane < part) {
                         const uint2 t = a.mask[b0 + 32 * full + lane];
-                        byte = (warp < 4 ? t.x >> (8 * warp) : t.y >> (8 * (warp - 4))) & 0xffu;
+                        byte = (tr < 4 ? t.x >> (8 * tr) : t.y >> (8 * (tr - 4))) >> tc & 0xffu;
                     }
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
+                    for (int k = 0; k < COLS; ++k) {
                         const uint32_t bal = __ballot_sync(0xffffffffu, (byte >> k) & 1u);
                         if (lane == full) word[k] = bal;
                     }
                 }
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
+                for (int k = 0; k < COLS; ++k) {
                     uint32_t w = word[k];
                     const uint32_t c = __popc(w);
                     uint32_t at = c;
@@ -2402,6 +2408,30 @@ static int sort_ctas_per_sm()
 }
 
 
+// Tail segments and writing items, one wave of CTAs at most.  A segment's time is
+// what few of them take, so they get as many warps as fill the chip: 32 up to 8
+// segments per SM (capacity / 1024 of them), 16 up to 48, else 8, whose small CTAs
+// pack best.  Bin sort us with 32 / 16 / 8 warps:
+//   128x128, 4k            32 / 34 / 36       677x507, 101k        60 / 63 / 69
+//   857x479, 60k, 2 views  70 / 75 / 84       857x479, 120k, 3     76 / 75 / 83
+//   1352x1014, 300k       109 / 106 / 118     2704x2028, 1M       233 / 230 / 237
+//   1352x1014, 300k, 4    264 / 260 / 260     676x507, 200k, 16   391 / 348 / 320
+template <int WARPS>
+static void tail_count(const TileArgs& t, int64_t segs, const LaunchCtx& ctx)
+{
+    static const int per_sm = ctas_per_sm(k_tail_count<WARPS>, 32 * WARPS);
+    const int blocks = (int)std::min<int64_t>(segs, (int64_t)ctx.num_sms * per_sm);
+    launch_kernel(k_tail_count<WARPS>, blocks, 32 * WARPS, 0, ctx.stream, t);
+}
+
+template <int COLS>
+static void tile_write(const TileArgs& t, int64_t items, const LaunchCtx& ctx)
+{
+    static const int per_sm = ctas_per_sm(k_tile_write<COLS>, 32 * 64 / COLS);
+    const int blocks = (int)std::min<int64_t>(items, (int64_t)ctx.num_sms * per_sm);
+    launch_kernel(k_tile_write<COLS>, blocks, 32 * 64 / COLS, 0, ctx.stream, t);
+}
+
 // Whether a call takes k_small_lists: a list may hold every row, and its blocks,
 // which fill an SM, run in one wave.
 static bool small_lists(int64_t n_rows, int64_t total_super, int num_sms)
@@ -2570,17 +2600,20 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         // saturation), the rest of the units and the tail in parallel segments, the
         // prefix over head and segments with the ranges, K and the capacity check,
         // then the heads' and segments' writes in one pass
-        static const int per_sm_f[2] = {ctas_per_sm(k_tail_count, 256), ctas_per_sm(k_tile_write, 256)};
-        auto blocks_f = [&](int write) {
-            return (int)std::min<int64_t>(L.max_segs + (write ? sb : 0), (int64_t)ctx.num_sms * per_sm_f[write]);
-        };
+        // warps per segment by the segments per SM (see tail_count)
+        const int64_t segs = L.max_segs + sb;
+        const int tier = segs <= 8 * (int64_t)ctx.num_sms ? 0 : (segs <= 48 * (int64_t)ctx.num_sms ? 1 : 2);
         count_launch(small ? 4 : 6);
         if (!small) launch_kernel(k_unit_sort<false>, blocks_u(0), kUnitThreads, 0, s, u);
         launch_kernel(k_head_count, 2 * sb, kHeadEntries, 0, s, t);
         if (!small) launch_kernel(k_unit_sort<true>, blocks_u(1), kUnitThreads, 0, s, u);
-        launch_kernel(k_tail_count, blocks_f(0), 256, 0, s, t);
+        if (tier == 0) tail_count<32>(t, L.max_segs, ctx);
+        else if (tier == 1) tail_count<16>(t, L.max_segs, ctx);
+        else tail_count<8>(t, L.max_segs, ctx);
         launch_kernel(k_tile_ranges, (int)((vb.total_tiles + kRangeTiles - 1) / kRangeTiles), 256, 0, s, t, tr);
-        launch_kernel(k_tile_write, blocks_f(1), 256, 0, s, t);
+        if (tier == 0) tile_write<2>(t, segs, ctx);
+        else if (tier == 1) tile_write<4>(t, segs, ctx);
+        else tile_write<8>(t, segs, ctx);
         if ((err = cudaGetLastError()) != cudaSuccess || tr.order) return err;
         return launch_tile_order(bins, L.total_tiles, U(L.off_tord), status, ctx, true);
     }

@@ -72,3 +72,27 @@ def test_capacity_and_tile_order(W, H):
     e = np.where(got > 0, np.floor(np.log2(np.maximum(got, 1))), 0)
     cls = np.where(got > 0, 1 + 8 * e + np.floor((got / 2.0 ** e - 1) * 8), 0)  # eight classes per power of two
     assert (np.diff(cls) <= 0).all()
+
+
+def test_warps_per_segment():
+    """The tail's passes take 32, 16 or 8 warps per segment by the capacity; the lists are the same."""
+    rng = np.random.default_rng(11)
+    views = [scenes.identity_view(250, 130, 128.0, 0.5)]
+    n = 9000
+    rects, z, visible = _rects(n, 16, 9, rng), _depths("uniform", n, rng), rng.uniform(size=n) < 0.9
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    caps = [1024 * sms * k for k in (4, 20, 50)]
+    for cap in caps:
+        _check(views, n, rects, z, visible, cap=cap)
+    # with culling and ended lists, on a scene of full lists
+    scene, arc = scenes.arc_scene(n=30000)
+    G, out = raster.Gaussians.from_scene(scene, "cuda"), []
+    for cap in caps:
+        R = raster.Rasterizer(G.n3, G.n4, arc[:1], capacity=cap)
+        R.forward(G)
+        torch.cuda.synchronize()
+        R.check()
+        K = R.instances()
+        out.append((K, R.vals[:K].clone(), R.keys[:K].clone(), R.ranges.clone()))
+    for o in out[1:]:
+        assert o[0] == out[0][0] and all(torch.equal(a, b) for a, b in zip(o[1:], out[0][1:]))
