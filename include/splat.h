@@ -272,10 +272,9 @@ splat_status splat_slice_project(const splat_g3 *g3, const splat_g4 *g4, const s
  * Every visible row emits one instance per tile of its rectangle, keyed by
  * (global tile index, camera depth); the instances are sorted by that key,
  * stably, ties in emission order (row r ascending, tiles row major).  Because
- * the depth part of the key is the same for every instance of a row, the
- * depth digits of this LSD radix sort are sorted once per row before the
- * duplication, then the tile digits after it; the resulting order is the
- * same.  Writes bins->keys/vals (first K entries), bins->ranges (every tile,
+ * the depth part of the key is the same for every instance of a row, no pass
+ * sorts instances by it: rows are ordered by depth before they are listed in
+ * tiles; the resulting order is the same.  Writes bins->keys/vals (first K entries), bins->ranges (every tile,
  * [0,0) when empty) and *bins->n_instances = K.  K > capacity sets
  * SPLAT_ERR_CAPACITY with the required count in status[2..3] and n_instances;
  * on the binned path (see splat_set_tile_sort) the intermediate super-tile
@@ -566,8 +565,8 @@ int64_t splat_launch_count(void);
 /*
  * Selects how splat_bin_sort orders the instances by tile (the result is the
  * same):  0 = automatic (default), 1 = tile-digit radix passes over the
- * instance list, 2 = binned partition: the rows split by 8x8-tile super-tile,
- * then each super-tile's list filtered into its tiles' lists (used
+ * instance list, 2 = binned partition: the rows listed by 8x8-tile super-tile,
+ * each super-tile's list sorted by depth and filtered into its tiles' lists (used
  * automatically when every view has at most 40960 tiles; never for a view of
  * more than 1023 super-tiles in x or y or more than about 5000 in all, which
  * take the radix passes).  Host-side global (the library default of

@@ -1555,7 +1555,7 @@ struct TileArgs {
 // margin for the rounding of the T products (a product of (1 - alpha) below
 // e^-9.25 at every pixel; the kernels' T rounds by about 2^-23 an update, which
 // the margin covers for 2e5 updates, and a cut falls within the first
-// kHeadEntries entries of a list).  The sums are exact integers, so the
+// kLongHead entries of a list).  The sums are exact integers, so the
 // cut does not depend on the order of any reduction.
 constexpr float kSatScale = 65536.f;                       // fixed point of -ln(1 - alpha)
 constexpr uint32_t kSatThreshold = (uint32_t)(9.25 * 65536);  // -ln(1e-4) = 9.2103 plus the margin
