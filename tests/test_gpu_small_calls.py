@@ -27,12 +27,13 @@ def test_one_view(n, kind):
            rng.uniform(size=n) < 0.9)
 
 
-@pytest.mark.parametrize("n", [300, 2730, 2731])
-def test_three_views(n):
+@pytest.mark.parametrize("n,V", [(300, 3), (2730, 3), (2731, 3), (8192, 4), (8193, 4), (6554, 5)])
+def test_several_views(n, V):
     rng = np.random.default_rng(n)
-    views = [scenes.identity_view(W, H, 200.0, 0.5) for W, H in ((300, 170), (64, 20), (129, 257))]
+    sizes = ((300, 170), (64, 20), (129, 257), (16, 16), (200, 140))
+    views = [scenes.identity_view(W, H, 200.0, 0.5) for W, H in sizes[:V]]
     rects = np.concatenate([_rects(n, (v.W + 15) // 16, (v.H + 15) // 16, rng, 12) for v in views])
-    _check(views, n, rects, _depths("uniform", 3 * n, rng), rng.uniform(size=3 * n) < 0.7)
+    _check(views, n, rects, _depths("uniform", V * n, rng), rng.uniform(size=V * n) < 0.7)
 
 
 @pytest.mark.parametrize("n", [511, 2047, 2048, 2049, 4097])
