@@ -2231,8 +2231,9 @@ __global__ void __launch_bounds__(32 * 64 / COLS) k_tile_write(TileArgs a)
                     first[k] += total;
                 }
             }
-            __syncthreads();
+            if (b0 + kFilterSeg < b1) __syncthreads();  // (block-uniform) s_row is rewritten
         }
+        __syncthreads();  // s_tk, s_gs and s_row are rewritten, also after an item without entries
     }
 }
 
