@@ -1343,14 +1343,13 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_lists(SmallArgs s)
             if (a.n_needed) *a.n_needed = 0;
         }
     }
-    if (status_failed(a.status)) return;
     if (tid == 0) m.n = 0u;
+    if (block_failed(a.status)) return;  // (the last super-tile's block sets it)
     int v = 0;
     for (int q = 1; q < a.V; ++q)
         if (gs >= a.super_base[q]) v = q;
     const int ls = gs - a.super_base[v], sy = ls / a.STX[v], sx = ls - sy * a.STX[v];
-    __syncthreads();
-    // rows of this view and the views before it, at most kPer per thread, four with all their loads in flight
+    // rows of this view and the views before it, at most 4 kPer per thread, four with all their loads in flight
     const int first = (int)(v * a.n), end = first + (int)a.n;
     uint32_t before = 0u;  // entries of the lists before this one
     for (int r0 = tid; r0 - tid < end; r0 += 4 * kSmallThreads) {

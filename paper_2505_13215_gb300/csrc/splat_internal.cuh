@@ -59,6 +59,12 @@ __device__ __forceinline__ bool status_failed(const int32_t* status)
     return *((volatile const int32_t*)status) != 0;
 }
 
+// status_failed, the same for every thread of the block (a barrier): for kernels
+// whose own blocks set the status.  Threads that read it one by one could part: a
+// block that starts while another one fails would go on with some of its warps, on
+// shared memory that the others have not written.
+__device__ __forceinline__ bool block_failed(const int32_t* status) { return __syncthreads_or(status_failed(status)); }
+
 // ---------------------------------------------------------------------------
 // Relaxed / acquire / release global accesses for the decoupled look-backs
 // ---------------------------------------------------------------------------
