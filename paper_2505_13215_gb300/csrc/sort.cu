@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(PassArgs a)
     __shared__ uint32_t s_tmp[8];
     __shared__ int64_t s_ticket;
 
-    if (status_failed(a.status)) return;
+    if (block_failed(a.status)) return;
     const int64_t n = a.n_dev ? min(*a.n_dev, a.cap) : a.n_host;
     if (n <= 0) return;
     const int64_t parts = (n + kSortPart - 1) / kSortPart;
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(ScanArgs a)
     __shared__ int64_t s_ticket;
     __shared__ unsigned long long s_excl;
     constexpr unsigned long long kA = 1ull << 62, kP = 2ull << 62, kM = (1ull << 62) - 1;
-    if (status_failed(a.status)) return;  // the row order is not valid after a failed sort
+    if (block_failed(a.status)) return;  // the row order is not valid after a failed sort
     const int64_t parts = (a.n_rows + kScanPart - 1) / kScanPart;
     const int tid = threadIdx.x;
     for (;;) {
@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(256) k_cell_scan(CellArgs a)
     __shared__ unsigned long long s_excl;
     __shared__ int s_gs;
     constexpr unsigned long long kA = 1ull << 62, kP = 2ull << 62, kM = (1ull << 62) - 1;
-    if (status_failed(a.status)) return;
+    if (block_failed(a.status)) return;
     const int tid = threadIdx.x;
     if (tid == 0) s_gs = (int)atomicAdd(a.ticket, 1u);
     __syncthreads();
@@ -1685,7 +1685,7 @@ __global__ void __launch_bounds__(256) k_tile_ranges(TileArgs a, TileRangeArgs r
     __shared__ int64_t s_ticket;
     __shared__ uint32_t s_cls[kOrderClasses];
     constexpr unsigned long long kA = 1ull << 62, kP = 2ull << 62, kM = (1ull << 62) - 1;
-    if (status_failed(a.status)) return;
+    if (block_failed(a.status)) return;
     const int tid = threadIdx.x;
     if (tid == 0) s_ticket = atomicAdd(r.ticket, 1u);
     for (int c = tid; c < (int)kOrderClasses; c += blockDim.x) s_cls[c] = 0u;
