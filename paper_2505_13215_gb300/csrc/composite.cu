@@ -308,9 +308,9 @@ struct FwdOccupancy {
 // STATS: also count, per warp, the pixel-Gaussian pairs evaluated (power
 // computed) and blended, into stats[0..1] (diagnostic instantiation only).
 template <int PPL, bool STATS>
-__global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks) k_composite_fwd(splat_proj proj, const uint32_t* __restrict__ vals,
-                                                                   const uint2* __restrict__ ranges,
-                                                                   const uint32_t* __restrict__ order, ViewBatch vb,
+__global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks) k_composite_fwd(splat_proj proj, const uint32_t* vals,
+                                                                   const uint2* ranges,
+                                                                   const uint32_t* order, ViewBatch vb,
                                                                    splat_image img, L1Fuse l1, int32_t* status,
                                                                    unsigned long long* stats)
 {
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, FwdOccupancy<PPL>::kMinBlocks
     if (unit >= (int64_t)vb.total_tiles * BANDS) return;
     // tiles in the bin sort's order (longest list first) when it wrote one
     const int slot = (int)(unit / BANDS), band = (int)(unit % BANDS);
-    const int tile = order ? (int)__ldg(order + slot) : slot;
+    const int tile = order ? (int)order[slot] : slot;
     const int v = find_view(vb, tile);
     const ViewParams& vp = vb.v[v];
     const int local = tile - vp.tile_base;
@@ -712,10 +712,10 @@ __device__ __forceinline__ bool bwd_gaussian(const Feat& f, const ColTerms& ct, 
 
 // STATS: also count the pairs evaluated and blended into stats[2..3].
 template <int PPL, bool STATS>
-__global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks) k_composite_bwd(splat_proj proj, const uint32_t* __restrict__ vals,
-                                                                   const uint2* __restrict__ ranges,
-                                                                   const uint32_t* __restrict__ order, ViewBatch vb,
-                                                                   splat_image img, const float* __restrict__ dL,
+__global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks) k_composite_bwd(splat_proj proj, const uint32_t* vals,
+                                                                   const uint2* ranges,
+                                                                   const uint32_t* order, ViewBatch vb,
+                                                                   splat_image img, const float* dL,
                                                                    float* dproj, int32_t* status,
                                                                    unsigned long long* stats)
 {
@@ -736,7 +736,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks
     if (unit >= (int64_t)vb.total_tiles * BANDS) return;
     // tiles in the bin sort's order (longest list first) when it wrote one
     const int slot = (int)(unit / BANDS), band = (int)(unit % BANDS);
-    const int tile = order ? (int)__ldg(order + slot) : slot;
+    const int tile = order ? (int)order[slot] : slot;
     const int v = find_view(vb, tile);
     const ViewParams& vp = vb.v[v];
     const int local = tile - vp.tile_base;
@@ -907,8 +907,8 @@ __global__ void __launch_bounds__(kCompWarps * 32, BwdOccupancy<PPL>::kMinBlocks
 // L1 photometric loss of the rendered images against a target (the loss of
 // the paper's training step): loss += sum |img - target|, dL/dimg =
 // sign(img - target) * scale.
-__global__ void __launch_bounds__(256) k_l1_loss(const float* __restrict__ img, const float* __restrict__ target,
-                                                 int64_t n, float scale, float* __restrict__ dL, float* loss)
+__global__ void __launch_bounds__(256) k_l1_loss(const float* img, const float* target,
+                                                 int64_t n, float scale, float* dL, float* loss)
 {
     wait_for_previous_kernel();
     float acc = 0.f;
@@ -950,7 +950,7 @@ cudaError_t launch_l1_loss(const float* img, const float* target, int64_t n, flo
 }
 
 // *loss = the sum of the kLossParts partial sums
-__global__ void __launch_bounds__(256) k_loss_sum(const float* __restrict__ partial, float* loss)
+__global__ void __launch_bounds__(256) k_loss_sum(const float* partial, float* loss)
 {
     wait_for_previous_kernel();
     float acc = 0.f;

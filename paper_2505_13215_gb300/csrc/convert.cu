@@ -22,7 +22,7 @@ template <int DT>
 __device__ __forceinline__ bool is_static(const splat_g4& g4, int64_t i, float tau)
 {
     using S = Storage<DT>;
-    const float st = S::ld((const typename S::T*)g4.log_scale + i * 4 + 3);
+    const float st = S::template ld<true>((const typename S::T*)g4.log_scale + i * 4 + 3);
     return expf(st) > tau;
 }
 
@@ -160,8 +160,8 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_scatter(splat_g4 g4, spla
         if (st) {
             const int64_t d = g3.n + before;
             float ql[4], qr[4];
-            load4<DT>(g4.ql, i, ql);
-            load4<DT>(g4.qr, i, qr);
+            load4<DT, true>(g4.ql, i, ql);
+            load4<DT, true>(g4.qr, i, qr);
             const float il = inv_norm4(ql), ir = inv_norm4(qr);
 #pragma unroll
             for (int c = 0; c < 4; ++c) { ql[c] *= il; qr[c] *= ir; }

@@ -161,7 +161,7 @@ __device__ __forceinline__ void sh_rgb(const unsigned char* sh0, const void* sh_
             c0[4 * q + 0] = v.x; c0[4 * q + 1] = v.y; c0[4 * q + 2] = v.z; c0[4 * q + 3] = v.w;
         }
     } else {
-        load_sh48<DT>(p, c0);
+        load_sh48<DT, true>(p, c0);
     }
     float r = 0.5f, g = 0.5f, b = 0.5f;
 #pragma unroll
@@ -172,7 +172,7 @@ __device__ __forceinline__ void sh_rgb(const unsigned char* sh0, const void* sh_
     }
     for (int n = 1; n <= T; ++n) {
         float cn[48];
-        load_sh48<DT>(p + 48 * n, cn);
+        load_sh48<DT, true>(p + 48 * n, cn);
         sh_accumulate(cn, time_weight(n, t), Y, r, g, b);
     }
     rgb[0] = r; rgb[1] = g; rgb[2] = b;
@@ -189,14 +189,14 @@ __device__ __forceinline__ void sh_weights(const typename Storage<DT>::T* p, con
         const float4* p4 = (const float4*)p;
 #pragma unroll
         for (int qq = 0; qq < 12; ++qq) {
-            const float4 v = __ldg(p4 + qq);
+            const float4 v = p4[qq];
             add(4 * qq, v.x); add(4 * qq + 1, v.y); add(4 * qq + 2, v.z); add(4 * qq + 3, v.w);
         }
     } else {
         const uint4* p4 = (const uint4*)p;
 #pragma unroll
         for (int qq = 0; qq < 6; ++qq) {
-            const uint4 v = __ldg(p4 + qq);
+            const uint4 v = p4[qq];
             const typename Storage<DT>::T* h = (const typename Storage<DT>::T*)&v;
 #pragma unroll
             for (int e = 0; e < 8; ++e)
@@ -216,16 +216,16 @@ struct Geo {
     float b[3];    // Sigma_{1:3,4}
 };
 
-template <int DT>
+template <int DT, bool NC>
 __device__ __forceinline__ void load_geo(const splat_g3& g3, const splat_g4& g4, int64_t i, bool is4, Geo& G)
 {
     if (is4) {
         float m[4], ls[4], ql[4], qr[4];
-        load4<DT>(g4.mean, i, m);
-        load4<DT>(g4.log_scale, i, ls);
-        load4<DT>(g4.ql, i, ql);
-        load4<DT>(g4.qr, i, qr);
-        const float o = load1<DT>(g4.opacity, i);
+        load4<DT, NC>(g4.mean, i, m);
+        load4<DT, NC>(g4.log_scale, i, ls);
+        load4<DT, NC>(g4.ql, i, ql);
+        load4<DT, NC>(g4.qr, i, qr);
+        const float o = load1<DT, NC>(g4.opacity, i);
         const float il = inv_norm4(ql), ir = inv_norm4(qr);
 #pragma unroll
         for (int k = 0; k < 4; ++k) { ql[k] *= il; qr[k] *= ir; }
@@ -263,10 +263,10 @@ __device__ __forceinline__ void load_geo(const splat_g3& g3, const splat_g4& g4,
     } else {
         const int64_t j = i - g4.n;
         float q[4], ls[3];
-        load3<DT>(g3.mean, j, G.mu);
-        load3<DT>(g3.log_scale, j, ls);
-        load4<DT>(g3.quat, j, q);
-        const float o = load1<DT>(g3.opacity, j);
+        load3<DT, NC>(g3.mean, j, G.mu);
+        load3<DT, NC>(g3.log_scale, j, ls);
+        load4<DT, NC>(g3.quat, j, q);
+        const float o = load1<DT, NC>(g3.opacity, j);
         const float iq = inv_norm4(q);
         float R[9];
         quat_to_rot(q[0] * iq, q[1] * iq, q[2] * iq, q[3] * iq, R);
@@ -325,7 +325,9 @@ __global__ void __launch_bounds__(kProjectThreads, 7) k_slice_project(splat_g3 g
         const int64_t i = wb + lane;
         const bool is4 = i < n4;
         Geo G;
-        if (i < N) load_geo<DT>(g3, g4, i, is4, G);
+        // (the parameters may be read non-coherently: the call clears the status word before this kernel, so
+        // whatever wrote them is complete when it starts)
+        if (i < N) load_geo<DT, true>(g3, g4, i, is4, G);
         if (staged) {
             cp_async_wait_all();
             __syncwarp();
@@ -535,7 +537,7 @@ struct ShPart {
 // another, and the heavy view-independent chain runs on full warps.
 template <int DT, int L>
 __global__ void __launch_bounds__(kAdjThreads, adjoint_blocks(DT, L)) k_adjoint(splat_g3 g3, splat_g4 g4, ViewBatch vb, splat_proj proj,
-                                                 const float* __restrict__ dproj, splat_grads3 dg3,
+                                                 const float* dproj, splat_grads3 dg3,
                                                  splat_grads4 dg4, int32_t* status)
 {
     wait_for_previous_kernel();
@@ -568,7 +570,7 @@ __global__ void __launch_bounds__(kAdjThreads, adjoint_blocks(DT, L)) k_adjoint(
         const int64_t i = c0 + lane;
         if (i < N) {
             Geo G;
-            load_geo<DT>(g3, g4, i, i < n4, G);
+            load_geo<DT, false>(g3, g4, i, i < n4, G);
             const float g15[15] = {G.mu[0], G.mu[1], G.mu[2], G.S.xx, G.S.xy, G.S.xz, G.S.yy, G.S.yz, G.S.zz,
                                    G.op, G.mu_t, G.inv_n2, G.b[0], G.b[1], G.b[2]};
 #pragma unroll

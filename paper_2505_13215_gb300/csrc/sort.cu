@@ -1028,7 +1028,7 @@ __device__ __forceinline__ uint32_t second_level(const SortSmem<THREADS>& s, uin
 // lists of 1M Gaussians at 4 x 2704x2028.)
 template <int THREADS>
 __device__ __forceinline__ void sort_unit(SortSmem<THREADS>& s, const unsigned long long (&e)[kPer], int n,
-                                          uint32_t* __restrict__ dst)
+                                          uint32_t* dst)
 {
     const int tid = threadIdx.x;
     uint32_t dmin = 0xffffffffu, dmax = 0u, rmin = 0xffffffffu, rmax = 0u;
@@ -1148,7 +1148,7 @@ __device__ __forceinline__ void sort_unit(SortSmem<THREADS>& s, const unsigned l
 // one a long unit is bound by their latency: 545 -> 160 us for a view whose
 // 300k rows all share one depth).
 template <typename F>
-__device__ __forceinline__ void each_entry(const unsigned long long* __restrict__ src, uint32_t n, F f)
+__device__ __forceinline__ void each_entry(const unsigned long long* src, uint32_t n, F f)
 {
     for (uint32_t i0 = threadIdx.x; i0 < n; i0 += 8 * kUnitThreads) {
         unsigned long long x[8];
