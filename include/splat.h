@@ -492,7 +492,7 @@ splat_status splat_bin_sort_noalloc(const splat_proj *proj, const splat_view *vi
  * read during the call only.
  */
 typedef struct {
-    int32_t pixels_per_lane_fwd;  /* 2, 4 or 8; 0: library default (splat_set_pixels_per_lane) */
+    int32_t pixels_per_lane_fwd;  /* 2, 4 or 8; 0: the library's setting (splat_set_pixels_per_lane) */
     int32_t pixels_per_lane_bwd;  /* 2, 4 or 8; 0: library default                           */
     int32_t tile_sort;            /* 0 automatic, 1 radix, 2 binned; -1: splat_set_tile_sort */
     int32_t tile_cull;            /* 0 off, 1 on; -1: splat_set_tile_cull                    */
@@ -551,8 +551,8 @@ void splat_set_spin_limit(int64_t iterations);
 /*
  * Tuning knob of the compositing kernels: pixels each lane owns (2, 4 or 8,
  * evaluated in pairs; one warp covers 32 x that many pixels of a 16x16
- * tile).  Other values are ignored.  Until it is called each launch chooses by
- * its number of tiles.  Host-side global (the library default
+ * tile), or 0, the default: each launch chooses by its number of tiles.  Other
+ * values are ignored.  Host-side global (the library default
  * of splat_options.pixels_per_lane_*); the results do not depend
  * on it beyond floating-point summation order of the gradients.
  */

@@ -237,8 +237,8 @@ void splat_set_tile_cull(int on) { g_tile_cull.store(on ? 1 : 0); }
 
 void splat_set_pixels_per_lane(int fwd, int bwd)
 {
-    if (ppl_ok(fwd)) g_ppl_fwd.store(fwd);
-    if (ppl_ok(bwd)) g_ppl_bwd.store(bwd);
+    if (ppl_ok(fwd) || fwd == 0) g_ppl_fwd.store(fwd);
+    if (ppl_ok(bwd) || bwd == 0) g_ppl_bwd.store(bwd);
 }
 
 const char* splat_status_string(int32_t code)
