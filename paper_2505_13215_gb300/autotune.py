@@ -3,9 +3,12 @@
 Chooses the tile-instance capacity (the measured instance count K times a
 headroom) and the pixels-per-lane of the two compositing kernels (which sets
 how many warps share a 16x16 tile), by timing full training steps of the
-actual workload with CUDA events.  The choice is applied to the tuned
-rasterizer only (its splat_options), and cached in a JSON file keyed by
-(views, resolutions, Gaussian counts, storage dtype).
+actual workload with CUDA events.  The setting that the rasterizer came with
+(by default the library's own choice by the number of tiles) is timed with the
+candidates, so that tuning never ends slower than leaving it alone.  The choice
+is applied to the tuned rasterizer only (its splat_options), and cached in a
+JSON file keyed by (views, resolutions, Gaussian counts, storage dtype, device,
+build of the library): times of other kernels or another device say nothing.
 """
 from __future__ import annotations
 
@@ -15,13 +18,26 @@ from typing import Dict, Optional
 
 import torch
 
+from . import build
+
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "autotune.json")
 CANDIDATES = ((8, 8), (8, 4), (4, 8), (4, 4), (2, 4))
 
 
 def _key(R, G) -> str:
     res = ",".join("%dx%d" % (w, h) for w, h in zip(R.W, R.H))
-    return "V%d:%s:n3=%d:n4=%d:%s" % (R.V, res, G.n3, G.n4, str(G.dtype).replace("torch.", ""))
+    return "V%d:%s:n3=%d:n4=%d:%s:%s" % (R.V, res, G.n3, G.n4, str(G.dtype).replace("torch.", ""), _build_key())
+
+
+def _build_key() -> str:
+    """The device and the build of the library (the digest of its sources)."""
+    try:
+        with open(os.path.join(build.OUT_DIR, "libsplat.stamp")) as fh:
+            stamp = fh.read().strip()[:16]
+    except OSError:
+        stamp = "unknown"
+    device = torch.cuda.get_device_name() if torch.cuda.is_available() else "cpu"
+    return "%s:%s" % (device, stamp)
 
 
 def _load() -> Dict:
@@ -59,7 +75,7 @@ def _time_steps(R, G, target, reps: int) -> float:
 def tune(R, G, target: torch.Tensor, reps: int = 6, rounds: int = 2, use_cache: bool = True,
          candidates=CANDIDATES) -> Dict:
     """Pick capacity and pixels-per-lane for (R, G); applies them and returns the choice.
-    Every candidate is timed in `rounds` interleaved rounds of `reps` steps and
+    Every candidate, and the rasterizer's present setting, is timed in `rounds` interleaved rounds of `reps` steps and
     keeps its fastest round, so that a transient slowdown of one trial does not
     decide the choice."""
     key = _key(R, G)
@@ -70,6 +86,11 @@ def tune(R, G, target: torch.Tensor, reps: int = 6, rounds: int = 2, use_cache: 
         R.set_options(ppl_fwd=c["ppl_fwd"], ppl_bwd=c["ppl_bwd"])
         c = dict(c, K=K, capacity=R.capacity, cached=True)
         return c
+    own = getattr(R, "options", None)  # the rasterizer's setting so far: 0 leaves the choice to the library
+    if own is not None and candidates is CANDIDATES:
+        present = (int(own.pixels_per_lane_fwd), int(own.pixels_per_lane_bwd))
+        if present not in candidates:
+            candidates = candidates + (present,)
     ms = {c: float("inf") for c in candidates}
     for _ in range(rounds):
         for fwd, bwd in candidates:
