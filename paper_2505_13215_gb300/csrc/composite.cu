@@ -124,9 +124,11 @@ __device__ __forceinline__ bool reaches_unit(const RawRows& raw, int lane, float
 {
     const float2 xy = raw.xy[lane];
     const float4 co = raw.co[lane];
+    // the quotient stays positive where the determinant is a few rounding errors, which ellipse_consts, whose own
+    // a c - b b may be contracted differently, may find on the other side of 0
     const float ac = co.x * co.z;
     const float R2 = -2.f * __logf(__fdividef(kAlphaMin, co.w)) *
-                         (1.0001f + 2e-6f * __fdividef(ac, ac - co.y * co.y)) + 2e-3f;
+                         (1.0001f + 2e-6f * __fdividef(ac, fmaxf(ac - co.y * co.y, 1e-8f * ac))) + 2e-3f;
     // rows and columns exchanged: the extent along y inside a band of x
     float4 g0, g1;
     ellipse_consts(xy.y, xy.x, co.z, co.y, co.x, R2, g0, g1);
