@@ -572,6 +572,8 @@ __global__ void __launch_bounds__(256) k_ranges(const uint32_t* keys, const int6
 // the order does not depend on the arrival order in a cell.
 // ---------------------------------------------------------------------------
 
+// a row's super-rectangle is packed into four bytes (CellArgs::rec)
+static_assert((kMaxImage / kTile + 7) / 8 <= 255, "super-tile coordinates in a byte");
 constexpr int64_t kBinMaxTiles = 40960;  // per view: the binned path's default range
 constexpr int kSplitMaxSmem = 200 * 1024;
 constexpr int kMaxBins = 1024;           // depth bins per super-tile
@@ -2264,9 +2266,10 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 constexpr int kSuperShift = 3;  // super-tiles of 8 x 8 tiles
 
-// Bytes the workspace took when both paths sorted the rows by depth with radix
-// passes.  It stays the least that is asked for, so that the sizes callers hold
-// and the limit of splat_bin_sort_noalloc are what they were.
+// Bytes of the workspace's first layout, in which both paths sorted the rows by
+// depth with radix passes; none of its buffers is laid out so any more.  The sum
+// stays the least that is asked for, and the cells keep within it, so that the
+// sizes callers hold and the limit of splat_bin_sort_noalloc are what they were.
 static size_t legacy_bytes(const SortLayout& L, int64_t n_rows, int64_t capacity, int V, int smax)
 {
     size_t o = 0;

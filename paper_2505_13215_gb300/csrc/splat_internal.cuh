@@ -452,6 +452,8 @@ struct LaunchCtx {
 };
 LaunchCtx launch_ctx(void* stream, const splat_options* opt = nullptr);
 
+constexpr int kMaxImage = 16384;  // largest image width and height in pixels (splat_view)
+
 // Host-side argument checks shared by the entry points that take the same
 // arguments (splat_bin_sort and its allocation-free variant reject the same
 // calls).
@@ -462,7 +464,7 @@ inline bool host_valid_views(const splat_view* views, int V)
     if (!views || V < 1 || V > SPLAT_MAX_VIEWS) return false;
     for (int v = 0; v < V; ++v) {
         const splat_view& s = views[v];
-        if (s.W < 1 || s.H < 1 || s.W > 16384 || s.H > 16384) return false;
+        if (s.W < 1 || s.H < 1 || s.W > kMaxImage || s.H > kMaxImage) return false;
         if (!(s.fx > 0.f) || !(s.fy > 0.f) || !std::isfinite(s.cx) || !std::isfinite(s.cy)) return false;
         if (!(s.z_near > 0.f) || !std::isfinite(s.t)) return false;
     }
