@@ -553,7 +553,8 @@ __global__ void __launch_bounds__(256) k_ranges(const uint32_t* keys, const int6
 //                   reduction per entry, and packs the row's super-rectangle and
 //                   key into 8 bytes for the scatter.  Bins are equal steps of
 //                   the depth bits over the range of a sample of the view's rows
-//                   (depths outside fall into the first or last bin), so a bin's
+//                   (depths outside fall into the first or last bin), or runs
+//                   between samples where the rows lie on few depths; a bin's
 //                   entries are contiguous in the list's order
 //   k_cell_scan     block per super-tile: cell starts, the lists' ranges, K1, and
 //                   the sort units: runs of bins of about kUnit / 2 entries
@@ -582,7 +583,7 @@ constexpr int kUnitThreads = 256, kPer = kUnit / kUnitThreads;
 constexpr int kUnitStep = kUnit / 2;     // a unit starts at the first bin start at or after each multiple
 constexpr int kSortBuckets = 2048;
 constexpr int kSortBucketBits = 11;
-constexpr uint32_t kCrowded = 48;        // entries in one bucket above which a unit is sorted bitonically
+constexpr uint32_t kCrowded = 48;        // entries in one bucket above which a unit takes a second counting pass
 constexpr uint32_t kWholeUnit = 0xffffffffu;
 constexpr int kRowsPerThread = 2;         // of k_cell_count: 256 kRowsPerThread rows per block
 constexpr int kScatterRounds = 4;         // 32-entry rounds of a warp whose atomics are in flight together
@@ -603,7 +604,9 @@ struct CellArgs {
     int V, bin_bits, nbins;        // nbins = 2^bin_bits depth bins
     int copies;                    // of the cells (a power of two); a view's b-th run of 512 rows uses copy b % copies
     int64_t n;                     // rows per view
-    uint2* range;                  // [V] first depth bits and shift of the views' bins, from k_cell_count
+    uint2* range;                  // [V] first depth bits and shift of the views' bins (kSplitBins: by split), from
+                                   // k_cell_count
+    unsigned long long* split;     // [V][kSplits] bounds of the views' bins where kSplitBins
     int super_base[SPLAT_MAX_VIEWS + 1];
     int STX[SPLAT_MAX_VIEWS];
     uint2* rec;                    // [V * n] (super-rectangle x0 | y0 << 8 | x1 << 16 | y1 << 24, depth bits)
@@ -630,20 +633,52 @@ struct CellArgs {
     int64_t* n_needed;             // may be null
 };
 
-// range: first depth bits, shift; monotone in the key
-__device__ __forceinline__ uint32_t depth_bin(uint2 range, int nbins, uint32_t key)
+constexpr uint32_t kSplitBins = 32;  // range.y of a view whose bins are bounded by kSplits sampled entries
+constexpr int kSplits = 256;         // samples per view, one per thread of the count
+
+// An entry's place in a list's order, rows counted inside the view.
+__device__ __forceinline__ unsigned long long place_of(uint32_t key, uint32_t i)
 {
+    return (unsigned long long)key << 32 | i;
+}
+
+// Bin of row i of a view; monotone in (key, i).  range: first depth bits, shift.  split: kSplits ascending bounds
+// in shared memory, for kSplitBins.
+__device__ __forceinline__ uint32_t depth_bin(uint2 range, int nbins, uint32_t key, uint32_t i,
+                                              const unsigned long long* split)
+{
+    if (range.y == kSplitBins) {
+        const unsigned long long e = place_of(key, i);
+        uint32_t at = 0;  // bounds at or before e, 256 counting as 255
+#pragma unroll
+        for (int step = kSplits / 2; step > 0; step >>= 1)
+            if (split[at + step - 1] <= e) at += step;
+        if (nbins < 4 * kSplits) return nbins >= kSplits ? at : at * (uint32_t)nbins / kSplits;
+        // four equal steps between two bounds
+        const unsigned long long lo = at > 0 ? split[at - 1] : 0ull, w = (split[at] - lo) >> 2;
+        return 4u * at + (e >= lo + w) + (e >= lo + 2 * w) + (e >= lo + 3 * w);
+    }
     return key > range.x ? min((key - range.x) >> range.y, (uint32_t)nbins - 1u) : 0u;
 }
 
-// Depth bins of view v: the range of the depth bits of 256 of its rows, one per
-// thread, evenly spaced.  About one row in 128 lies outside; a camera far from a
-// small scene, whose depths share their leading bits, gets as fine a division as
-// any other (bins of a fixed part of an octave held a list's whole depth range:
-// 1060 against 340 us for 1M Gaussians seen from 40 times their extent).
-__device__ __forceinline__ uint2 sample_range(const CellArgs& a, int v, uint32_t (*s_mm)[8])
+// Depth bins of view v: equal steps of the depth bits over their range among 256
+// of its rows, one per thread, one from each of 256 runs of rows (at a scattered
+// place in the run: rows may come in a regular order).  About one row in 128 lies
+// outside; a camera far from a small scene, whose depths share their leading bits,
+// gets as fine a division as any other (bins of a fixed part of an octave held a
+// list's whole depth range: 1060 against 340 us for 1M Gaussians seen from 40 times
+// their extent).  Where many pairs of samples share a bin, the rows lie on few
+// depths: a plane that faces the camera, a flat scene.  The samples themselves,
+// ordered by depth and row, bound the bins then, so that no bin of a list gets
+// long, whatever the depths: a long bin is sorted by blocks that each read all of
+// it.  1M rows in 128x128, all at one depth 1332 -> 240 us, at two 815 -> 282; 300k
+// 276 -> 106 and 257 -> 104 (the radix sort of all rows took 283 and 200).  The test of
+// the samples costs nothing that shows.
+__device__ __forceinline__ uint2 sample_range(const CellArgs& a, int v, uint32_t (*s_mm)[8], unsigned long long* s_split)
 {
-    const int64_t step = a.n >= 256 ? a.n / 256 : 1, i = threadIdx.x * step;
+    const uint32_t tid = threadIdx.x;
+    const uint32_t step = a.n >= kSplits ? (uint32_t)(a.n / kSplits) : 1u;
+    const uint32_t i = tid * step + (tid * 0x9e3779b9u >> 8) % step;
     uint32_t lo = 0xffffffffu, hi = 0u;
     if (i < a.n) {
         const int64_t r = (int64_t)v * a.n + i;
@@ -651,11 +686,15 @@ __device__ __forceinline__ uint2 sample_range(const CellArgs& a, int v, uint32_t
         const uint32_t key = __float_as_uint(((const float4*)a.proj.rgb_depth)[r].w);
         if (nt > 0) lo = hi = key;
     }
+    const bool seen = lo <= hi;
+    const uint32_t key = lo;
+    uint32_t* s_key = (uint32_t*)s_split;
+    s_key[tid] = key;
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
-    if ((threadIdx.x & 31) == 0) {
-        s_mm[0][threadIdx.x >> 5] = lo;
-        s_mm[1][threadIdx.x >> 5] = hi;
+    if ((tid & 31) == 0) {
+        s_mm[0][tid >> 5] = lo;
+        s_mm[1][tid >> 5] = hi;
     }
     __syncthreads();
 #pragma unroll
@@ -664,7 +703,23 @@ __device__ __forceinline__ uint2 sample_range(const CellArgs& a, int v, uint32_t
         hi = max(hi, s_mm[1][w]);
     }
     if (lo > hi) return make_uint2(0u, 31u);  // none visible in the sample
-    return make_uint2(lo, (uint32_t)min(31, max(0, 32 - __clz(hi - lo) - a.bin_bits)));
+    const uint2 range = make_uint2(lo, (uint32_t)min(31, max(0, 32 - __clz(hi - lo) - a.bin_bits)));
+    // pairs of a scattered pairing (neighbours may be alike): a share p of the samples in one bin makes 256 p^2 of
+    // them, a sixth 7; rows spread evenly over the bins make one in four batches of 1024 bins, and 4 of 64
+    const uint32_t other = s_key[(77u * tid + 31u) & 255u];
+    const int pairs = __syncthreads_count(seen && other != 0xffffffffu &&
+                                          depth_bin(range, a.nbins, key, 0u, nullptr) ==
+                                              depth_bin(range, a.nbins, other, 0u, nullptr));
+    if (pairs < (a.nbins >= kSplits ? 8 : 32)) return range;
+    // order the samples by counting the smaller ones; those not seen come last
+    const unsigned long long e = seen ? place_of(key, i) : place_of(0xffffffffu, 0xffffff00u + tid);
+    s_split[kSplits + tid] = e;
+    __syncthreads();
+    int at = 0;
+    for (int q = 0; q < kSplits; ++q) at += s_split[kSplits + q] < e;
+    s_split[at] = e;
+    __syncthreads();
+    return make_uint2(0u, kSplitBins);
 }
 
 // The cells of the rows of count block `block` (the same in k_cell_count and k_cell_scatter).
@@ -684,6 +739,7 @@ __global__ void __launch_bounds__(256) k_cell_count(CellArgs a)
 {
     wait_for_previous_kernel();
     __shared__ uint32_t s_mm[2][8];
+    __shared__ unsigned long long s_split[2 * kSplits];
     const int v = blockIdx.y;
     const int64_t gt = ((int64_t)v * gridDim.x + blockIdx.x) * 256 + threadIdx.x;
     for (int64_t t = gt; t < a.total_tiles; t += (int64_t)gridDim.x * gridDim.y * 256) a.ranges[t] = make_uint2(0u, 0u);
@@ -706,9 +762,12 @@ __global__ void __launch_bounds__(256) k_cell_count(CellArgs a)
             depth[q] = ((const float4*)a.proj.rgb_depth)[r].w;
         }
     }
-    const uint2 range = sample_range(a, v, s_mm);
+    const uint2 range = sample_range(a, v, s_mm, s_split);
     uint32_t* cells = cell_copy(a, blockIdx.x);
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.range[v] = range;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) a.range[v] = range;
+        if (range.y == kSplitBins) a.split[v * kSplits + threadIdx.x] = s_split[threadIdx.x];
+    }
 #pragma unroll
     for (int q = 0; q < kRowsPerThread; ++q) {
         const int64_t i = (blockIdx.x * kRowsPerThread + q) * 256ll + threadIdx.x;
@@ -719,7 +778,7 @@ __global__ void __launch_bounds__(256) k_cell_count(CellArgs a)
             const int x0 = rc[q].x >> 3, y0 = rc[q].y >> 3, x1 = (rc[q].z + 7) >> 3, y1 = (rc[q].w + 7) >> 3;
             if (x1 > x0 && y1 > y0) {
                 pack = (uint32_t)x0 | (uint32_t)y0 << 8 | (uint32_t)x1 << 16 | (uint32_t)y1 << 24;
-                const uint32_t bin = depth_bin(range, a.nbins, key);
+                const uint32_t bin = depth_bin(range, a.nbins, key, (uint32_t)i, s_split);
                 for (int y = y0; y < y1; ++y) {
                     uint32_t* c = cells + (size_t)(a.super_base[v] + y * a.STX[v]) * a.nbins + bin;
                     for (int x = x0; x < x1; ++x) atomicAdd(c + (size_t)x * a.nbins, 1u);
@@ -873,7 +932,13 @@ __global__ void __launch_bounds__(256) k_cell_scatter(CellArgs a)
     const uint32_t c = w * ((rec.x >> 24) - y0);
     // first cell of the row, and of its entries' order in the warp: lane l owns [e, e + c)
     const uint32_t cell0 = (uint32_t)(a.super_base[v] + (int)y0 * a.STX[v] + (int)x0);
-    const uint32_t bin = depth_bin(a.range[v], a.nbins, rec.y);
+    const uint2 range = a.range[v];
+    __shared__ unsigned long long s_split[kSplits];
+    if (range.y == kSplitBins) {  // (block-uniform)
+        s_split[threadIdx.x] = a.split[v * kSplits + threadIdx.x];
+        __syncthreads();
+    }
+    const uint32_t bin = depth_bin(range, a.nbins, rec.y, (uint32_t)i, s_split);
     uint32_t* cells = cell_copy(a, blockIdx.x / kRowsPerThread);
     uint32_t e = c;
 #pragma unroll
@@ -942,6 +1007,7 @@ struct SortSmem {
     uint16_t at[kEntries];      // arrival in a second-level bucket
     uint32_t red[4][THREADS / 32], tmp[THREADS / 32];
     uint32_t n;
+    bool taken;                 // a part's entries are all in e
 };
 using UnitSmem = SortSmem<kUnitThreads>;
 
@@ -1016,6 +1082,25 @@ __device__ __forceinline__ uint32_t second_level(const SortSmem<THREADS>& s, uin
 {
     const uint32_t p = s.h[b], c = s.h[b + 1] - p;
     return c > kCrowded ? p + __umulhi((row - rmin) << up, c) : p;
+}
+
+// Sorts the P (a power of two) values of e in shared memory.
+template <int THREADS>
+__device__ __forceinline__ void sort_bitonic(unsigned long long* e, int P)
+{
+    for (int size = 2; size <= P; size <<= 1) {
+        for (int step = size >> 1; step > 0; step >>= 1) {
+            for (int t = threadIdx.x; t < P / 2; t += THREADS) {
+                const int i = 2 * t - (t & (step - 1)), j = i + step;
+                const unsigned long long x = e[i], y = e[j];
+                if ((x > y) == ((i & size) == 0)) {
+                    e[i] = y;
+                    e[j] = x;
+                }
+            }
+            __syncthreads();
+        }
+    }
 }
 
 // Sorts a unit of n <= kPer THREADS entries, entry t + THREADS k in e[k] of thread
@@ -1127,19 +1212,7 @@ __device__ __forceinline__ void sort_unit(SortSmem<THREADS>& s, const unsigned l
             while (P < n) P <<= 1;
             for (int i = n + tid; i < P; i += THREADS) s.e[i] = ~0ull;
             __syncthreads();
-            for (int size = 2; size <= P; size <<= 1) {
-                for (int step = size >> 1; step > 0; step >>= 1) {
-                    for (int t = tid; t < P / 2; t += THREADS) {
-                        const int i = 2 * t - (t & (step - 1)), j = i + step;
-                        const unsigned long long x = s.e[i], y = s.e[j];
-                        if ((x > y) == ((i & size) == 0)) {
-                            s.e[i] = y;
-                            s.e[j] = x;
-                        }
-                    }
-                    __syncthreads();
-                }
-            }
+            sort_bitonic<THREADS>(s.e, P);
             for (int i = tid; i < n; i += THREADS) dst[i] = (uint32_t)s.e[i];
         }
     }
@@ -1162,17 +1235,15 @@ __device__ __forceinline__ void each_entry(const unsigned long long* src, uint32
     }
 }
 
-// Bucket counts (scanned, in s.h) of those of src[0 .. n) within [lo, hi]; with
-// `all` of every entry, the first and the last bucket open-ended.
+// Bucket counts (scanned, in s.h) of those of src[0 .. n) within [lo, hi].
 __device__ __forceinline__ KeyRange count_range(UnitSmem& s, const unsigned long long* src, uint32_t n,
-                                                unsigned long long lo, unsigned long long hi, bool all = false)
+                                                unsigned long long lo, unsigned long long hi)
 {
     const KeyRange kr = key_range(lo, hi, kSortBucketBits);
     for (int k = threadIdx.x; k < kSortBuckets; k += kUnitThreads) s.h[k] = 0u;
     __syncthreads();
     each_entry(src, n, [&](unsigned long long e) {
-        if (all || (e >= lo && e <= hi))
-            atomicAdd(&s.h[e > lo ? min((e - lo) >> kr.shift, (unsigned long long)kSortBuckets - 1) : 0ull], 1u);
+        if (e >= lo && e <= hi) atomicAdd(&s.h[(e - lo) >> kr.shift], 1u);
     });
     __syncthreads();
     scan_buckets(s, s.h);
@@ -1180,38 +1251,48 @@ __device__ __forceinline__ KeyRange count_range(UnitSmem& s, const unsigned long
 }
 
 // Part g of a unit of more than kUnit entries (one depth bin of a crowded
-// list): the parts' blocks each count the whole unit by value and take the
-// entries of the g-th run of buckets, about kUnitStep of them, so that any
-// number of blocks share a long unit without waiting for one another.
+// list): the parts' blocks each read the whole unit and take the entries between
+// two of its sorted samples, about kUnitStep of them, so that any number of
+// blocks share a long unit without waiting for one another.  (Samples, not equal
+// steps of the key: where many entries share one depth next to others, the steps
+// would hold them all in one part: 84 ms for 500k of them.)
 // Sets the value range [lo, hi] of the part, the number of its entries and their
-// first position in the unit.
+// first position in the unit, and leaves the entries in s.e if they are no more
+// than kUnit.
 __device__ __noinline__ void part_range(UnitSmem& s, const unsigned long long* src, uint32_t n, uint32_t g,
                                         unsigned long long& lo, unsigned long long& hi, uint32_t& left, uint32_t& out)
 {
-    const int tid = threadIdx.x;
-    // buckets over the range of a sample of kUnit entries, the first and the last open-ended
-    uint32_t dmin = 0xffffffffu, dmax = 0u, rmin = 0xffffffffu, rmax = 0u;
+    const uint32_t tid = threadIdx.x, parts = (n + kUnitStep - 1) / kUnitStep;
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-        const unsigned long long x = src[(unsigned long long)(tid + kUnitThreads * k) * n / kUnit];
-        dmin = min(dmin, (uint32_t)(x >> 32));
-        dmax = max(dmax, (uint32_t)(x >> 32));
-        rmin = min(rmin, (uint32_t)x);
-        rmax = max(rmax, (uint32_t)x);
+        const unsigned long long i = tid + kUnitThreads * k;
+        s.e[i] = src[i * n / kUnit];
     }
-    block_bounds(s, dmin, dmax, rmin, rmax, lo, hi);
     __syncthreads();
-    const KeyRange kr = count_range(s, src, n, lo, hi, true);
-    const int b0 = lower_bound(s.h, kSortBuckets, g * kUnitStep), b1 = lower_bound(s.h, kSortBuckets, (g + 1) * kUnitStep);
-    out = s.h[b0];
-    left = s.h[b1] - out;
-    hi = b1 < kSortBuckets ? lo + ((unsigned long long)b1 << kr.shift) - 1 : ~0ull;
-    lo = b0 > 0 ? lo + ((unsigned long long)b0 << kr.shift) : 0ull;
+    sort_bitonic<kUnitThreads>(s.e, kUnit);
+    lo = g > 0 ? s.e[(unsigned long long)g * kUnit / parts] : 0ull;
+    hi = g + 1 < parts ? s.e[(unsigned long long)(g + 1) * kUnit / parts] - 1 : ~0ull;
+    if (tid == 0) s.n = s.red[0][0] = 0u;
+    __syncthreads();
+    uint32_t below = 0u;
+    each_entry(src, n, [&](unsigned long long e) {
+        below += e < lo;
+        if (e >= lo && e <= hi) {
+            const uint32_t at = atomicAdd(&s.n, 1u);
+            if (at < (uint32_t)kUnit) s.e[at] = e;
+        }
+    });
+    below = __reduce_add_sync(0xffffffffu, below);
+    if ((tid & 31) == 0) atomicAdd(&s.red[0][0], below);
+    __syncthreads();
+    left = s.n;
+    out = s.red[0][0];
+    if (tid == 0) s.taken = left <= (uint32_t)kUnit;
     __syncthreads();
 }
 
 // The first up to kUnit entries by value of a part's `left` ones in [lo, hi] into
-// s.e: returns their number and the value top up to which they go (0: none).  A
+// s.e, unless part_range left them there: returns their number and the value top up to which they go (0: none).  A
 // part that holds more than kUnit (one crowded bucket) goes through several of
 // these, each found by counting again over ever finer buckets (entries are unique,
 // so this ends).
@@ -1220,6 +1301,7 @@ __device__ __noinline__ uint32_t take_range(UnitSmem& s, const unsigned long lon
 {
     const int tid = threadIdx.x;
     top = hi;
+    if (s.taken) return left;
     uint32_t m = left;
     while (m > (uint32_t)kUnit && lo < top) {
         const KeyRange kr = count_range(s, src, n, lo, top);
@@ -2255,7 +2337,7 @@ struct SortLayout {
     // binned path
     int bin_bits, copies;
     int64_t queue_cap;
-    size_t off_rec, off_range, off_cell, off_cell_lb, off_queue, off_nqueue, off_rlb, off_total, off_vals1, off_sranges,
+    size_t off_rec, off_range, off_split, off_cell, off_cell_lb, off_queue, off_nqueue, off_rlb, off_total, off_vals1, off_sranges,
         off_ninst1, off_segbase, off_segcnt, off_segsuper, off_sathead, off_nhead, off_mask;
     // both
     size_t off_tord, off_tickets, zero_begin, zero_end;
@@ -2361,6 +2443,7 @@ SortLayout sort_layout(int64_t n_rows, int64_t capacity, int V, const int* TX, c
         L.off_mask = take(8 * (size_t)capacity);  // the unsorted entries, then the coverage words
         L.off_rec = take(8 * (size_t)n_rows);
         L.off_range = take(8 * (size_t)std::max(V, 1));
+        L.off_split = take(8 * (size_t)kSplits * std::max(V, 1));
         // units of lists of more than kUnit entries: at most 2 n / kUnitStep + 1 of a list of n
         const int64_t per_view = V > 0 ? n_rows / V : 0;
         const int64_t most = std::min<int64_t>(capacity, per_view * L.total_super);
@@ -2504,6 +2587,7 @@ cudaError_t launch_bin_sort(const splat_proj& proj, const ViewBatch& vb, const s
         c.nbins = 1 << L.bin_bits;
         c.n = proj.n;
         c.range = (uint2*)(w + L.off_range);
+        c.split = (unsigned long long*)(w + L.off_split);
         for (int v = 0; v < vb.V; ++v) c.STX[v] = STX[v];
         for (int v = 0; v <= vb.V; ++v) c.super_base[v] = super_base[v];
         c.rec = (uint2*)(w + L.off_rec);
