@@ -35,6 +35,7 @@ def test_the_setting_returns_to_automatic():
     G, views = _scene(20, 10)  # 200 tiles: 800 units at 2 pixels per lane, 400 at 4, 200 at 8
     R = raster.Rasterizer(G.n3, G.n4, views)
     R.autotune_capacity(G)
+    R.forward(G)  # lists in the buffers of the new capacity
     target = torch.zeros_like(R.rgb)
     assert _launches(R, target) == 2
     abi.splat_set_pixels_per_lane(8, 8)
@@ -47,6 +48,8 @@ def test_the_setting_returns_to_automatic():
     assert _launches(R, target) == 1
     R.set_options(ppl_fwd=0)
     assert _launches(R, target) == 2
+    torch.cuda.synchronize()
+    R.check()
 
 
 @pytest.mark.parametrize("tiles_per_sm", [2, 4, 10, 40])
