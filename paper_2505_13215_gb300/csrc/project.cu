@@ -118,7 +118,13 @@ __device__ __forceinline__ void sh_accumulate(const float c[48], float w, const 
 // (V = 8, 500k Gaussians: 108 us).  The warp copies its 32 rows together instead: 82
 // us; V = 2, 1M: 80 -> 67.  V = 1 reads a row once and wants L1 for it (300k: 16.5 us
 // direct, 18 staged) and 16-bit rows are half as long (staged: V = 1 33 -> 42 us, V = 4
-// 81 -> 89 at 1M): these stay with direct loads.
+// 81 -> 89 at 1M): these stay with direct loads.  The copy starts with the geometry's
+// loads, before it is known whether a view sees the Gaussian, and pays where about a
+// quarter (V = 8) or half (V = 2) of a view's Gaussians are seen: 1M of which no view
+// sees one take 118 us instead of 94 at V = 8 and 59 instead of 34 at V = 2, of which
+// views see 0.7 154 instead of 219 and 66 instead of 73.  Copying only rows that a
+// view has seen adds the copy's latency: 82 -> 100 us for the 500k at V = 8, 66 -> 75
+// for the 1M at V = 2.
 constexpr int kShStride = 208;
 constexpr int kProjectThreads = 128;
 
