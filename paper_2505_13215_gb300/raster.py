@@ -207,6 +207,7 @@ class Rasterizer:
         self.capacity = capacity
         self.keys = torch.empty((capacity if self.keep_keys else 0,), dtype=torch.int32, device=self.device)
         self.vals = torch.empty((capacity,), dtype=torch.int32, device=self.device)
+        self.ranges.zero_()  # the lists are gone: until the next sort every tile is empty
         self.cbins = abi.splat_bins(capacity, self.keys.data_ptr() if self.keep_keys else None, self.vals.data_ptr(),
                                     self.ranges.data_ptr(), self.n_instances.data_ptr(), self.tile_order.data_ptr(),
                                     self.n_needed.data_ptr())
