@@ -1961,9 +1961,12 @@ __device__ __forceinline__ uint32_t inner_columns(const float4& g0, const float4
 // it is on its way to close within the reach (one that stays open keeps the tail
 // alive, and a window costs about what three windows of the tail cost); its tail
 // starts where it stopped.  On 1M Gaussians at 4 x 2704x2028 the lists shrink
-// from 87M to 26M instances: head 139 -> 305 us, but the rest of the lists' sort
-// 78 -> 33, tail 259 -> 54, writes 237 -> 85.  Batches of fewer super-tiles than
-// two per SM keep short heads: there the tail's parallel segments are faster.
+// from 87M to 23M instances: head 139 -> 305 us, but the rest of the lists' sort
+// 78 -> 33, tail 259 -> 54, writes 237 -> 85.  The rule does not weigh the saving
+// against the windows: on 300k at 4 x 1352x1014 the head takes 75 us instead of 42
+// and the passes behind it save about 18 (the sort 8 us slower in the step).
+// Batches of fewer super-tiles than two per SM keep short heads: there the tail's
+// parallel segments are faster.
 // Bound by the entries' gathers (three sectors each) and by issue.  One CTA per
 // tile row with its entries queued per row and a warp per tile column re-read
 // every entry eight times and evaluated the weights on the few lanes listed in
