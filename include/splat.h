@@ -568,8 +568,9 @@ int64_t splat_launch_count(void);
  * instance list, 2 = binned partition: the rows listed by 8x8-tile super-tile,
  * each super-tile's list sorted by depth and filtered into its tiles' lists (used
  * automatically when every view has at most 40960 tiles; never for a view of
- * more than about 2900 super-tiles, which takes the radix passes).  Host-side global (the library default of
- * splat_options.tile_sort); splat_workspace_size depends on it.
+ * more than about 2900 super-tiles, which takes the radix passes).  Host-side
+ * global (the library default of splat_options.tile_sort);
+ * splat_workspace_size depends on it.
  */
 void splat_set_tile_sort(int mode);
 
